@@ -33,7 +33,7 @@ def _nvcc() -> str:
 def _sources():
     cu = sorted(glob.glob(os.path.join(CSRC, "*.cu")))
     cpp = sorted(glob.glob(os.path.join(CSRC, "*.cpp")))
-    hdr = sorted(glob.glob(os.path.join(CSRC, "*.h"))) + [os.path.join(INCLUDE, "gblu.h")]
+    hdr = sorted(glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.cuh"))) + [os.path.join(INCLUDE, "gblu.h")]
     return cu, cpp, hdr
 
 

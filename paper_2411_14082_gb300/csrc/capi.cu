@@ -11,6 +11,7 @@
 
 #include <algorithm>
 #include <climits>
+#include <cmath>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
@@ -81,9 +82,9 @@ struct gblu_ctx {
     gblu_opts opts{};
     int sm_count = 0;
     int l2_bytes = 0;
-    int ref_blocks_per_sm = 0, ref_grid = 0, solve_grid = 0, res_blocks = 0, trail_per_sm = 0;
-    int batch_blocks_per_sm = 0;   // refactor_batch_kernel CTAs that fit on an SM
-    int ref32_blocks_per_sm = 0, ref32_grid = 0;
+    // re-factorization CTAs that fit on an SM, with kRefSmemTwo and kRefSmemThree
+    int ref_blocks_per_sm[2] = {0, 0}, batch_blocks_per_sm[3] = {0, 0, 0}, ref32_blocks_per_sm[2] = {0, 0};
+    int solve_grid = 0, res_blocks = 0, trail_per_sm = 0;
     bool f32_valid = false, f32_widened = false;   // single-precision factors of the last call
     int32_t force_col = -1;                        // forced check failure of the next refactorization
     double t_tail[4] = {0, 0, 0, 0};               // last tail run: kernel, repack, schedule, upload (ms)
@@ -116,6 +117,19 @@ struct gblu_ctx {
     DBuf<int64_t> LUp;
     DBuf<int32_t> LUi, nU, rows, finish, task_ptr, task_cols, amap, piv, pinv;
     DBuf<uint8_t> chain;
+    // panels of the re-factorization and the scratch of those beyond shared memory
+    DBuf<PanelDesc> pan;
+    DBuf<int32_t> pan_id, prow, ppref;
+    DBuf<int32_t> ctask_ptr, ctask_cols, camap;   // tasks without panels (Schedule::ctask_ptr)
+    DBuf<uint8_t> pmask;
+    DBuf<PanelRun> prun;
+    DBuf<unsigned char> pscratch;
+    // trailing block: its matrix, per-column counts before it, and the
+    // words of its launches (tickets, flags, column maxima, reciprocals)
+    DBuf<double> tb_S;
+    DBuf<int32_t> tb_nux;
+    DBuf<unsigned long long> tb_words;
+    int32_t pscratch_ctas = 0;
     // re-prediction: steps whose predicted row is not the preferred one, and
     // the pivot choice read back (step, non-finite flag)
     DBuf<uint8_t> strict;
@@ -246,6 +260,8 @@ int sms_used(const gblu_ctx *h)
     return (h->opts.max_sms > 0 && h->opts.max_sms < h->sm_count) ? h->opts.max_sms : h->sm_count;
 }
 int pgrid(const gblu_ctx *h, int per_sm) { return std::max(1, per_sm) * sms_used(h); }
+// the handle's shared-memory configuration (index of the blocks_per_sm arrays)
+int cfg(const gblu_ctx *h) { return h->W.smem == kRefSmemTwo ? 0 : 1; }
 
 template <class T>
 int ensure(gblu_ctx *h, DBuf<T> &b, size_t count)
@@ -357,6 +373,9 @@ static int upload_solve(gblu_ctx *h, cudaStream_t st, bool l_rows_done)
     return GBLU_OK;
 }
 
+// row pitch of the trailing block's matrix (values)
+static size_t block_pitch(int32_t m) { return ((size_t)m + 31) & ~(size_t)31; }
+
 // Install a factor structure: schedule on the host, arrays on the device.
 // values (optional) are the factor values in canonical order.  With
 // defer_solve only what the re-factorization reads is built and uploaded
@@ -368,10 +387,12 @@ int install_structure(gblu_ctx *h, Structure &&S, const std::vector<double> *val
     h->S = std::move(S);
     h->struct_version++;
     h->f32_valid = false;
-    const int resident_warps = h->ref_blocks_per_sm * h->sm_count * (kRefThreads / 32);
+    const int resident_warps = h->ref_blocks_per_sm[1] * h->sm_count * (kRefThreads / 32);
     const SolveSplit sp = solve_split(h->opts);
     const auto t_s = std::chrono::steady_clock::now();
-    build_schedule(h->P, h->S, h->opts.alpha, resident_warps, h->opts.sched_mode, h->opts.warp_column_max, sp,
+    const int panel_ctas =   // scratch panels only run with kRefSmemTwo
+        std::max(h->ref_blocks_per_sm[0], std::max(h->batch_blocks_per_sm[0], h->ref32_blocks_per_sm[0])) * h->sm_count;
+    build_schedule(h->P, h->S, h->opts.alpha, resident_warps, panel_ctas, h->opts.sched_mode, h->opts.warp_column_max, sp,
                    h->opts.dense_min_rows, h->W, defer_solve);
     h->solve_pending = defer_solve;
     const auto t_u = std::chrono::steady_clock::now();
@@ -388,7 +409,7 @@ int install_structure(gblu_ctx *h, Structure &&S, const std::vector<double> *val
     if (h->W.pull_cols > 0) {
         // one scratch per CTA that a persistent launch can hold; only while it
         // stays within kPullScratchBytes (the columns are pushed otherwise)
-        const int slots = std::max(h->ref_blocks_per_sm, h->batch_blocks_per_sm) * h->sm_count;
+        const int slots = std::max(h->ref_blocks_per_sm[1], h->batch_blocks_per_sm[1]) * h->sm_count;
         const size_t bytes = (size_t)slots * (size_t)n * (sizeof(double) + sizeof(unsigned long long));
         if (bytes <= kPullScratchBytes) {
             CK(upload(h, h->pull_start, h->W.pull_start, st));
@@ -402,6 +423,28 @@ int install_structure(gblu_ctx *h, Structure &&S, const std::vector<double> *val
             CU(cudaMemsetAsync(h->pull_lock.p, 0, sizeof(int32_t) * (size_t)slots, st));
             h->pull_slots = slots;
         }
+    }
+    if (!h->W.ctask_ptr.empty()) {
+        CK(upload(h, h->ctask_ptr, h->W.ctask_ptr, st));
+        CK(upload(h, h->ctask_cols, h->W.ctask_cols, st));
+        CK(upload(h, h->camap, h->W.camap, st));
+    }
+    CK(upload(h, h->pan, h->W.pan, st));
+    CK(upload(h, h->pan_id, h->W.pan_id, st));
+    CK(upload(h, h->prow, h->W.prow, st));
+    CK(upload(h, h->pmask, h->W.pmask, st));
+    CK(upload(h, h->ppref, h->W.ppref, st));
+    CK(upload(h, h->prun, h->W.prun, st));
+    if (h->W.tb_m > 0) {
+        const size_t m = (size_t)h->W.tb_m;
+        CK(upload(h, h->tb_nux, h->W.tb_nux, st));
+        CK(ensure(h, h->tb_S, m * block_pitch(h->W.tb_m)));
+        CK(ensure(h, h->tb_words, 2 * m + block_steps(h->W.tb_m)));
+    }
+    h->pscratch_ctas = 0;
+    if (h->W.pscratch > 0) {
+        CK(ensure(h, h->pscratch, (size_t)panel_ctas * (size_t)h->W.pscratch));
+        h->pscratch_ctas = panel_ctas;
     }
     CK(upload(h, h->dense_s0, h->W.dense_s0, st));
     if (h->W.dense_m > 0) CK(ensure(h, h->dense, (size_t)h->W.dense_m * h->W.dense_m));
@@ -500,16 +543,39 @@ RefactorArgs refactor_args(gblu_ctx *h, const double *Ax)
         a.pull_slots = h->pull_slots;
     }
     a.n = h->S.n;
+    a.pan_id = h->pan_id.p;
+    a.pan = h->pan.p;
+    a.prow = h->prow.p;
+    a.ppref = h->ppref.p;
+    a.pmask = h->pmask.p;
+    a.prun = h->prun.p;
+    a.smem_bytes = h->W.smem;
+    a.pscratch = h->pscratch.p;
+    a.pscratch_bytes = h->W.pscratch;
+    a.pscratch_ctas = h->pscratch_ctas;
     return a;
 }
 
 // the launches of one checked re-factorization; ep = the epoch the kernels
 // store in the ready flags, or -1: read it from the control block (graph
 // replay, where the epoch changes between launches of the same graph)
-int issue_refactor(gblu_ctx *h, const double *Ax, cudaStream_t st, int ep)
+// block: the trailing block densely (block.cu).  A check that fails then
+// only says that some check fails.
+int issue_refactor(gblu_ctx *h, const double *Ax, cudaStream_t st, int ep, bool block = false)
 {
     KL(launch_begin_refactor(h->ctl, st));
     RefactorArgs a = refactor_args(h, Ax);
+    const size_t m = (size_t)h->W.tb_m, pitch = block_pitch(h->W.tb_m);
+    if (block) {
+        a.no_stop = 0;
+        a.tb_p = h->W.tb_p;
+        a.tb_S = h->tb_S.p;
+        a.tb_ld = (int64_t)pitch;
+        a.dense_p = h->W.tb_p;   // its columns outside panels
+        a.dense_s0 = h->tb_nux.p;
+        CU(cudaMemsetAsync(h->tb_S.p, 0, m * pitch * sizeof(double), st));
+        CU(cudaMemsetAsync(h->tb_words.p, 0, (m + block_steps((int)m)) * sizeof(unsigned long long), st));
+    }
     const std::vector<int32_t> &ltp = h->W.level_task_ptr;
     const int32_t div = h->W.div_level;   // the schedule already follows sched_mode
     for (int32_t l = 0; l < div; l++) {   // cluster mode: one launch per level
@@ -521,7 +587,31 @@ int issue_refactor(gblu_ctx *h, const double *Ax, cudaStream_t st, int ep)
     if (ltp[div] < ntask) {               // pipeline mode: one persistent launch
         a.task_begin = ltp[div];
         a.ntasks = ntask - ltp[div];
-        KL(launch_refactor_tasks(a, true, pgrid(h, h->ref_blocks_per_sm), ep, st));
+        KL(launch_refactor_tasks(a, true, pgrid(h, h->ref_blocks_per_sm[cfg(h)]), ep, st));
+    }
+    if (block) {
+        BlockArgs b{};
+        b.S = h->tb_S.p;
+        b.ld = (int64_t)pitch;
+        b.m = h->W.tb_m;
+        b.p = h->W.tb_p;
+        b.eps = h->opts.pivot_tol;
+        b.ctl = h->ctl;
+        b.LUp = h->LUp.p;
+        b.LUi = h->LUi.p;
+        b.nux = h->tb_nux.p;
+        b.LUx = h->vals.p;
+        b.finish = h->finish.p;
+        b.epoch = ep;
+        b.spin_limit = h->opts.spin_limit;
+        b.colmax = h->tb_words.p;                       // m, zeroed above
+        b.ticket = (int32_t *)(h->tb_words.p + m);      // one word per step: ticket, flag
+        b.flag = b.ticket + block_steps((int)m);
+        b.inv = (double *)(h->tb_words.p + m + block_steps((int)m));
+        long long nl = 0;
+        const int e = launch_block_lu(b, st, &nl);
+        h->launches += nl;
+        if (e != 0) return fail(GBLU_ERR_CUDA, "trailing block launch failed: %s", cudaGetErrorString((cudaError_t)e));
     }
     if (h->W.dense_m > 0) {   // the dense tail: blocked LU of the block, then scatter
         DenseArgs2 d{};
@@ -544,10 +634,27 @@ int issue_refactor(gblu_ctx *h, const double *Ax, cudaStream_t st, int ep)
     return GBLU_OK;
 }
 
+// the trailing block is factored densely unless the checks have to be made
+// column by column (a forced failure, a re-prediction's strict columns)
+static bool block_applies(const gblu_ctx *h) { return h->W.tb_m > 0 && h->force_col < 0 && !h->strict_on; }
+
 // A deferred install's solve part is finished on the host while the
 // re-factorization runs.
 int run_refactor(gblu_ctx *h, const double *Ax, cudaStream_t st, int *interrupted)
 {
+    if (block_applies(h)) {
+        h->epoch++;
+        CK(issue_refactor(h, Ax, st, h->epoch, true));
+        CK(finish_install(h, st));
+        CK(read_ctl(h, st));
+        CK(status_code(h));
+        if (!h->hctl->interrupted) {
+            *interrupted = 0;
+            h->last_first_bad = -1;
+            return GBLU_OK;
+        }
+        // a check failed: column by column, in the caller's mode
+    }
     h->epoch++;
     CK(issue_refactor(h, Ax, st, h->epoch));
     CK(finish_install(h, st));
@@ -876,7 +983,7 @@ int restart_on_structure(gblu_ctx *h, const double *Ax, cudaStream_t st, bool no
     a.no_stop = no_stop ? 1 : 0;
     a.task_begin = 0;
     a.ntasks = (int32_t)h->W.task_ptr.size() - 1;
-    KL(launch_refactor_tasks(a, true, pgrid(h, h->ref_blocks_per_sm), h->epoch, st));
+    KL(launch_refactor_tasks(a, true, pgrid(h, h->ref_blocks_per_sm[cfg(h)]), h->epoch, st));
     CK(read_ctl(h, st));
     CK(status_code(h));
     *interrupted = h->hctl->interrupted || h->hctl->first_bad != INT_MAX;
@@ -1101,14 +1208,14 @@ int gblu_create(gblu_handle *out, int device, const gblu_opts *o)
     if (e == cudaSuccess) e = cudaMalloc((void **)&h->ctl, sizeof(DevCtl));
     if (e == cudaSuccess) e = cudaMemset(h->ctl, 0, sizeof(DevCtl));
     int r = 0;
-    if (e == cudaSuccess) r = refactor_setup(kRefCapLong, &h->ref_blocks_per_sm, &h->batch_blocks_per_sm);
-    if (e == cudaSuccess && r == 0) r = refactor_setup_f32(kRefCapLong, &h->ref32_blocks_per_sm);
+    if (e == cudaSuccess) r = refactor_setup(h->ref_blocks_per_sm, h->batch_blocks_per_sm);
+    if (e == cudaSuccess && r == 0) r = refactor_setup_f32(h->ref32_blocks_per_sm);
     if (e == cudaSuccess && r == 0) r = solve_syncfree_grid(&h->solve_grid);
     int trail_per_sm = 0;
     if (e == cudaSuccess && r == 0) r = trail_setup(&trail_per_sm);
     if (e == cudaSuccess && r == 0) r = dense_setup(GBLU_DENSE_MAX_ROWS);
     if (e == cudaSuccess && r == 0) r = tail_setup();
-    if (e != cudaSuccess || r != 0 || h->ref_blocks_per_sm < 1 || h->batch_blocks_per_sm < 1) {
+    if (e != cudaSuccess || r != 0 || h->ref_blocks_per_sm[0] < 1 || h->batch_blocks_per_sm[0] < 1) {
         const char *msg = cudaGetErrorString(e != cudaSuccess ? e : (cudaError_t)r);
         if (h->hctl) cudaFreeHost(h->hctl);
         if (h->ctl) cudaFree(h->ctl);
@@ -1116,8 +1223,6 @@ int gblu_create(gblu_handle *out, int device, const gblu_opts *o)
         cudaGetLastError();
         return fail(GBLU_ERR_CUDA, "device setup failed: %s", msg);
     }
-    h->ref_grid = h->ref_blocks_per_sm * h->sm_count;
-    h->ref32_grid = h->ref32_blocks_per_sm * h->sm_count;
     h->res_blocks = h->sm_count * 4;
     h->trail_per_sm = std::max(1, trail_per_sm);
     *out = h;
@@ -1135,6 +1240,9 @@ void gblu_destroy(gblu_handle h)
         release(h, h->LUp); release(h, h->LUi); release(h, h->nU); release(h, h->rows); release(h, h->chain);
         release(h, h->finish); release(h, h->task_ptr); release(h, h->task_cols); release(h, h->amap);
         release(h, h->piv); release(h, h->pinv); release(h, h->vals);
+        release(h, h->pan); release(h, h->pan_id); release(h, h->prow); release(h, h->ppref); release(h, h->pmask);
+        release(h, h->prun); release(h, h->pscratch); release(h, h->tb_S); release(h, h->tb_nux); release(h, h->tb_words);
+        release(h, h->ctask_ptr); release(h, h->ctask_cols); release(h, h->camap);
         release(h, h->Lrp); release(h, h->Urp); release(h, h->Lcol); release(h, h->Lslot);
         release(h, h->Ucol); release(h, h->Uslot); release(h, h->Udiag);
         release(h, h->lsv_rows); release(h, h->usv_rows); release(h, h->lbs); release(h, h->ubs);
@@ -1569,6 +1677,58 @@ static int batch_group(gblu_ctx *h, int32_t nsets)
     return std::min(g, (int)nsets);
 }
 
+// A large batch of a structure whose columns are all short takes the columns
+// one per warp: in a panel a CTA waits for its dependencies and barriers,
+// while the warps of eight columns wait for themselves.  The line is where
+// the two took equal time on grids: 528 unknowns at 80 sets, 1,147 at 55
+// (96 sets: 1.04 ms against 1.45 ms; 8 sets: 0.69 ms against 0.36 ms), 3,300
+// at 30, 7,200 at 20.
+static bool columns_batch(const gblu_ctx *h, int32_t nsets)
+{
+    return !h->W.ctask_ptr.empty() && (double)nsets * std::sqrt((double)h->S.n) > kColumnBatch;
+}
+
+// the argument block of a batch's sets
+static RefactorArgs batch_args(gblu_ctx *h, bool columns)
+{
+    RefactorArgs a = refactor_args(h, nullptr);
+    a.dense_p = INT_MAX;   // the dense tail is not used in batches
+    if (columns) {
+        a.task_ptr = h->ctask_ptr.p;
+        a.task_cols = h->ctask_cols.p;
+        a.amap = h->camap.p;
+        a.pan_id = nullptr;
+        a.smem_bytes = kRefSmemColumns;
+        a.pscratch_ctas = 0;
+    }
+    return a;
+}
+
+// the launches of a batch's re-factorization (argument blocks args_dev, all
+// like base but for the sets' buffers)
+static int issue_batch(gblu_ctx *h, int32_t nsets, const RefactorArgs *args_dev, const RefactorArgs &base, bool columns,
+                       int epoch, cudaStream_t st)
+{
+    KL(launch_begin_batch(h->bctl.p, nsets, h->bticket.p, st));
+    RefactorArgs a0 = base;
+    const std::vector<int32_t> &ltp = columns ? h->W.clevel_task_ptr : h->W.level_task_ptr;
+    const int32_t div = h->W.div_level;
+    for (int32_t l = 0; l < div; l++) {   // cluster mode
+        a0.task_begin = ltp[l];
+        a0.ntasks = ltp[l + 1] - ltp[l];
+        KL(launch_refactor_batch(args_dev, a0, nsets, false, 0, epoch, h->bticket.p, st, nsets));
+    }
+    const int32_t ntask = (int32_t)(columns ? h->W.ctask_ptr : h->W.task_ptr).size() - 1;
+    if (ltp[div] < ntask) {               // pipeline mode
+        a0.task_begin = ltp[div];
+        a0.ntasks = ntask - ltp[div];
+        KL(launch_refactor_batch(args_dev, a0, nsets, true,
+                                 pgrid(h, h->batch_blocks_per_sm[columns ? 2 : cfg(h)]), epoch,
+                                 h->bticket.p, st, batch_group(h, nsets)));
+    }
+    return GBLU_OK;
+}
+
 int gblu_refactorize_batch(gblu_handle h, int32_t nsets, const double *Ax_dev, int64_t ax_stride,
                            double *LUx_dev, int64_t lu_stride, int32_t *failed, int32_t *n_failed,
                            void *stream)
@@ -1593,7 +1753,8 @@ int gblu_refactorize_batch(gblu_handle h, int32_t nsets, const double *Ax_dev, i
     CK(ensure(h, h->bticket, 1));
     h->epoch++;
     h->n_refactor += nsets;
-    const RefactorArgs base = refactor_args(h, nullptr);
+    const bool columns = columns_batch(h, nsets);
+    const RefactorArgs base = batch_args(h, columns);
     h->bargs_host.assign(nsets, base);
     for (int32_t s = 0; s < nsets; s++) {
         RefactorArgs &as = h->bargs_host[s];
@@ -1601,25 +1762,9 @@ int gblu_refactorize_batch(gblu_handle h, int32_t nsets, const double *Ax_dev, i
         as.LUx = LUx_dev + s * lu_stride;
         as.finish = h->bfinish.p + (size_t)s * n;
         as.ctl = h->bctl.p + s;
-        as.dense_p = INT_MAX;   // the dense tail is not used in batches
     }
     CU(cudaMemcpyAsync(h->bargs.p, h->bargs_host.data(), sizeof(RefactorArgs) * nsets, cudaMemcpyHostToDevice, st));
-    KL(launch_begin_batch(h->bctl.p, nsets, h->bticket.p, st));
-    RefactorArgs a0 = base;
-    const std::vector<int32_t> &ltp = h->W.level_task_ptr;
-    const int32_t div = h->W.div_level;
-    for (int32_t l = 0; l < div; l++) {   // cluster mode
-        a0.task_begin = ltp[l];
-        a0.ntasks = ltp[l + 1] - ltp[l];
-        KL(launch_refactor_batch(h->bargs.p, a0, nsets, false, 0, h->epoch, h->bticket.p, st, nsets));
-    }
-    const int32_t ntask = (int32_t)h->W.task_ptr.size() - 1;
-    if (ltp[div] < ntask) {               // pipeline mode
-        a0.task_begin = ltp[div];
-        a0.ntasks = ntask - ltp[div];
-        KL(launch_refactor_batch(h->bargs.p, a0, nsets, true, pgrid(h, h->batch_blocks_per_sm), h->epoch, h->bticket.p, st,
-                                 batch_group(h, nsets)));
-    }
+    CK(issue_batch(h, nsets, h->bargs.p, base, columns, h->epoch, st));
     h->bctl_host.resize(nsets);
     CU(cudaMemcpyAsync(h->bctl_host.data(), h->bctl.p, sizeof(DevCtl) * nsets, cudaMemcpyDeviceToHost, st));
     CU(cudaStreamSynchronize(st));
@@ -1716,8 +1861,13 @@ int gblu_refactorize_multi(int32_t nh, gblu_handle *hs, const double *const *Ax_
         gblu_ctx *h = h0;   // the launch is counted on the leading handle
         bool pull = false;
         for (int32_t i = 0; i < nh; i++) pull = pull || hs[i]->pull_slots > 0;
-        KL(launch_refactor_multi(h0->bargs.p, h0->bargs_host[0], nh, h0->morder.p, (int)h0->morder_n, pgrid(h0, h0->batch_blocks_per_sm),
-                                 ep, h0->bticket.p, st, pull));
+        // the larger shared memory if any handle needs it: the handles with
+        // panels in a scratch per CTA do
+        int smem = 0;
+        for (int32_t i = 0; i < nh; i++) smem = std::max(smem, hs[i]->W.smem);
+        KL(launch_refactor_multi(h0->bargs.p, nh, h0->morder.p, (int)h0->morder_n,
+                                 pgrid(h0, h0->batch_blocks_per_sm[smem == kRefSmemTwo ? 0 : 1]), smem, ep, h0->bticket.p,
+                                 st, pull));
         h->launches++;   // the control-block reset kernel
     }
     for (int32_t i = 0; i < nh; i++)
@@ -1880,7 +2030,7 @@ static int capture_step(gblu_ctx *h)
     int rc = GBLU_OK;
     if (cudaMemcpyAsync(&h->ctl->epoch, h->epoch_host, sizeof(int32_t), cudaMemcpyHostToDevice, gs) != cudaSuccess)
         rc = fail(GBLU_ERR_CUDA, "graph capture: epoch copy failed");
-    if (rc == GBLU_OK) rc = issue_refactor(h, h->stage_ax.p, gs, -1);
+    if (rc == GBLU_OK) rc = issue_refactor(h, h->stage_ax.p, gs, -1, block_applies(h));
     if (rc == GBLU_OK &&
         cudaMemcpyAsync(h->hctl, h->ctl, sizeof(DevCtl), cudaMemcpyDeviceToHost, gs) != cudaSuccess)
         rc = fail(GBLU_ERR_CUDA, "graph capture: status copy failed");
@@ -1937,8 +2087,16 @@ int gblu_step(gblu_handle h, const double *Ax_dev, const double *b_dev, double *
     h->last_first_bad = h->hctl->interrupted ? h->hctl->first_bad : -1;
     if (!h->hctl->interrupted) return GBLU_OK;
     // the check failed: the solve of the replay is void; restart, solve again
-    h->n_repivot++;
-    int rc = run_restart(h, h->stage_ax.p, st);
+    // (with a trailing block, the first failing step is not known yet)
+    int rc = GBLU_OK;
+    if (block_applies(h)) {
+        h->n_refactor--;
+        rc = gblu_refactorize(h, h->stage_ax.p, stream, nullptr);
+        if (rc == GBLU_REPIVOTED) rc = GBLU_OK;
+    } else {
+        h->n_repivot++;
+        rc = run_restart(h, h->stage_ax.p, st);
+    }
     if (rc != GBLU_OK) {
         h->factorized = false;
         return rc;
@@ -1970,14 +2128,14 @@ static int capture_step_batch(gblu_ctx *h, int32_t nsets, const double *Ax_dev, 
         h->bgctl_cap = nsets;
     }
     if (!h->gstream) CU(cudaStreamCreateWithFlags(&h->gstream, cudaStreamNonBlocking));
-    const RefactorArgs base = refactor_args(h, nullptr);
+    const bool columns = columns_batch(h, nsets);
+    const RefactorArgs base = batch_args(h, columns);
     std::vector<RefactorArgs> args(nsets, base);
     for (int32_t s = 0; s < nsets; s++) {
         args[s].Ax = Ax_dev + s * ax_stride;
         args[s].LUx = LUx_dev + s * lu_stride;
         args[s].finish = h->bfinish.p + (size_t)s * n;
         args[s].ctl = h->bctl.p + s;
-        args[s].dense_p = INT_MAX;   // the dense tail is not used in batches
     }
     cudaStream_t gs = h->gstream;
     CU(cudaMemcpyAsync(h->bgargs.p, args.data(), sizeof(RefactorArgs) * nsets, cudaMemcpyHostToDevice, gs));
@@ -1987,22 +2145,7 @@ static int capture_step_batch(gblu_ctx *h, int32_t nsets, const double *Ax_dev, 
     int rc = GBLU_OK;
     auto step = [&]() -> int {
         CU(cudaMemsetAsync(h->bfinish.p, 0, sizeof(int32_t) * (size_t)nsets * n, gs));
-        KL(launch_begin_batch(h->bctl.p, nsets, h->bticket.p, gs));
-        RefactorArgs a0 = base;
-        const std::vector<int32_t> &ltp = h->W.level_task_ptr;
-        const int32_t div = h->W.div_level;
-        for (int32_t l = 0; l < div; l++) {
-            a0.task_begin = ltp[l];
-            a0.ntasks = ltp[l + 1] - ltp[l];
-            KL(launch_refactor_batch(h->bgargs.p, a0, nsets, false, 0, 1, h->bticket.p, gs, nsets));
-        }
-        const int32_t ntask = (int32_t)h->W.task_ptr.size() - 1;
-        if (ltp[div] < ntask) {
-            a0.task_begin = ltp[div];
-            a0.ntasks = ntask - ltp[div];
-            KL(launch_refactor_batch(h->bgargs.p, a0, nsets, true, pgrid(h, h->batch_blocks_per_sm), 1, h->bticket.p, gs,
-                                     batch_group(h, nsets)));
-        }
+        CK(issue_batch(h, nsets, h->bgargs.p, base, columns, 1, gs));
         CU(cudaMemcpyAsync(h->bgctl_host, h->bctl.p, sizeof(DevCtl) * nsets, cudaMemcpyDeviceToHost, gs));
         return solve_values(h, LUx_dev, lu_stride, b_dev, b_stride, x_dev, x_stride, nsets, gs);
     };
@@ -2225,7 +2368,7 @@ int gblu_refactorize_f32(gblu_handle h, const double *Ax_dev, void *stream, int3
     if (!Ax_dev) return fail(GBLU_ERR_INVALID_INPUT, "null Ax_dev");
     DeviceGuard g(h->device);
     cudaStream_t st = (cudaStream_t)stream;
-    CK(ensure(h, h->vals32, (size_t)h->S.nnz()));
+    CK(ensure(h, h->vals32, (size_t)h->S.nnz() + 4));   // the panels' copies take whole 16-byte units
     h->epoch++;
     h->n_refactor++;
     KL(launch_begin_refactor(h->ctl, st));
@@ -2236,6 +2379,8 @@ int gblu_refactorize_f32(gblu_handle h, const double *Ax_dev, void *stream, int3
     a.LUx = h->vals32.p; a.finish = d.finish; a.task_ptr = d.task_ptr; a.task_cols = d.task_cols;
     a.cap_short = d.cap_short; a.cap_long = d.cap_long; a.eps = d.eps; a.spin_limit = d.spin_limit;
     a.ctl = d.ctl;
+    a.pan_id = d.pan_id; a.pan = d.pan; a.prow = d.prow; a.ppref = d.ppref; a.pmask = d.pmask; a.prun = d.prun;
+    a.smem_bytes = d.smem_bytes; a.pscratch = d.pscratch; a.pscratch_bytes = d.pscratch_bytes; a.pscratch_ctas = d.pscratch_ctas;
     const std::vector<int32_t> &ltp = h->W.level_task_ptr;
     const int32_t div = h->W.div_level;
     for (int32_t l = 0; l < div; l++) {
@@ -2247,7 +2392,7 @@ int gblu_refactorize_f32(gblu_handle h, const double *Ax_dev, void *stream, int3
     if (ltp[div] < ntask) {
         a.task_begin = ltp[div];
         a.ntasks = ntask - ltp[div];
-        KL(launch_refactor_tasks_f32(a, true, pgrid(h, h->ref32_blocks_per_sm), h->epoch, st));
+        KL(launch_refactor_tasks_f32(a, true, pgrid(h, h->ref32_blocks_per_sm[cfg(h)]), h->epoch, st));
     }
     // the pivots in double: a pivot that single precision cannot place
     // clearly on the passing side of the threshold fails here, and the

@@ -69,6 +69,34 @@ struct Structure {
 };
 
 // Everything derived from a Structure that the kernels use.
+// Panels of the re-factorization: up to kPanelMax consecutive columns
+// k0 .. k0+nc-1 of one supernode of L, computed together by one CTA on the
+// union of their patterns (slots): nu rows above k0, ascending, then the nc
+// diagonal-block rows, then the rows of the last column's L part.
+struct PanelDesc {
+    int64_t uoff;   // prow/pmask[uoff + s] = row and column mask of slot s < nu + nc
+    int64_t poff;   // ppref[poff + (s / 32) * nc + c] = entries of column c in slots below 32*(s/32)
+    int64_t roff;   // first of nruns runs in prun
+    int32_t k0, nc, nu, nruns;
+    int32_t nux, nrunsx;   // slots and runs of dependencies before the trailing block (k0 in the block)
+};
+// w <= kPanelRun consecutive dependencies j0 .. at slots t .. t+w-1 in one
+// supernode of L; wm = w | (mask of the panel's columns that have any of
+// them) << 8; L(:, j0+w-1) has nR rows, from LUi[lbl] on
+struct alignas(8) PanelRun {
+    int32_t t, wm, nR, j0;
+    int64_t lbl;
+};
+constexpr int kPanelRun = 16, kPanelRunBig = 16;   // (panels in a scratch)
+constexpr int kPanelWideRows = 256;   // most L rows below a panel of more than four columns
+constexpr int kPanelMax = 8;
+// columns of more entries count as long (Schedule::smem)
+constexpr int32_t kLongColumn = 3200;
+// sets * sqrt(n) from which a batch takes short columns one per warp
+constexpr double kColumnBatch = 1800.0;
+// row stride of a panel's work vector
+constexpr int panel_ld(int nc) { return nc <= 4 ? 4 : 8; }
+
 struct Schedule {
     // refactor: EGraph levels (Section II-B) and dual-mode split
     std::vector<int32_t> level_ptr;   // n_levels+1
@@ -80,7 +108,25 @@ struct Schedule {
     // tasks of level l < div_level are [level_task_ptr[l], level_task_ptr[l+1]),
     // the sync-free tasks start at level_task_ptr[div_level]
     std::vector<int32_t> task_ptr, task_cols, level_task_ptr;
-    std::vector<int32_t> amap;        // A slot -> position inside its column
+    // panels: a task of one column k with pan_id[k] >= 0 is that panel;
+    // pscratch = bytes of work vector and rows that the largest panel beyond
+    // shared memory needs (0: none)
+    std::vector<PanelDesc> pan;
+    std::vector<int32_t> pan_id;      // panel of its first column, -1 elsewhere
+    BigVec<int32_t> prow, ppref;
+    BigVec<uint8_t> pmask;
+    BigVec<PanelRun> prun;
+    int64_t pscratch = 0;
+    int32_t smem = 0;                 // dynamic shared memory of the CTAs
+    // trailing block factored densely (block.cu): columns [tb_p, n), tb_m of
+    // them (0: none); every one is in a panel; tb_nux[c] = entries of column
+    // tb_p + c in rows before the block
+    int32_t tb_p = 0, tb_m = 0;
+    std::vector<int32_t> tb_nux;
+    std::vector<int32_t> amap;        // A slot -> position inside its column (in a panel: its slot)
+    // the same tasks without panels, for large batches of a structure whose
+    // columns are all short (empty otherwise): one warp per column
+    std::vector<int32_t> ctask_ptr, ctask_cols, clevel_task_ptr, camap;
     BigVec<int32_t> LUi_orig;         // L entries: original row ids (U: step ids)
     // chain[j] = 1 iff L(:,j) = {j+1} followed by the rows of L(:,j+1), i.e.
     // j and j+1 are consecutive columns of one supernode of L
@@ -139,6 +185,11 @@ struct Schedule {
 constexpr int kPullMaxL = 64;
 constexpr int kPullMinRuns = 256;
 constexpr size_t kPullScratchBytes = (size_t)1 << 30;
+// trailing block: at least kBlockMin columns, at most kBlockMax (302 MB of
+// values), at least kBlockDensity of its entries in the factor
+constexpr int kBlockCols = 16, kBlockMin = 128, kBlockMax = 6144;
+constexpr double kBlockDensity = 0.96;
+constexpr size_t kPanelScratchBytes = (size_t)1 << 30;
 
 struct SolveSplit {
     double density = 0.0;   // > 0: longest trailing block at least this dense
@@ -184,7 +235,7 @@ int64_t unsymmetric_entries(const Pattern &P);
 // The schedule of a structure; with defer_solve, only what the
 // re-factorization reads (the solve part follows by build_solve_schedule)
 void build_schedule(const Pattern &P, const Structure &S, double alpha,
-                    int resident_warps, int sched_mode, int cap_short, const SolveSplit &split,
+                    int resident_warps, int panel_ctas, int sched_mode, int cap_short, const SolveSplit &split,
                     int dense_min_rows, Schedule &W, bool defer_solve = false);
 void build_solve_schedule(const Structure &S, const SolveSplit &split, Schedule &W);
 // levels of the column dependency graph; with cut < n, the dependencies of
@@ -265,6 +316,23 @@ struct RefactorArgsT {
     unsigned long long *pull_tag = nullptr, *pull_ctr = nullptr;
     int32_t *pull_lock = nullptr;
     int32_t pull_slots = 0, n = 0;
+    // panels (Schedule::pan); pscratch: per CTA (blockIdx.x) pscratch_bytes
+    // for the panels beyond shared memory
+    const int32_t *pan_id = nullptr;
+    const PanelDesc *pan = nullptr;
+    const int32_t *prow = nullptr, *ppref = nullptr;
+    const uint8_t *pmask = nullptr;
+    const PanelRun *prun = nullptr;
+    int32_t smem_bytes = 0;         // dynamic shared memory of a CTA
+    unsigned char *pscratch = nullptr;
+    int64_t pscratch_bytes = 0;
+    int32_t pscratch_ctas = 0;
+    // trailing block (Schedule::tb_p): panels at or after tb_p apply their
+    // dependencies before it and leave the rest in tb_S (row-major, pitch
+    // tb_ld); INT32_MAX: none
+    int32_t tb_p = INT32_MAX;
+    R *tb_S = nullptr;
+    int64_t tb_ld = 0;
 };
 using RefactorArgs = RefactorArgsT<double>;
 
@@ -324,8 +392,10 @@ struct SolveArgs {
 
 // kernel launchers (kernels.cu); each returns a cudaError_t as int
 int launch_begin_refactor(DevCtl *ctl, void *stream);
-int refactor_setup(int cap_long, int *blocks_per_sm, int *batch_blocks_per_sm);
-int refactor_setup_f32(int cap_long, int *blocks_per_sm);
+// CTAs per SM with kRefSmemTwo ([0]), kRefSmemThree ([1]) and, of the batch
+// kernel, without panels ([2])
+int refactor_setup(int *blocks_per_sm, int *batch_blocks_per_sm);
+int refactor_setup_f32(int *blocks_per_sm);
 int launch_refactor_tasks(const RefactorArgs &a, bool pipeline, int grid, int epoch, void *stream);
 // the same tasks with single-precision factor values (no dense tail)
 int launch_refactor_tasks_f32(const RefactorArgsT<float> &a, bool pipeline, int grid, int epoch, void *stream);
@@ -333,8 +403,8 @@ int launch_refactor_tasks_f32(const RefactorArgsT<float> &a, bool pipeline, int 
 int launch_begin_batch(DevCtl *ctl, int nsets, int32_t *ticket, void *stream);
 int launch_refactor_batch(const RefactorArgs *sets_dev, const RefactorArgs &a0, int nsets, bool pipeline,
                           int grid, int epoch, int32_t *ticket, void *stream, int group);
-int launch_refactor_multi(const RefactorArgs *sets_dev, const RefactorArgs &a0, int nsets, const SetTask *order_dev,
-                          int npairs, int grid, int epoch, int32_t *ticket, void *stream, bool pull);
+int launch_refactor_multi(const RefactorArgs *sets_dev, int nsets, const SetTask *order_dev, int npairs, int grid,
+                          int smem, int epoch, int32_t *ticket, void *stream, bool pull);
 int launch_begin_tail(DevCtl *ctl, unsigned long long pool_base, void *stream);
 int launch_tail_init(int32_t n, const int32_t *restart_mask, const int32_t *piv_old,
                      int32_t *pinv, int32_t *piv, int32_t *done, int epoch, void *stream);
@@ -365,6 +435,25 @@ struct DenseArgs2 {
     int32_t *finish;
     int epoch;
 };
+// LU of the trailing block (block.cu)
+struct BlockArgs {
+    double *S;                      // m x m, row-major, pitch ld
+    int64_t ld;
+    int32_t m, p;                   // columns, first of them
+    double eps;
+    DevCtl *ctl;
+    const int64_t *LUp;
+    const int32_t *LUi, *nux;
+    double *LUx;
+    int32_t *finish;
+    int epoch;                      // -1: read it from the control block
+    long long spin_limit;
+    int32_t *ticket, *flag;         // one per step, zeroed
+    unsigned long long *colmax;     // bits of max |x| over each column's L rows, zeroed
+    double *inv;                    // reciprocals of the diagonal
+};
+int block_steps(int m);
+int launch_block_lu(const BlockArgs &a, void *stream, long long *launches);
 constexpr int kDenseNb = 8;         // panel width
 int dense_setup(int max_rows);
 int launch_dense_lu(const DenseArgs2 &d, void *stream, long long *launches);
@@ -408,7 +497,16 @@ int trail_setup(int *blocks_per_sm);
 
 constexpr int kRefThreads = 256;       // 8 warps per refactor CTA
 constexpr int kRefCapShort = 640;      // work-vector entries per warp (short columns)
-constexpr int kRefCapLong = 8 * kRefCapShort;  // per CTA (long columns), 60 KB: 3 CTAs per SM
+constexpr int kRefCapLong = 8 * kRefCapShort;  // per CTA (long columns), 60 KB
+// dynamic shared memory of a re-factorization CTA: two CTAs per SM, or three
+// (and a larger L1) where most of the work is in columns beyond panels
+constexpr int kRefSmemTwo = 100 * 1024, kRefSmemThree = 65 * 1024;
+// of a launch without panels: the column kernels' work vectors alone
+constexpr int kRefSmemColumns = kRefCapLong * (int)(sizeof(double) + sizeof(int32_t));
+// stage ring of a panel: four stages of kStageCap values (work vector in
+// shared memory), or three of kStageCapBig; kPanelRing = bytes of the former
+constexpr int kStageCap = 576, kStageCapBig = 2112;
+constexpr int kPanelRing = 4 * (kStageCap * 8 + 128 * 4 + 128);
 constexpr int kTailThreads = 256;
 constexpr int kSolveWarpsPerBlock = 8;
 constexpr int kSolveBlockRows = 32;   // rows of one block of the sparse solves

@@ -261,7 +261,11 @@ __device__ bool col_warp(const RefactorArgsT<R> &a, int k, R *xs, int32_t *rs, i
         R *Sc = a.S + (int64_t)(k - a.dense_p) * a.dense_ld;
         if (in_smem)
             for (int i = lane; i < nD; i += 32) a.LUx[beg + i] = xs[i];
-        for (int i = nD + lane; i < len; i += 32) Sc[i - nD] = x[i];
+        if (a.tb_ld) {   // trailing block (block.cu): row-major
+            for (int i = nD + lane; i < len; i += 32) a.tb_S[(int64_t)(rows[i] - a.dense_p) * a.tb_ld + (k - a.dense_p)] = x[i];
+        } else {
+            for (int i = nD + lane; i < len; i += 32) Sc[i - nD] = x[i];
+        }
         return false;
     }
     // m = max |x(L rows)|, NaN if one of them is NaN; with an infinite m or
@@ -777,7 +781,11 @@ __device__ bool col_grp(const RefactorArgsT<R> &a, int k, R *xs, int32_t *rs, in
         R *Sc = a.S + (int64_t)(k - a.dense_p) * a.dense_ld;
         if (in_smem)
             for (int i = tid; i < nD; i += kT) a.LUx[beg + i] = xs[i];
-        for (int i = nD + tid; i < len; i += kT) Sc[i - nD] = x[i];
+        if (a.tb_ld) {
+            for (int i = nD + tid; i < len; i += kT) a.tb_S[(int64_t)(rows[i] - a.dense_p) * a.tb_ld + (k - a.dense_p)] = x[i];
+        } else {
+            for (int i = nD + tid; i < len; i += kT) Sc[i - nD] = x[i];
+        }
         return false;
     }
     // m = max |x(L rows)|, NaN if one of them is NaN; with an infinite m or
@@ -810,6 +818,18 @@ __device__ bool col_grp(const RefactorArgsT<R> &a, int k, R *xs, int32_t *rs, in
     return false;
 }
 
+}  // namespace
+
+}  // namespace gblu
+
+#include "panel.cuh"
+
+namespace gblu {
+
+namespace {
+
+using namespace dev;
+
 __global__ void begin_refactor_kernel(DevCtl *ctl)
 {
     ctl->ticket = 0;
@@ -820,16 +840,29 @@ __global__ void begin_refactor_kernel(DevCtl *ctl)
     ctl->where_k = -1;
 }
 
-// One task of the schedule: one long column (whole CTA), two medium
+// static shared memory of a task: a panel's, or two groups'
+template <typename R>
+union TaskShared {
+    PanelShared<R> pan;
+    GroupShared<R> grp[2];
+};
+
+// One task of the schedule: a panel, one long column (whole CTA), two medium
 // columns (a half each) or up to 8 short ones (a warp each); true = stop.
-template <typename R, bool kWait, bool kDense, bool kPull>
-__device__ __forceinline__ bool run_task(const RefactorArgsT<R> &a, int tt, R *xs, int32_t *rs, int epoch,
-                                         GroupShared<R> *s_grp)
+template <typename R, bool kWait, bool kDense, bool kPull, bool kPanel>
+__device__ __forceinline__ bool run_task(const RefactorArgsT<R> &a, const RefactorArgsT<R> *ap, int tt, R *xs, int32_t *rs, int epoch,
+                                         TaskShared<R> &s_sh, PanelBars &bars)
 {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int c0 = __ldg(a.task_ptr + tt), c1 = __ldg(a.task_ptr + tt + 1);
     const int k0 = __ldg(a.task_cols + c0);
     const int64_t len0 = __ldg(a.LUp + k0 + 1) - __ldg(a.LUp + k0);
+    if constexpr (kPanel) {
+        const int id = c1 - c0 == 1 ? __ldg(a.pan_id + k0) : -1;
+        if (id >= 0)
+            return run_panel<R>(ap, id, reinterpret_cast<unsigned char *>(xs), a.smem_bytes, s_sh.pan, bars, epoch, kWait);
+    }
+    GroupShared<R> *s_grp = s_sh.grp;
     if (c1 - c0 == 1 && len0 > a.cap_short)            // one long column: whole CTA
         return col_grp<R, kWait, kDense, kWarps, kPull>(a, k0, xs, rs, epoch, 0, a.cap_long, s_grp[0]);
     if (c1 - c0 == 2 && len0 > a.cap_short) {          // two medium columns: a half each
@@ -846,28 +879,31 @@ __device__ __forceinline__ bool run_task(const RefactorArgsT<R> &a, int tt, R *x
     return __syncthreads_or(ws);
 }
 
-// Tasks [task_begin, task_begin + ntasks): one per CTA in cluster mode
-// (persistent == 0), taken by ticket in pipeline mode (persistent == 1).
+// Tasks [task_begin, task_begin + ntasks): dealt to the CTAs in cluster mode
+// (persistent == 0; one each, or several where panels use the CTAs'
+// scratches, of which there are pscratch_ctas), taken by ticket in pipeline mode (persistent == 1).
 template <typename R, bool kWait, bool kDense, bool kPull>
-__global__ void __launch_bounds__(kThreads, 3) refactor_task_kernel(RefactorArgsT<R> a, int epoch, int persistent)
+__global__ void __launch_bounds__(kThreads, 3) refactor_task_kernel(const __grid_constant__ RefactorArgsT<R> a, int epoch, int persistent)
 {
     // a replayed graph passes -1: the epoch was written to the control block
     if (epoch < 0) epoch = ld_volatile(&a.ctl->epoch);
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_t, s_quit;
-    __shared__ GroupShared<R> s_grp[2];
+    __shared__ TaskShared<R> s_sh;
+    __shared__ PanelBars s_bars;
+    if (threadIdx.x == 0) init_bars(s_bars);
     R *xs = reinterpret_cast<R *>(smem);
     int32_t *rs = reinterpret_cast<int32_t *>(smem + (size_t)a.cap_long * sizeof(R));
     for (int iter = 0;; ++iter) {
         if (threadIdx.x == 0) {
-            s_t = persistent ? atomicAdd(&a.ctl->ticket, 1) : (iter == 0 ? (int)blockIdx.x : a.ntasks);
+            s_t = persistent ? atomicAdd(&a.ctl->ticket, 1) : (int)blockIdx.x + iter * (int)gridDim.x;
             s_quit = ld_volatile(&a.ctl->interrupted) || ld_volatile(&a.ctl->status);
         }
         __syncthreads();
         const int t = s_t, quit = s_quit;
         __syncthreads();
         if (t >= a.ntasks || quit) break;
-        if (run_task<R, kWait, kDense, kPull>(a, a.task_begin + t, xs, rs, epoch, s_grp)) break;
+        if (run_task<R, kWait, kDense, kPull, true>(a, &a, a.task_begin + t, xs, rs, epoch, s_sh, s_bars)) break;
     }
 }
 
@@ -908,14 +944,17 @@ __device__ __forceinline__ int group_task(long long t, int ntasks, int nsets, in
     return task;
 }
 
-template <bool kWait, bool kPull>
+// kPanel = false: a task list without panels (the column kernels alone)
+template <bool kWait, bool kPull, bool kPanel>
 __global__ void __launch_bounds__(kThreads, 3)
 refactor_batch_kernel(const RefactorArgs *sets, int nsets, int task_begin, int ntasks, int epoch, int persistent,
                       int32_t *ticket, const SetTask *order, int group)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_t, s_skip;
-    __shared__ GroupShared<double> s_grp[2];
+    __shared__ TaskShared<double> s_sh;
+    __shared__ PanelBars s_bars;
+    if (threadIdx.x == 0) init_bars(s_bars);
     double *xs = reinterpret_cast<double *>(smem);
     int32_t *rs = reinterpret_cast<int32_t *>(smem + (size_t)sets[0].cap_long * sizeof(double));
     // ticket t: task t / nsets of set t % nsets, or, with an order array
@@ -923,7 +962,7 @@ refactor_batch_kernel(const RefactorArgs *sets, int nsets, int task_begin, int n
     const long long total = order ? (long long)ntasks : (long long)ntasks * nsets;
     for (int iter = 0;; ++iter) {
         if (threadIdx.x == 0) {
-            const long long t = persistent ? (long long)atomicAdd(ticket, 1) : (iter == 0 ? (long long)blockIdx.x : total);
+            const long long t = persistent ? (long long)atomicAdd(ticket, 1) : (long long)blockIdx.x + (long long)iter * gridDim.x;
             s_t = t < total ? (int)t : -1;
             s_skip = 0;
             if (t < total) {
@@ -942,7 +981,7 @@ refactor_batch_kernel(const RefactorArgs *sets, int nsets, int task_begin, int n
         // a local copy: stores through the work vector cannot alias it, so its
         // fields stay in registers instead of being reloaded from memory
         const RefactorArgs as = sets[si];
-        run_task<double, kWait, false, kPull>(as, task, xs, rs, epoch, s_grp);
+        run_task<double, kWait, false, kPull, kPanel>(as, sets + si, task, xs, rs, epoch, s_sh, s_bars);
     }
 }
 
@@ -974,13 +1013,14 @@ __global__ void begin_batch_kernel(DevCtl *ctl, int nsets, int32_t *ticket)
     if (blockIdx.x == 0 && threadIdx.x == 0) *ticket = 0;
 }
 
-template <typename R>
-size_t task_smem(const RefactorArgsT<R> &a)
-{
-    return (size_t)a.cap_long * (sizeof(R) + sizeof(int32_t));
-}
-
 }  // namespace
+
+// CTAs of a cluster-mode launch of `tasks` tasks
+template <typename R>
+static unsigned level_grid(const RefactorArgsT<R> &a, long long tasks)
+{
+    return (unsigned)(a.pscratch_ctas > 0 ? std::min<long long>(tasks, a.pscratch_ctas) : tasks);
+}
 
 int launch_begin_refactor(DevCtl *ctl, void *stream)
 {
@@ -995,9 +1035,9 @@ static cudaError_t allow_smem(K kernel, size_t sm, cudaError_t e)
     return e == cudaSuccess ? cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) : e;
 }
 
-int refactor_setup(int cap_long, int *blocks_per_sm, int *batch_blocks_per_sm)
+int refactor_setup(int *blocks_per_sm, int *batch_blocks_per_sm)
 {
-    const size_t sm = (size_t)cap_long * (sizeof(double) + sizeof(int32_t));
+    const size_t sm = kRefSmemTwo;
     cudaError_t e = cudaSuccess;
     e = allow_smem(refactor_task_kernel<double, true, false, false>, sm, e);
     e = allow_smem(refactor_task_kernel<double, false, false, false>, sm, e);
@@ -1005,27 +1045,32 @@ int refactor_setup(int cap_long, int *blocks_per_sm, int *batch_blocks_per_sm)
     e = allow_smem(refactor_task_kernel<double, false, true, false>, sm, e);
     e = allow_smem(refactor_task_kernel<double, true, false, true>, sm, e);
     e = allow_smem(refactor_task_kernel<double, false, false, true>, sm, e);
-    e = allow_smem(refactor_batch_kernel<true, false>, sm, e);
-    e = allow_smem(refactor_batch_kernel<false, false>, sm, e);
-    e = allow_smem(refactor_batch_kernel<true, true>, sm, e);
-    e = allow_smem(refactor_batch_kernel<false, true>, sm, e);
+    e = allow_smem(refactor_batch_kernel<true, false, true>, sm, e);
+    e = allow_smem(refactor_batch_kernel<false, false, true>, sm, e);
+    e = allow_smem(refactor_batch_kernel<true, true, true>, sm, e);
+    e = allow_smem(refactor_batch_kernel<false, true, true>, sm, e);
+    e = allow_smem(refactor_batch_kernel<true, false, false>, sm, e);
+    e = allow_smem(refactor_batch_kernel<false, false, false>, sm, e);
     if (e != cudaSuccess) return (int)e;
-    // persistent grids are sized for the instantiation that fits fewest
-    int b[3] = {0, 0, 0};
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b[0], refactor_task_kernel<double, true, false, false>, kThreads, sm);
+    // persistent grids are sized for the instantiation that fits fewest (the
+    // batch kernel keeps a copy of its set's argument block)
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b[1], refactor_task_kernel<double, true, true, false>, kThreads, sm);
-    if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b[2], refactor_task_kernel<double, true, false, true>, kThreads, sm);
-    *blocks_per_sm = std::min(b[0], std::min(b[1], b[2]));
-    // the batch kernel keeps a copy of its set's argument block (it spills a
-    // few registers at three CTAs per SM, which measured faster than two)
-    int c[2] = {0, 0};
-    if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c[0], refactor_batch_kernel<true, false>, kThreads, sm);
-    if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c[1], refactor_batch_kernel<true, true>, kThreads, sm);
-    *batch_blocks_per_sm = std::min(c[0], c[1]);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&batch_blocks_per_sm[2], refactor_batch_kernel<true, false, false>,
+                                                          kThreads, kRefSmemColumns);
+    for (int i = 0; i < 2 && e == cudaSuccess; i++) {
+        const size_t bytes = i == 0 ? kRefSmemTwo : kRefSmemThree;
+        int b[5] = {0, 0, 0, 0, 0};
+        auto fit = [&](int &out, auto kernel) {
+            if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&out, kernel, kThreads, bytes);
+        };
+        fit(b[0], refactor_task_kernel<double, true, false, false>);
+        fit(b[1], refactor_task_kernel<double, true, true, false>);
+        fit(b[2], refactor_task_kernel<double, true, false, true>);
+        fit(b[3], refactor_batch_kernel<true, false, true>);
+        fit(b[4], refactor_batch_kernel<true, true, true>);
+        blocks_per_sm[i] = std::min(b[0], std::min(b[1], b[2]));
+        batch_blocks_per_sm[i] = std::min(b[3], b[4]);
+    }
     return (int)e;
 }
 
@@ -1043,28 +1088,34 @@ int launch_refactor_batch(const RefactorArgs *sets_dev, const RefactorArgs &a0, 
     cudaStream_t st = (cudaStream_t)stream;
     if (group < 1 || group > nsets) group = nsets;
     if (pipeline) {
-        if (a0.pull_start)
-            refactor_batch_kernel<true, true><<<grid, kThreads, task_smem(a0), st>>>(
+        if (!a0.pan_id)
+            refactor_batch_kernel<true, false, false><<<grid, kThreads, a0.smem_bytes, st>>>(
+                sets_dev, nsets, a0.task_begin, a0.ntasks, epoch, 1, ticket, nullptr, group);
+        else if (a0.pull_start)
+            refactor_batch_kernel<true, true, true><<<grid, kThreads, a0.smem_bytes, st>>>(
                 sets_dev, nsets, a0.task_begin, a0.ntasks, epoch, 1, ticket, nullptr, group);
         else
-            refactor_batch_kernel<true, false><<<grid, kThreads, task_smem(a0), st>>>(
+            refactor_batch_kernel<true, false, true><<<grid, kThreads, a0.smem_bytes, st>>>(
                 sets_dev, nsets, a0.task_begin, a0.ntasks, epoch, 1, ticket, nullptr, group);
     } else {
         // a level launch has no waits: one group holding every set
         const long long blocks = (long long)a0.ntasks * nsets;
         if (blocks > INT_MAX) return (int)cudaErrorInvalidValue;
-        if (a0.pull_start)
-            refactor_batch_kernel<false, true><<<(unsigned)blocks, kThreads, task_smem(a0), st>>>(
+        if (!a0.pan_id)
+            refactor_batch_kernel<false, false, false><<<level_grid(a0, blocks), kThreads, a0.smem_bytes, st>>>(
+                sets_dev, nsets, a0.task_begin, a0.ntasks, epoch, 0, ticket, nullptr, nsets);
+        else if (a0.pull_start)
+            refactor_batch_kernel<false, true, true><<<level_grid(a0, blocks), kThreads, a0.smem_bytes, st>>>(
                 sets_dev, nsets, a0.task_begin, a0.ntasks, epoch, 0, ticket, nullptr, nsets);
         else
-            refactor_batch_kernel<false, false><<<(unsigned)blocks, kThreads, task_smem(a0), st>>>(
+            refactor_batch_kernel<false, false, true><<<level_grid(a0, blocks), kThreads, a0.smem_bytes, st>>>(
                 sets_dev, nsets, a0.task_begin, a0.ntasks, epoch, 0, ticket, nullptr, nsets);
     }
     return (int)cudaGetLastError();
 }
 
-int launch_refactor_multi(const RefactorArgs *sets_dev, const RefactorArgs &a0, int nsets, const SetTask *order_dev,
-                          int npairs, int grid, int epoch, int32_t *ticket, void *stream, bool pull)
+int launch_refactor_multi(const RefactorArgs *sets_dev, int nsets, const SetTask *order_dev, int npairs, int grid,
+                          int smem, int epoch, int32_t *ticket, void *stream, bool pull)
 {
     if (npairs <= 0 || nsets <= 0) return 0;
     cudaStream_t st = (cudaStream_t)stream;
@@ -1072,33 +1123,31 @@ int launch_refactor_multi(const RefactorArgs *sets_dev, const RefactorArgs &a0, 
     begin_multi_kernel<<<g, 256, 0, st>>>(sets_dev, nsets, ticket);
     // pull: some set has wide columns (each set's argument block says which)
     if (pull)
-        refactor_batch_kernel<true, true><<<grid, kThreads, task_smem(a0), st>>>(sets_dev, nsets, 0, npairs, epoch, 1, ticket,
+        refactor_batch_kernel<true, true, true><<<grid, kThreads, smem, st>>>(sets_dev, nsets, 0, npairs, epoch, 1, ticket,
                                                                        order_dev, 1);
     else
-        refactor_batch_kernel<true, false><<<grid, kThreads, task_smem(a0), st>>>(sets_dev, nsets, 0, npairs, epoch, 1, ticket,
+        refactor_batch_kernel<true, false, true><<<grid, kThreads, smem, st>>>(sets_dev, nsets, 0, npairs, epoch, 1, ticket,
                                                                        order_dev, 1);
     return (int)cudaGetLastError();
 }
 
-int refactor_setup_f32(int cap_long, int *blocks_per_sm)
+int refactor_setup_f32(int *blocks_per_sm)
 {
-    const size_t sm = (size_t)cap_long * (sizeof(float) + sizeof(int32_t));
-    cudaError_t e = cudaFuncSetAttribute(refactor_task_kernel<float, true, false, false>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(refactor_task_kernel<float, false, false, false>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return (int)e;
-    return (int)cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, refactor_task_kernel<float, true, false, false>,
-                                                              kThreads, sm);
+    cudaError_t e = cudaSuccess;
+    e = allow_smem(refactor_task_kernel<float, true, false, false>, kRefSmemTwo, e);
+    e = allow_smem(refactor_task_kernel<float, false, false, false>, kRefSmemTwo, e);
+    for (int i = 0; i < 2 && e == cudaSuccess; i++)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm[i], refactor_task_kernel<float, true, false, false>,
+                                                          kThreads, i == 0 ? kRefSmemTwo : kRefSmemThree);
+    return (int)e;
 }
 
 int launch_refactor_tasks_f32(const RefactorArgsT<float> &a, bool pipeline, int grid, int epoch, void *stream)
 {
     if (a.ntasks <= 0) return 0;
     cudaStream_t st = (cudaStream_t)stream;
-    if (pipeline) refactor_task_kernel<float, true, false, false><<<grid, kThreads, task_smem(a), st>>>(a, epoch, 1);
-    else refactor_task_kernel<float, false, false, false><<<a.ntasks, kThreads, task_smem(a), st>>>(a, epoch, 0);
+    if (pipeline) refactor_task_kernel<float, true, false, false><<<grid, kThreads, a.smem_bytes, st>>>(a, epoch, 1);
+    else refactor_task_kernel<float, false, false, false><<<level_grid(a, a.ntasks), kThreads, a.smem_bytes, st>>>(a, epoch, 0);
     return (int)cudaGetLastError();
 }
 
@@ -1108,14 +1157,14 @@ int launch_refactor_tasks(const RefactorArgs &a, bool pipeline, int grid, int ep
     cudaStream_t st = (cudaStream_t)stream;
     const bool dense = a.dense_p < INT_MAX;   // a dense tail is in use
     if (pipeline) {
-        if (dense) refactor_task_kernel<double, true, true, false><<<grid, kThreads, task_smem(a), st>>>(a, epoch, 1);
-        else if (a.pull_start) refactor_task_kernel<double, true, false, true><<<grid, kThreads, task_smem(a), st>>>(a, epoch, 1);
-        else refactor_task_kernel<double, true, false, false><<<grid, kThreads, task_smem(a), st>>>(a, epoch, 1);
+        if (dense) refactor_task_kernel<double, true, true, false><<<grid, kThreads, a.smem_bytes, st>>>(a, epoch, 1);
+        else if (a.pull_start) refactor_task_kernel<double, true, false, true><<<grid, kThreads, a.smem_bytes, st>>>(a, epoch, 1);
+        else refactor_task_kernel<double, true, false, false><<<grid, kThreads, a.smem_bytes, st>>>(a, epoch, 1);
     } else {
-        if (dense) refactor_task_kernel<double, false, true, false><<<a.ntasks, kThreads, task_smem(a), st>>>(a, epoch, 0);
+        if (dense) refactor_task_kernel<double, false, true, false><<<level_grid(a, a.ntasks), kThreads, a.smem_bytes, st>>>(a, epoch, 0);
         else if (a.pull_start)
-            refactor_task_kernel<double, false, false, true><<<a.ntasks, kThreads, task_smem(a), st>>>(a, epoch, 0);
-        else refactor_task_kernel<double, false, false, false><<<a.ntasks, kThreads, task_smem(a), st>>>(a, epoch, 0);
+            refactor_task_kernel<double, false, false, true><<<level_grid(a, a.ntasks), kThreads, a.smem_bytes, st>>>(a, epoch, 0);
+        else refactor_task_kernel<double, false, false, false><<<level_grid(a, a.ntasks), kThreads, a.smem_bytes, st>>>(a, epoch, 0);
     }
     return (int)cudaGetLastError();
 }

@@ -532,8 +532,218 @@ void build_solve_schedule(const Structure &S, const SolveSplit &split, Schedule 
     W.solve_ready = true;
 }
 
+// Panels of the re-factorization (Schedule::pan): the columns of each
+// supernode of L whose neighbours also depend on one another, cut from the
+// lowest up.  kPanelMax columns while they have at most kPanelWideRows rows
+// below them and their union fits in a CTA's shared memory (1,167 slots),
+// else four, in shared memory (2,204 slots) or in a scratch of the CTA
+// (allow_scratch).  Wide columns and the dense
+// tail stay single.
+static void build_panels(const Structure &S, int panel_ctas, bool allow_scratch, Schedule &W)
+{
+    const int32_t n = S.n;
+    W.pan.clear();
+    W.prow.clear();
+    W.pmask.clear();
+    W.ppref.clear();
+    W.prun.clear();
+    W.pan_id.assign(n, -1);
+    W.pscratch = 0;
+    if (W.dense_m > 0 || n == 0) return;
+    // link[j]: columns j and j+1 may share a panel
+    auto link = [&](int32_t j) {
+        return j + 1 != W.tb_p && W.chain[j] && !W.pull_start[j] && !W.pull_start[j + 1] && S.nU[j + 1] >= 2 &&
+               S.LUi[S.LUp[j + 1] + S.nU[j + 1] - 2] == j;
+    };
+    const int64_t smem = W.smem;
+    auto fits = [smem](int64_t slots, int nc) {
+        return slots * (8 * panel_ld(nc) + 4) <= smem - kPanelRing;
+    };
+    struct Part {
+        std::vector<PanelDesc> pan;
+        std::vector<int32_t> prow, ppref;
+        std::vector<uint8_t> pmask;
+        int64_t scratch = 0;
+    };
+    // small structures stay on this thread
+    auto in_chunks = [&](int32_t m, int32_t chunk, auto &&fn) {
+        if (S.nnz() < (1 << 19)) fn(0, m, 0);
+        else parallel_chunks(m, chunk, fn);
+    };
+    const int32_t chunk = 1024, nparts = (n + chunk - 1) / chunk;
+    std::vector<Part> parts(nparts);
+    in_chunks(n, chunk, [&](int32_t c0, int32_t c1, int) {
+        // one call has every part when it runs serially
+        for (int32_t b = c0; b < c1; b += chunk) {
+            Part &pt = parts[b / chunk];
+            std::vector<std::pair<int32_t, uint8_t>> u, v, m;
+            // the union of the U rows above k of columns k .. k+nc-1
+            auto join = [&](int32_t k, int nc) {
+                u.clear();
+                for (int c = 0; c < nc; c++) {
+                    const int32_t *r = S.LUi.data() + S.LUp[k + c];
+                    const int32_t cnt = (int32_t)(std::lower_bound(r, r + S.nU[k + c], k) - r);
+                    const uint8_t bit = (uint8_t)(1u << c);
+                    v.clear();
+                    size_t i = 0;
+                    int32_t q = 0;
+                    while (i < u.size() || q < cnt) {
+                        if (q == cnt || (i < u.size() && u[i].first < r[q])) v.push_back(u[i++]);
+                        else if (i == u.size() || r[q] < u[i].first) v.push_back({r[q++], bit});
+                        else { v.push_back({u[i].first, (uint8_t)(u[i].second | bit)}); i++; q++; }
+                    }
+                    u.swap(v);
+                }
+            };
+            const int32_t e = std::min(b + chunk, n);
+            int32_t k = b;
+            while (k < e && k > 0 && link(k - 1)) k++;   // a chain that began in an earlier part
+            while (k < e) {
+                int32_t end = k + 1;
+                while (end < n && link(end - 1)) end++;
+                for (; k < end;) {
+                    const int32_t left = end - k;
+                    if (left == 1) { k++; break; }   // a column of its own
+                    int nc = std::min<int32_t>(left, kPanelMax);
+                    auto l_rows = [&](int c) { return S.LUp[k + c + 1] - S.LUp[k + c] - S.nU[k + c]; };
+                    auto most = [&](int c) {   // the union has at least this many slots
+                        int64_t mx = 0;
+                        for (int i = 0; i < c; i++) mx = std::max(mx, (int64_t)S.nU[k + i] - 1 - i);
+                        return mx + c + l_rows(c - 1);
+                    };
+                    int64_t slots = 0;
+                    if (nc > 4) {
+                        bool ok = l_rows(nc - 1) <= kPanelWideRows && fits(most(nc), nc);
+                        if (ok) {
+                            join(k, nc);
+                            slots = (int64_t)u.size() + nc + l_rows(nc - 1);
+                            ok = fits(slots, nc);
+                        }
+                        if (!ok) nc = 4;
+                    }
+                    if (nc <= 4) {
+                        join(k, nc);
+                        slots = (int64_t)u.size() + nc + l_rows(nc - 1);
+                        if (!fits(slots, nc) && !allow_scratch) { k++; continue; }
+                    }
+                    const int64_t need = slots * (8 * panel_ld(nc) + 4);
+                    if (!fits(slots, nc)) pt.scratch = std::max(pt.scratch, (need + 255) / 256 * 256);
+                    PanelDesc d;
+                    d.k0 = k;
+                    d.nc = nc;
+                    d.nu = (int32_t)u.size();
+                    d.uoff = (int64_t)pt.prow.size();
+                    d.poff = (int64_t)pt.ppref.size();
+                    d.roff = 0;
+                    d.nruns = 0;
+                    int32_t cnt[kPanelMax] = {};
+                    for (int32_t s = 0; s < d.nu; s++) {
+                        if (s % 32 == 0)
+                            for (int c = 0; c < nc; c++) pt.ppref.push_back(cnt[c]);
+                        pt.prow.push_back(u[s].first);
+                        pt.pmask.push_back(u[s].second);
+                        for (int c = 0; c < nc; c++) cnt[c] += (u[s].second >> c) & 1;
+                    }
+                    for (int q = 0; q < nc; q++) {   // diagonal-block rows
+                        unsigned mk = 0;
+                        for (int c = 0; c < nc; c++) {
+                            const int32_t *r = S.LUi.data() + S.LUp[k + c];
+                            if (q >= c || std::binary_search(r, r + S.nU[k + c], k + q)) mk |= 1u << c;
+                        }
+                        pt.prow.push_back(k + q);
+                        pt.pmask.push_back((uint8_t)mk);
+                    }
+                    pt.pan.push_back(d);
+                    k += nc;
+                }
+                k = end;
+            }
+        }
+    });
+    std::vector<int64_t> op(nparts + 1, 0), ou(nparts + 1, 0), of(nparts + 1, 0);
+    for (int32_t i = 0; i < nparts; i++) {
+        op[i + 1] = op[i] + (int64_t)parts[i].pan.size();
+        ou[i + 1] = ou[i] + (int64_t)parts[i].prow.size();
+        of[i + 1] = of[i] + (int64_t)parts[i].ppref.size();
+        W.pscratch = std::max(W.pscratch, parts[i].scratch);
+    }
+    if (W.pscratch > 0 && (size_t)W.pscratch * (size_t)panel_ctas > kPanelScratchBytes && allow_scratch) {
+        // long columns one at a time
+        build_panels(S, panel_ctas, false, W);
+        return;
+    }
+    W.pan.resize(op[nparts]);
+    W.prow.resize(ou[nparts]);
+    W.pmask.resize(ou[nparts]);
+    W.ppref.resize(of[nparts]);
+    in_chunks(nparts, 1, [&](int32_t i0, int32_t i1, int) {
+        for (int32_t i = i0; i < i1; i++) {
+            Part &pt = parts[i];
+            std::copy(pt.prow.begin(), pt.prow.end(), W.prow.begin() + ou[i]);
+            std::copy(pt.pmask.begin(), pt.pmask.end(), W.pmask.begin() + ou[i]);
+            std::copy(pt.ppref.begin(), pt.ppref.end(), W.ppref.begin() + of[i]);
+            for (size_t q = 0; q < pt.pan.size(); q++) {
+                PanelDesc d = pt.pan[q];
+                d.uoff += ou[i];
+                d.poff += of[i];
+                W.pan[op[i] + (int64_t)q] = d;
+                W.pan_id[d.k0] = (int32_t)(op[i] + (int64_t)q);
+            }
+            pt = Part();
+        }
+    });
+    // runs of up to kPanelRun linked dependencies; the last kPanelRun
+    // dependencies, which may still be in progress when the panel meets
+    // them, are cut where a panel of theirs begins, so that a run waits for
+    // no more columns than it needs
+    const int32_t npan = (int32_t)W.pan.size(), pchunk = 64, nrp = (npan + pchunk - 1) / pchunk;
+    std::vector<std::vector<PanelRun>> runs(nrp);
+    in_chunks(npan, pchunk, [&](int32_t p0, int32_t p1, int) {
+        for (int32_t p = p0; p < p1; p++) {
+            std::vector<PanelRun> &out = runs[p / pchunk];
+            PanelDesc &d = W.pan[p];
+            const int32_t *u = W.prow.data() + d.uoff;
+            const uint8_t *m = W.pmask.data() + d.uoff;
+            d.roff = (int64_t)out.size();
+            const int32_t kl = d.k0 + d.nc - 1;
+            const int most = fits(d.nu + d.nc + S.LUp[kl + 1] - S.LUp[kl] - S.nU[kl], d.nc) ? kPanelRun : kPanelRunBig;
+            for (int32_t s = 0; s < d.nu;) {
+                int w = 1;
+                unsigned mk = m[s];
+                while (w < most && s + w < d.nu && u[s + w] == u[s + w - 1] + 1 && W.chain[u[s + w - 1]] &&
+                       u[s + w] != W.tb_p && !(d.nu - (s + w) <= kPanelRun && W.pan_id[u[s + w]] >= 0)) {
+                    mk |= m[s + w];
+                    w++;
+                }
+                const int32_t jl = u[s + w - 1];
+                PanelRun r;
+                r.t = s;
+                r.wm = (int32_t)(w | (mk << 8));
+                r.lbl = S.LUp[jl] + S.nU[jl];
+                r.nR = (int32_t)(S.LUp[jl + 1] - r.lbl);
+                r.j0 = u[s];
+                out.push_back(r);
+                s += w;
+            }
+            d.nruns = (int32_t)((int64_t)out.size() - d.roff);
+            d.nux = (int32_t)(std::lower_bound(u, u + d.nu, W.tb_p) - u);
+            d.nrunsx = 0;
+            while (d.nrunsx < d.nruns && out[d.roff + d.nrunsx].t < d.nux) d.nrunsx++;
+        }
+    });
+    std::vector<int64_t> orr(nrp + 1, 0);
+    for (int32_t i = 0; i < nrp; i++) orr[i + 1] = orr[i] + (int64_t)runs[i].size();
+    W.prun.resize(orr[nrp]);
+    in_chunks(nrp, 1, [&](int32_t i0, int32_t i1, int) {
+        for (int32_t i = i0; i < i1; i++) {
+            std::copy(runs[i].begin(), runs[i].end(), W.prun.begin() + orr[i]);
+            for (int32_t p = i * pchunk; p < std::min((i + 1) * pchunk, npan); p++) W.pan[p].roff += orr[i];
+        }
+    });
+}
+
 void build_schedule(const Pattern &P, const Structure &S, double alpha,
-                    int resident_warps, int sched_mode, int cap_short, const SolveSplit &split,
+                    int resident_warps, int panel_ctas, int sched_mode, int cap_short, const SolveSplit &split,
                     int dense_min_rows, Schedule &W, bool defer_solve)
 {
     const int32_t n = S.n;
@@ -610,8 +820,76 @@ void build_schedule(const Pattern &P, const Structure &S, double alpha,
         });
         W.pull_cols = cnt.load();
     }
+    // ---- trailing block: the longest [p, n) in which the factor holds at
+    // least kBlockDensity of the entries; of predicted structures (L and U^T
+    // have one pattern, so L's entries tell) without wide columns ----
+    W.tb_p = n;
+    W.tb_m = 0;
+    if (S.symmetric && W.dense_m == 0 && W.pull_cols == 0) {
+        int64_t held = 0;
+        for (int32_t p = n - 1; p >= 0 && n - p <= kBlockMax; p--) {
+            held += S.LUp[p + 1] - S.LUp[p] - S.nU[p];
+            const int64_t m = n - p;
+            if (m >= kBlockMin && (double)held >= kBlockDensity * 0.5 * (double)m * (double)(m - 1)) {
+                W.tb_p = p;
+                W.tb_m = (int32_t)m;
+            }
+        }
+    }
+    // ---- flops of one refactorization (partial sums of integers, exact in
+    // any order below 2^53), and those of long columns outside the block ----
+    double part[kHostThreads][3] = {};
+    parallel_ranges(n, S.LUp.data(), [&](int32_t k0, int32_t k1, int t) {
+        double fl = 0, outside = 0, lng = 0;
+        for (int32_t k = k0; k < k1; k++) {
+            const int64_t b = S.LUp[k], e = b + S.nU[k] - 1;
+            const int32_t lim = k < W.tb_p ? n : W.tb_p;
+            double f = 0, o = 0;
+            for (int64_t i = b; i < e; i++) {
+                const int32_t j = S.LUi[i];
+                const double v = 2.0 * (double)(S.LUp[j + 1] - S.LUp[j] - S.nU[j]);
+                f += v;
+                if (j < lim) o += v;
+            }
+            fl += f;
+            outside += o;
+            if (S.LUp[k + 1] - b > kLongColumn) lng += o;
+        }
+        part[t][0] = fl;
+        part[t][1] = outside;
+        part[t][2] = lng;
+    });
+    W.flops = 0;
+    double outside = 0, lng = 0;
+    for (const auto &v : part) {
+        W.flops += v[0];
+        outside += v[1];
+        lng += v[2];
+    }
+    // Two CTAs per SM hold the larger panels; three, with a larger L1, suit
+    // long columns, which are taken one at a time there (200x200x4 mesh: 74
+    // ms against 87 ms with panels in scratches), and wide columns, which
+    // wait most (256 sets of the bordered 141x141 grid: 354 ms against 384 ms)
+    const bool three = lng > 0.5 * outside || W.pull_cols > 0;
+    W.smem = three ? kRefSmemThree : kRefSmemTwo;
+    build_panels(S, panel_ctas, !three, W);
+    W.tb_nux.resize(W.tb_m);
+    for (int32_t c = 0; c < W.tb_m; c++) {
+        const int32_t *r = S.LUi.data() + S.LUp[W.tb_p + c];
+        W.tb_nux[c] = (int32_t)(std::lower_bound(r, r + S.nU[W.tb_p + c], W.tb_p) - r);
+    }
+    // pan_end[k] = panel of which k is the last column, in_pan[k]: k is in one
+    std::vector<int32_t> pan_end(n, -1);
+    std::vector<int32_t> in_pan(n, -1);
+    for (size_t p = 0; p < W.pan.size(); p++) {
+        const PanelDesc &d = W.pan[p];
+        for (int c = 0; c < d.nc; c++) in_pan[d.k0 + c] = (int32_t)p;
+        pan_end[d.k0 + d.nc - 1] = (int32_t)p;
+    }
     const double thr = alpha * (double)resident_warps;
     W.thr = thr;
+    bool all_short = !W.pan.empty() && W.dense_m == 0;
+    for (int32_t k = 0; k < n && all_short; k++) all_short = S.LUp[k + 1] - S.LUp[k] <= cap_short;
     // ---- EGraph levels, the dividing level (Section IV-B) and the tasks:
     // on a thread of their own, beside the slot maps and row-wise copies
     // below (they write disjoint members of W) ----
@@ -638,17 +916,20 @@ void build_schedule(const Pattern &P, const Structure &S, double alpha,
         // short ones in groups of up to 8.  A pending item is only merged with
         // the column that immediately follows it, so a task never comes before
         // a task holding one of its dependencies.  Groups stay inside a level
-        // before the dividing level.
-        W.task_ptr.assign(1, 0);
-        W.task_cols.clear();
-        W.task_cols.reserve(n);
-        W.level_task_ptr.assign(1, 0);
-        {
+        // before the dividing level.  A panel is a task of its own at the place
+        // of its last column: its columns' levels ascend, and a column that
+        // depends on any of them depends on the last.
+        auto tasks = [&](bool panels, std::vector<int32_t> &task_ptr, std::vector<int32_t> &task_cols,
+                         std::vector<int32_t> &level_task_ptr) {
+            task_ptr.assign(1, 0);
+            task_cols.clear();
+            task_cols.reserve(n);
+            level_task_ptr.assign(1, 0);
             const int64_t half = kRefCapLong / 2;   // medium: up to half the CTA's entries
             int32_t group = 0;      // short columns pending
             bool pend_med = false;  // one medium column pending
             auto close = [&]() {
-                if (group || pend_med) W.task_ptr.push_back((int32_t)W.task_cols.size());
+                if (group || pend_med) task_ptr.push_back((int32_t)task_cols.size());
                 group = 0;
                 pend_med = false;
             };
@@ -656,60 +937,67 @@ void build_schedule(const Pattern &P, const Structure &S, double alpha,
                 for (int32_t p = W.level_ptr[l]; p < W.level_ptr[l + 1]; p++) {
                     const int32_t k = W.level_cols[p];
                     const int64_t len = S.LUp[k + 1] - S.LUp[k];
-                    if (len > half || W.pull_start[k] > 0) {   // a whole CTA
+                    if (panels && in_pan[k] >= 0) {
+                        if (pan_end[k] < 0) continue;
                         close();
-                        W.task_cols.push_back(k);
-                        W.task_ptr.push_back((int32_t)W.task_cols.size());
+                        task_cols.push_back(W.pan[pan_end[k]].k0);
+                        task_ptr.push_back((int32_t)task_cols.size());
+                    } else if (len > half || W.pull_start[k] > 0) {   // a whole CTA
+                        close();
+                        task_cols.push_back(k);
+                        task_ptr.push_back((int32_t)task_cols.size());
                     } else if (len > cap_short) {
                         if (pend_med) {
-                            W.task_cols.push_back(k);
-                            W.task_ptr.push_back((int32_t)W.task_cols.size());
+                            task_cols.push_back(k);
+                            task_ptr.push_back((int32_t)task_cols.size());
                             pend_med = false;
                         } else {
                             close();
-                            W.task_cols.push_back(k);
+                            task_cols.push_back(k);
                             pend_med = true;
                         }
                     } else {
                         if (pend_med) close();
-                        W.task_cols.push_back(k);
+                        task_cols.push_back(k);
                         if (++group == 8) close();
                     }
                 }
                 if (l < W.div_level) {
                     close();
-                    W.level_task_ptr.push_back((int32_t)W.task_ptr.size() - 1);
+                    level_task_ptr.push_back((int32_t)task_ptr.size() - 1);
                 }
             }
             close();
-        }
+        };
+        tasks(true, W.task_ptr, W.task_cols, W.level_task_ptr);
+        W.ctask_ptr.clear();
+        W.ctask_cols.clear();
+        W.clevel_task_ptr.clear();
+        if (all_short) tasks(false, W.ctask_ptr, W.ctask_cols, W.clevel_task_ptr);
     });
-    // ---- flops of one refactorization (partial sums of integers, exact in
-    // any order below 2^53) ----
-    double part[kHostThreads] = {};
-    parallel_ranges(n, S.LUp.data(), [&](int32_t k0, int32_t k1, int t) {
-        double fl = 0;
-        for (int32_t k = k0; k < k1; k++)
-            for (int64_t e = S.LUp[k]; e < S.LUp[k] + S.nU[k] - 1; e++) {
-                const int32_t j = S.LUi[e];
-                fl += 2.0 * (double)(S.LUp[j + 1] - S.LUp[j] - S.nU[j]);
-            }
-        part[t] = fl;
-    });
-    W.flops = 0;
-    for (double v : part) W.flops += v;
     // ---- A slot -> position in its column (columns are sorted) ----
     const int64_t nnzA = (int64_t)P.Ai.size();
     W.amap.assign(nnzA, -1);
+    W.camap.assign(all_short ? nnzA : 0, -1);
     parallel_chunks(n, 2048, [&](int32_t c0, int32_t c1, int) {
         for (int32_t c = c0; c < c1; c++) {
             const int32_t k = P.qinv[c];
             const int32_t *col = S.LUi.data() + S.LUp[k];
             const int32_t len = (int32_t)(S.LUp[k + 1] - S.LUp[k]);
+            const PanelDesc *d = in_pan[k] >= 0 ? &W.pan[in_pan[k]] : nullptr;
             for (int32_t p = P.Ap[c]; p < P.Ap[c + 1]; p++) {
                 const int32_t s = S.pinv[P.Ai[p]];
                 const int32_t *it = std::lower_bound(col, col + len, s);
-                W.amap[p] = (it != col + len && *it == s) ? (int32_t)(it - col) : -1;
+                int32_t at = (it != col + len && *it == s) ? (int32_t)(it - col) : -1;
+                if (all_short) W.camap[p] = at;
+                if (d && at >= 0) {   // the slot in the panel
+                    const int32_t *u = W.prow.data() + d->uoff;
+                    if (s < d->k0) at = (int32_t)(std::lower_bound(u, u + d->nu, s) - u);
+                    else if (s < d->k0 + d->nc) at = d->nu + (s - d->k0);
+                    // L rows: the first d->k0 + d->nc - 1 - k of the column are in the diagonal block
+                    else at = d->nu + d->nc + (at - S.nU[k] - (d->k0 + d->nc - 1 - k));
+                }
+                W.amap[p] = at;
             }
         }
     });
