@@ -87,7 +87,7 @@ struct alignas(8) PanelRun {
     int32_t t, wm, nR, j0;
     int64_t lbl;
 };
-constexpr int kPanelRun = 16, kPanelRunBig = 16;   // (panels in a scratch)
+constexpr int kPanelRun = 16;
 constexpr int kPanelWideRows = 256;   // most L rows below a panel of more than four columns
 constexpr int kPanelMax = 8;
 // columns of more entries count as long (Schedule::smem)

@@ -550,11 +550,14 @@ static void build_panels(const Structure &S, int panel_ctas, bool allow_scratch,
     W.pan_id.assign(n, -1);
     W.pscratch = 0;
     if (W.dense_m > 0 || n == 0) return;
-    // link[j]: columns j and j+1 may share a panel
-    auto link = [&](int32_t j) {
-        return j + 1 != W.tb_p && W.chain[j] && !W.pull_start[j] && !W.pull_start[j + 1] && S.nU[j + 1] >= 2 &&
+    // link[j]: columns j and j+1 may share a panel; long chains are cut every
+    // 64 columns, the units that the host threads share
+    std::vector<uint8_t> link(n, 0);
+    for (int32_t j = 0, run = 1; j + 1 < n; j++) {
+        link[j] = j + 1 != W.tb_p && run < 64 && W.chain[j] && !W.pull_start[j] && !W.pull_start[j + 1] && S.nU[j + 1] >= 2 &&
                S.LUi[S.LUp[j + 1] + S.nU[j + 1] - 2] == j;
-    };
+        run = link[j] ? run + 1 : 1;
+    }
     const int64_t smem = W.smem;
     auto fits = [smem](int64_t slots, int nc) {
         return slots * (8 * panel_ld(nc) + 4) <= smem - kPanelRing;
@@ -563,6 +566,7 @@ static void build_panels(const Structure &S, int panel_ctas, bool allow_scratch,
         std::vector<PanelDesc> pan;
         std::vector<int32_t> prow, ppref;
         std::vector<uint8_t> pmask;
+        std::vector<PanelRun> prun;
         int64_t scratch = 0;
     };
     // small structures stay on this thread
@@ -570,79 +574,89 @@ static void build_panels(const Structure &S, int panel_ctas, bool allow_scratch,
         if (S.nnz() < (1 << 19)) fn(0, m, 0);
         else parallel_chunks(m, chunk, fn);
     };
-    const int32_t chunk = 1024, nparts = (n + chunk - 1) / chunk;
+    const int32_t chunk = 128, nparts = (n + chunk - 1) / chunk;
     std::vector<Part> parts(nparts);
+    std::vector<uint8_t> first(n, 0);   // column k begins a panel
     in_chunks(n, chunk, [&](int32_t c0, int32_t c1, int) {
+        std::vector<uint64_t> u, v;   // union rows: row << 8 | mask of the columns that have it
+        // the union of the U rows above k of columns k .. k+nc-1; its size
+        auto join = [&](int32_t k, int nc) -> int64_t {
+            int64_t most = 0, nu = 0;
+            for (int c = 0; c < nc; c++) most += S.nU[k + c];
+            if ((int64_t)u.size() < most) { u.resize(most); v.resize(most); }
+            for (int c = 0; c < nc; c++) {
+                const int32_t *r = S.LUi.data() + S.LUp[k + c];
+                const int32_t *re = std::lower_bound(r, r + S.nU[k + c], k);
+                const uint64_t bit = (uint64_t)1 << c, *p = u.data(), *pe = p + nu;
+                uint64_t *o = v.data();
+                while (p < pe && r < re) {
+                    const int32_t a = (int32_t)(*p >> 8), b = *r;
+                    *o++ = a <= b ? (*p | (a == b ? bit : 0)) : (((uint64_t)b << 8) | bit);
+                    p += a <= b;
+                    r += b <= a;
+                }
+                while (p < pe) *o++ = *p++;
+                while (r < re) *o++ = ((uint64_t)*r++ << 8) | bit;
+                nu = o - v.data();
+                u.swap(v);
+            }
+            return nu;
+        };
         // one call has every part when it runs serially
         for (int32_t b = c0; b < c1; b += chunk) {
             Part &pt = parts[b / chunk];
-            std::vector<std::pair<int32_t, uint8_t>> u, v, m;
-            // the union of the U rows above k of columns k .. k+nc-1
-            auto join = [&](int32_t k, int nc) {
-                u.clear();
-                for (int c = 0; c < nc; c++) {
-                    const int32_t *r = S.LUi.data() + S.LUp[k + c];
-                    const int32_t cnt = (int32_t)(std::lower_bound(r, r + S.nU[k + c], k) - r);
-                    const uint8_t bit = (uint8_t)(1u << c);
-                    v.clear();
-                    size_t i = 0;
-                    int32_t q = 0;
-                    while (i < u.size() || q < cnt) {
-                        if (q == cnt || (i < u.size() && u[i].first < r[q])) v.push_back(u[i++]);
-                        else if (i == u.size() || r[q] < u[i].first) v.push_back({r[q++], bit});
-                        else { v.push_back({u[i].first, (uint8_t)(u[i].second | bit)}); i++; q++; }
-                    }
-                    u.swap(v);
-                }
-            };
             const int32_t e = std::min(b + chunk, n);
             int32_t k = b;
-            while (k < e && k > 0 && link(k - 1)) k++;   // a chain that began in an earlier part
+            while (k < e && k > 0 && link[k - 1]) k++;   // a chain that began in an earlier part
             while (k < e) {
                 int32_t end = k + 1;
-                while (end < n && link(end - 1)) end++;
-                for (; k < end;) {
+                while (end < n && link[end - 1]) end++;
+                while (k < end) {
                     const int32_t left = end - k;
                     if (left == 1) { k++; break; }   // a column of its own
                     int nc = std::min<int32_t>(left, kPanelMax);
                     auto l_rows = [&](int c) { return S.LUp[k + c + 1] - S.LUp[k + c] - S.nU[k + c]; };
-                    auto most = [&](int c) {   // the union has at least this many slots
+                    auto least = [&](int c) {   // the union has at least this many slots
                         int64_t mx = 0;
                         for (int i = 0; i < c; i++) mx = std::max(mx, (int64_t)S.nU[k + i] - 1 - i);
                         return mx + c + l_rows(c - 1);
                     };
-                    int64_t slots = 0;
+                    int64_t nu = 0, slots = 0;
                     if (nc > 4) {
-                        bool ok = l_rows(nc - 1) <= kPanelWideRows && fits(most(nc), nc);
+                        bool ok = l_rows(nc - 1) <= kPanelWideRows && fits(least(nc), nc);
                         if (ok) {
-                            join(k, nc);
-                            slots = (int64_t)u.size() + nc + l_rows(nc - 1);
+                            nu = join(k, nc);
+                            slots = nu + nc + l_rows(nc - 1);
                             ok = fits(slots, nc);
                         }
                         if (!ok) nc = 4;
                     }
                     if (nc <= 4) {
-                        join(k, nc);
-                        slots = (int64_t)u.size() + nc + l_rows(nc - 1);
+                        if (!allow_scratch && !fits(least(nc), nc)) { k++; continue; }
+                        nu = join(k, nc);
+                        slots = nu + nc + l_rows(nc - 1);
                         if (!fits(slots, nc) && !allow_scratch) { k++; continue; }
                     }
                     const int64_t need = slots * (8 * panel_ld(nc) + 4);
                     if (!fits(slots, nc)) pt.scratch = std::max(pt.scratch, (need + 255) / 256 * 256);
-                    PanelDesc d;
+                    PanelDesc d{};
                     d.k0 = k;
                     d.nc = nc;
-                    d.nu = (int32_t)u.size();
+                    d.nu = (int32_t)nu;
                     d.uoff = (int64_t)pt.prow.size();
                     d.poff = (int64_t)pt.ppref.size();
-                    d.roff = 0;
-                    d.nruns = 0;
+                    pt.prow.resize(d.uoff + nu + nc);
+                    pt.pmask.resize(d.uoff + nu + nc);
+                    pt.ppref.resize(d.poff + (nu + 31) / 32 * nc);
+                    int32_t *row = pt.prow.data() + d.uoff, *pref = pt.ppref.data() + d.poff;
+                    uint8_t *msk = pt.pmask.data() + d.uoff;
                     int32_t cnt[kPanelMax] = {};
-                    for (int32_t s = 0; s < d.nu; s++) {
+                    for (int64_t s = 0; s < nu; s++) {
                         if (s % 32 == 0)
-                            for (int c = 0; c < nc; c++) pt.ppref.push_back(cnt[c]);
-                        pt.prow.push_back(u[s].first);
-                        pt.pmask.push_back(u[s].second);
-                        for (int c = 0; c < nc; c++) cnt[c] += (u[s].second >> c) & 1;
+                            for (int c = 0; c < nc; c++) *pref++ = cnt[c];
+                        row[s] = (int32_t)(u[s] >> 8);
+                        msk[s] = (uint8_t)u[s];
+                        for (int c = 0; c < nc; c++) cnt[c] += (int32_t)(u[s] >> c) & 1;
                     }
                     for (int q = 0; q < nc; q++) {   // diagonal-block rows
                         unsigned mk = 0;
@@ -650,9 +664,10 @@ static void build_panels(const Structure &S, int panel_ctas, bool allow_scratch,
                             const int32_t *r = S.LUi.data() + S.LUp[k + c];
                             if (q >= c || std::binary_search(r, r + S.nU[k + c], k + q)) mk |= 1u << c;
                         }
-                        pt.prow.push_back(k + q);
-                        pt.pmask.push_back((uint8_t)mk);
+                        row[nu + q] = k + q;
+                        msk[nu + q] = (uint8_t)mk;
                     }
+                    first[k] = 1;
                     pt.pan.push_back(d);
                     k += nc;
                 }
@@ -660,7 +675,7 @@ static void build_panels(const Structure &S, int panel_ctas, bool allow_scratch,
             }
         }
     });
-    std::vector<int64_t> op(nparts + 1, 0), ou(nparts + 1, 0), of(nparts + 1, 0);
+    std::vector<int64_t> op(nparts + 1, 0), ou(nparts + 1, 0), of(nparts + 1, 0), orr(nparts + 1, 0);
     for (int32_t i = 0; i < nparts; i++) {
         op[i + 1] = op[i] + (int64_t)parts[i].pan.size();
         ou[i + 1] = ou[i] + (int64_t)parts[i].prow.size();
@@ -668,76 +683,64 @@ static void build_panels(const Structure &S, int panel_ctas, bool allow_scratch,
         W.pscratch = std::max(W.pscratch, parts[i].scratch);
     }
     if (W.pscratch > 0 && (size_t)W.pscratch * (size_t)panel_ctas > kPanelScratchBytes && allow_scratch) {
-        // long columns one at a time
-        build_panels(S, panel_ctas, false, W);
+        build_panels(S, panel_ctas, false, W);   // long columns one at a time
         return;
     }
     W.pan.resize(op[nparts]);
     W.prow.resize(ou[nparts]);
     W.pmask.resize(ou[nparts]);
     W.ppref.resize(of[nparts]);
-    in_chunks(nparts, 1, [&](int32_t i0, int32_t i1, int) {
+    // The arrays of the parts in one, and the runs: up to kPanelRun linked
+    // dependencies; the last kPanelRun dependencies, which may still be in
+    // progress when the panel meets them, are cut where a panel of theirs
+    // begins, so that a run waits for no more columns than it needs
+    in_chunks(nparts, 4, [&](int32_t i0, int32_t i1, int) {
         for (int32_t i = i0; i < i1; i++) {
             Part &pt = parts[i];
             std::copy(pt.prow.begin(), pt.prow.end(), W.prow.begin() + ou[i]);
             std::copy(pt.pmask.begin(), pt.pmask.end(), W.pmask.begin() + ou[i]);
             std::copy(pt.ppref.begin(), pt.ppref.end(), W.ppref.begin() + of[i]);
-            for (size_t q = 0; q < pt.pan.size(); q++) {
-                PanelDesc d = pt.pan[q];
+            for (size_t p = 0; p < pt.pan.size(); p++) {
+                PanelDesc &d = W.pan[op[i] + (int64_t)p];
+                d = pt.pan[p];
+                const int32_t *u = pt.prow.data() + d.uoff;
+                const uint8_t *m = pt.pmask.data() + d.uoff;
+                const int64_t r0 = (int64_t)pt.prun.size();
+                for (int32_t s = 0; s < d.nu;) {
+                    int w = 1;
+                    unsigned mk = m[s];
+                    while (w < kPanelRun && s + w < d.nu && u[s + w] == u[s + w - 1] + 1 && W.chain[u[s + w - 1]] &&
+                           u[s + w] != W.tb_p && !(d.nu - (s + w) <= kPanelRun && first[u[s + w]])) {
+                        mk |= m[s + w];
+                        w++;
+                    }
+                    const int32_t jl = u[s + w - 1];
+                    PanelRun r;
+                    r.t = s;
+                    r.wm = (int32_t)(w | (mk << 8));
+                    r.lbl = S.LUp[jl] + S.nU[jl];
+                    r.nR = (int32_t)(S.LUp[jl + 1] - r.lbl);
+                    r.j0 = u[s];
+                    pt.prun.push_back(r);
+                    s += w;
+                }
+                d.nruns = (int32_t)((int64_t)pt.prun.size() - r0);
+                d.nux = (int32_t)(std::lower_bound(u, u + d.nu, W.tb_p) - u);
+                d.nrunsx = 0;
+                while (d.nrunsx < d.nruns && pt.prun[r0 + d.nrunsx].t < d.nux) d.nrunsx++;
+                d.roff = r0;
                 d.uoff += ou[i];
                 d.poff += of[i];
-                W.pan[op[i] + (int64_t)q] = d;
-                W.pan_id[d.k0] = (int32_t)(op[i] + (int64_t)q);
+                W.pan_id[d.k0] = (int32_t)(op[i] + (int64_t)p);
             }
-            pt = Part();
         }
     });
-    // runs of up to kPanelRun linked dependencies; the last kPanelRun
-    // dependencies, which may still be in progress when the panel meets
-    // them, are cut where a panel of theirs begins, so that a run waits for
-    // no more columns than it needs
-    const int32_t npan = (int32_t)W.pan.size(), pchunk = 64, nrp = (npan + pchunk - 1) / pchunk;
-    std::vector<std::vector<PanelRun>> runs(nrp);
-    in_chunks(npan, pchunk, [&](int32_t p0, int32_t p1, int) {
-        for (int32_t p = p0; p < p1; p++) {
-            std::vector<PanelRun> &out = runs[p / pchunk];
-            PanelDesc &d = W.pan[p];
-            const int32_t *u = W.prow.data() + d.uoff;
-            const uint8_t *m = W.pmask.data() + d.uoff;
-            d.roff = (int64_t)out.size();
-            const int32_t kl = d.k0 + d.nc - 1;
-            const int most = fits(d.nu + d.nc + S.LUp[kl + 1] - S.LUp[kl] - S.nU[kl], d.nc) ? kPanelRun : kPanelRunBig;
-            for (int32_t s = 0; s < d.nu;) {
-                int w = 1;
-                unsigned mk = m[s];
-                while (w < most && s + w < d.nu && u[s + w] == u[s + w - 1] + 1 && W.chain[u[s + w - 1]] &&
-                       u[s + w] != W.tb_p && !(d.nu - (s + w) <= kPanelRun && W.pan_id[u[s + w]] >= 0)) {
-                    mk |= m[s + w];
-                    w++;
-                }
-                const int32_t jl = u[s + w - 1];
-                PanelRun r;
-                r.t = s;
-                r.wm = (int32_t)(w | (mk << 8));
-                r.lbl = S.LUp[jl] + S.nU[jl];
-                r.nR = (int32_t)(S.LUp[jl + 1] - r.lbl);
-                r.j0 = u[s];
-                out.push_back(r);
-                s += w;
-            }
-            d.nruns = (int32_t)((int64_t)out.size() - d.roff);
-            d.nux = (int32_t)(std::lower_bound(u, u + d.nu, W.tb_p) - u);
-            d.nrunsx = 0;
-            while (d.nrunsx < d.nruns && out[d.roff + d.nrunsx].t < d.nux) d.nrunsx++;
-        }
-    });
-    std::vector<int64_t> orr(nrp + 1, 0);
-    for (int32_t i = 0; i < nrp; i++) orr[i + 1] = orr[i] + (int64_t)runs[i].size();
-    W.prun.resize(orr[nrp]);
-    in_chunks(nrp, 1, [&](int32_t i0, int32_t i1, int) {
+    for (int32_t i = 0; i < nparts; i++) orr[i + 1] = orr[i] + (int64_t)parts[i].prun.size();
+    W.prun.resize(orr[nparts]);
+    in_chunks(nparts, 4, [&](int32_t i0, int32_t i1, int) {
         for (int32_t i = i0; i < i1; i++) {
-            std::copy(runs[i].begin(), runs[i].end(), W.prun.begin() + orr[i]);
-            for (int32_t p = i * pchunk; p < std::min((i + 1) * pchunk, npan); p++) W.pan[p].roff += orr[i];
+            std::copy(parts[i].prun.begin(), parts[i].prun.end(), W.prun.begin() + orr[i]);
+            for (int64_t p = op[i]; p < op[i + 1]; p++) W.pan[p].roff += orr[i];
         }
     });
 }
