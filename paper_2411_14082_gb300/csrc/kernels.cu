@@ -493,26 +493,37 @@ __global__ void begin_solve_kernel(DevCtl *ctl, double *y, double *z, double *el
     }
 }
 
-// value of v[j] once it is published; false if the wait gave up
-__device__ __forceinline__ bool await_value(const double *v, int j, const SolveArgs &a, int site,
-                                            int row, double &out)
+// Waits until every lane's value is published: lane's value is v[j], b the
+// bits it last saw there (wanted lanes only; the warp is converged).  The
+// lanes whose value is missing poll together.  Returns false if the wait
+// gave up.
+__device__ __forceinline__ bool await_warp(const double *v, int j, bool want, unsigned long long &b, const SolveArgs &a,
+                                           int site, int row)
 {
-    unsigned long long b = ld_relaxed_u64(v + j);
-    long long it = 0;
-    while (b == kSentinel) {
+    for (long long it = 0; __any_sync(kFull, want && b == kSentinel);) {
         // the shared status word is read only every 64 polls: thousands of
-        // waiting lanes polling one address would queue on its L2 slice
-        if (++it > a.spin_limit || ((it & 63) == 0 && ld_volatile(&a.ctl->status))) {
+        // waiting warps polling one address would queue on its L2 slice
+        if (++it > a.spin_limit || ((it & 63) == 0 && __any_sync(kFull, ld_volatile(&a.ctl->status)))) {
             set_status(a.ctl, GBLU_ERR_DEVICE_TIMEOUT);
             a.ctl->where = site;
             a.ctl->where_k = row;
             return false;
         }
         __nanosleep(32);
-        b = ld_relaxed_u64(v + j);
+        if (want && b == kSentinel) b = ld_relaxed_u64(v + j);
     }
-    out = __longlong_as_double((long long)b);
     return true;
+}
+
+// value of v[j] once it is published, for every lane that wants one; false
+// if the wait gave up
+__device__ __forceinline__ bool await_value(const double *v, int j, bool want, const SolveArgs &a, int site, int row,
+                                            double &out)
+{
+    unsigned long long b = want ? ld_relaxed_u64(v + j) : 0ull;
+    const bool ok = await_warp(v, j, want, b, a, site, row);
+    out = want ? __longlong_as_double((long long)b) : 0.0;
+    return ok;
 }
 
 // ---------------------------------------------------------------------------
@@ -530,90 +541,48 @@ __device__ __forceinline__ bool await_value(const double *v, int j, const SolveA
 // launch give identical bits.
 constexpr int kBR = kSolveBlockRows;
 
-// forward: sum over the entries of row i outside its block (all but its last q)
-// v[j] for four columns at once: one relaxed load each in flight, then a
-// bounded wait on those still holding the sentinel
-__device__ __forceinline__ bool fetch4(const double *v, const int (&j)[4], bool wait, const SolveArgs &a, int site,
-                                       int row, double (&out)[4])
+// sum over CSR entries of one row: entry t of n (t = 0 .. n-1, in the order
+// in which their values are produced) is at e0 + dir * t; lane takes t =
+// lane, lane + 32, ..., four in flight, applied in ascending t
+__device__ __forceinline__ bool row_ext(const double *LUx, const int32_t *col, const int32_t *slot, const double *vec,
+                                        int64_t e0, int dir, int n, int lane, bool wait, const SolveArgs &a, int site,
+                                        int i, double &s)
 {
-    if (!wait) {
+    double acc = 0.0;
+    for (int t0 = 0; t0 < n; t0 += 128) {
+        int j[4];
+        double lv[4];
+        unsigned long long b[4];
+        bool in[4];
 #pragma unroll
-        for (int u = 0; u < 4; u++) out[u] = __ldcg(v + j[u]);
-        return true;
+        for (int u = 0; u < 4; u++) {
+            const int t = t0 + 32 * u + lane;
+            in[u] = t < n;
+            j[u] = in[u] ? __ldg(col + e0 + dir * t) : 0;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; u++) lv[u] = in[u] ? __ldg(LUx + __ldg(slot + e0 + dir * (t0 + 32 * u + lane))) : 0.0;
+#pragma unroll
+        for (int u = 0; u < 4; u++) b[u] = in[u] ? (wait ? ld_relaxed_u64(vec + j[u]) : (unsigned long long)__double_as_longlong(__ldcg(vec + j[u]))) : 0ull;
+        if (wait) {
+#pragma unroll
+            for (int u = 3; u >= 0; u--)   // the last produced first: the others are then there
+                if (t0 + 32 * u < n && !await_warp(vec, j[u], in[u], b[u], a, site, i)) return false;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; u++)
+            if (in[u]) acc = fma(lv[u], __longlong_as_double((long long)b[u]), acc);
     }
-    unsigned long long b[4];
-#pragma unroll
-    for (int u = 0; u < 4; u++) b[u] = ld_relaxed_u64(v + j[u]);
-    bool ok = true;
-#pragma unroll
-    for (int u = 0; u < 4; u++) {
-        if (b[u] != kSentinel) out[u] = __longlong_as_double((long long)b[u]);
-        else if (ok) ok = await_value(v, j[u], a, site, row, out[u]);
-    }
-    return ok;
+    s = warp_sum(acc);
+    return true;
 }
 
+// forward: sum over the entries of row i outside its block (all but its last
+// q), ascending columns
 __device__ __forceinline__ bool lrow_ext(const SolveArgs &a, int i, int q, int lane, bool wait, double &s)
 {
     const int64_t rb = __ldg(a.Lrp + i), re = __ldg(a.Lrp + i + 1) - q;
-    double acc = 0.0;
-    bool ok = true;
-    int64_t e = rb + lane;
-    // four entries per lane in flight, applied in the same order as one by one
-    for (; e + 96 < re && ok; e += 128) {
-        int j[4];
-        double lv[4], yv[4];
-#pragma unroll
-        for (int u = 0; u < 4; u++) j[u] = __ldg(a.Lcol + e + 32 * u);
-#pragma unroll
-        for (int u = 0; u < 4; u++) lv[u] = __ldg(a.LUx + __ldg(a.Lslot + e + 32 * u));
-        ok = fetch4(a.y, j, wait, a, 3, i, yv);
-#pragma unroll
-        for (int u = 0; u < 4; u++) acc = fma(lv[u], yv[u], acc);
-    }
-    for (; e < re; e += 32) {
-        const int j = __ldg(a.Lcol + e);
-        double yj = 0.0;
-        if (!wait) yj = __ldcg(a.y + j);
-        else if (ok) ok = await_value(a.y, j, a, 3, i, yj);
-        acc = fma(__ldg(a.LUx + __ldg(a.Lslot + e)), yj, acc);
-    }
-    s = warp_sum(acc);
-    return __all_sync(kFull, ok);
-}
-
-// forward block finish: lane p < w holds e = the outside sum of row f+p
-// the block's unit lower triangle: lane p < w holds row f+p's entries
-// L(f+p, f .. f+p-1), its last p entries (loaded before the block's values
-// are awaited, off the dependency chain)
-__device__ __forceinline__ void lblock_load(const SolveArgs &a, int f, int w, int lane, double (&tv)[kBR - 1])
-{
-    const int64_t rend = lane < w ? __ldg(a.Lrp + f + lane + 1) - lane : 0;
-#pragma unroll
-    for (int d = 0; d < kBR - 1; d++)
-        tv[d] = (d < lane && lane < w) ? __ldg(a.LUx + __ldg(a.Lslot + rend + d)) : 0.0;
-}
-
-// forward block finish: lane p < w holds e = the outside sum of row f+p
-__device__ __forceinline__ void lblock_solve(const SolveArgs &a, int f, int w, int lane, double e,
-                                             const double (&tv)[kBR - 1])
-{
-    double v = lane < w ? __ldg(a.b + __ldg(a.piv + f + lane)) - e : 0.0;
-#pragma unroll
-    for (int d = 0; d < kBR - 1; d++) {
-        if (d < w - 1) {
-            const double yd = __shfl_sync(kFull, v, d);
-            if (lane > d && lane < w) v = fma(-tv[d], yd, v);
-        }
-    }
-    if (lane < w) st_relaxed_f64(a.y + f + lane, v);
-}
-
-__device__ __forceinline__ void lblock_finish(const SolveArgs &a, int f, int w, int lane, double e)
-{
-    double tv[kBR - 1];
-    lblock_load(a, f, w, lane, tv);
-    lblock_solve(a, f, w, lane, e, tv);
+    return row_ext(a.LUx, a.Lcol, a.Lslot, a.y, rb, 1, (int)(re - rb), lane, wait, a, 3, i, s);
 }
 
 // backward: sum over the entries of row i outside its block (all but its
@@ -623,70 +592,133 @@ __device__ __forceinline__ bool urow_ext(const SolveArgs &a, int i, int q, int w
 {
     // entries in the trailing block's columns were summed into far[i] already
     const int64_t rb = __ldg(a.Urp + i) + (w - 1 - q), re = a.ufar ? __ldg(a.ufar + i) : __ldg(a.Urp + i + 1);
-    double acc = 0.0;
-    bool ok = true;
-    int64_t e = re - 1 - lane;
-    // four entries per lane in flight, applied in the same order as one by one
-    for (; e - 96 >= rb && ok; e -= 128) {
-        int j[4];
-        double uv[4], zv[4];
-#pragma unroll
-        for (int u = 0; u < 4; u++) j[u] = __ldg(a.Ucol + e - 32 * u);
-#pragma unroll
-        for (int u = 0; u < 4; u++) uv[u] = __ldg(a.LUx + __ldg(a.Uslot + e - 32 * u));
-        ok = fetch4(a.z, j, wait, a, 4, i, zv);
-#pragma unroll
-        for (int u = 0; u < 4; u++) acc = fma(uv[u], zv[u], acc);
-    }
-    for (; e >= rb; e -= 32) {
-        const int j = __ldg(a.Ucol + e);
-        double zj = 0.0;
-        if (!wait) zj = __ldcg(a.z + j);
-        else if (ok) ok = await_value(a.z, j, a, 4, i, zj);
-        acc = fma(__ldg(a.LUx + __ldg(a.Uslot + e)), zj, acc);
-    }
-    s = warp_sum(acc);
+    if (!row_ext(a.LUx, a.Ucol, a.Uslot, a.z, re - 1, -1, (int)(re - rb), lane, wait, a, 4, i, s)) return false;
     if (a.ufar) s += __ldcg(a.far + i);
-    return __all_sync(kFull, ok);
+    return true;
+}
+
+// Finishing a block: the triangle goes into the warp's shared memory, and
+// the right-hand side into registers, before the block's values are awaited.
+// keep() holds a loaded value at its place: without it the compiler moves
+// loads (and the division) behind the waits, to their first use, where each
+// step of the substitution paid an L2 round trip.  The triangle is a 32 x 32
+// tile that every lane reads without a branch, and a lane that a step leaves
+// alone keeps its value by a select: a divergent step cost 430 to 600 cycles,
+// of which the arithmetic (a shuffle and a multiply-add of 64 cycles) is about
+// 100.  What bounds the solves is this chain through the blocks; one solve,
+// before and after: 2,020 unknowns 0.44 -> 0.16 ms, 110x109x4 mesh 2.1 ->
+// 1.15 ms, 150x150x4 mesh 2.85 -> 1.60 ms.
+constexpr int kTriDoubles = kBR * kBR;
+constexpr int kSolveSmem = kSolveWarpsPerBlock * kTriDoubles * (int)sizeof(double);   // 64 KB per CTA
+__device__ __forceinline__ void keep(double &v) { asm volatile("" : "+d"(v)); }
+
+// the block's unit lower triangle: lane p < w holds row f+p's entries
+// L(f+p, f .. f+p-1), its last p entries, at tri[d * 32 + p], d < p; returns
+// the rows' right-hand side
+__device__ __forceinline__ double lblock_load(const SolveArgs &a, int f, int w, int lane, double *tri)
+{
+    double rhs = lane < w ? __ldg(a.b + __ldg(a.piv + f + lane)) : 0.0;
+    const int64_t rend = lane < w ? __ldg(a.Lrp + f + lane + 1) - lane : 0;
+    for (int d0 = 0; d0 < w - 1; d0 += 8) {   // eight entries in flight
+        double v[8];
+#pragma unroll
+        for (int u = 0; u < 8; u++)
+            v[u] = (d0 + u < lane && lane < w) ? __ldg(a.LUx + __ldg(a.Lslot + rend + d0 + u)) : 0.0;
+#pragma unroll
+        for (int u = 0; u < 8; u++) tri[(d0 + u) * kBR + lane] = v[u];
+    }
+    keep(rhs);
+    __syncwarp();
+    return rhs;
+}
+
+// forward block finish: lane p < w holds e = the outside sum of row f+p
+__device__ __forceinline__ void lblock_solve(const SolveArgs &a, int f, int w, int lane, double rhs, double e,
+                                             const double *tri)
+{
+    double v = lane < w ? rhs - e : 0.0;
+    for (int d0 = 0; d0 < w - 1; d0 += 8) {
+        double l[8];
+#pragma unroll
+        for (int u = 0; u < 8; u++) l[u] = tri[(d0 + u) * kBR + lane];
+#pragma unroll
+        for (int u = 0; u < 8; u++) {   // (steps past w - 1 have zeros)
+            const double nv = fma(-l[u], __shfl_sync(kFull, v, d0 + u), v);
+            v = lane > d0 + u && d0 + u < w - 1 ? nv : v;
+        }
+    }
+    if (lane < w) st_relaxed_f64(a.y + f + lane, v);
+    __syncwarp();   // the triangle is read: the warp's next block may overwrite it
+}
+
+__device__ __forceinline__ void lblock_finish(const SolveArgs &a, int f, int w, int lane, double e, double *tri)
+{
+    const double rhs = lblock_load(a, f, w, lane, tri);
+    lblock_solve(a, f, w, lane, rhs, e, tri);
 }
 
 // the block's upper triangle: lane p < w holds row f+p's entries
-// U(f+p, f+p+1 .. f+w-1) (its first w-1-p entries) and the reciprocal of
-// its diagonal, computed by every lane at once (a division per step of the
-// substitution would sit on the dependency chain)
-__device__ __forceinline__ void ublock_load(const SolveArgs &a, int f, int w, int lane, double (&tu)[kBR], double &rd)
+// U(f+p, f+p+1 .. f+w-1) (its first w-1-p entries) at tri[d * 32 + p], d > p;
+// the reciprocal of its diagonal, computed by every lane at once (a division per step of the substitution would sit on
+// the dependency chain); and the rows' right-hand side (final: the forward
+// solve's)
+__device__ __forceinline__ double ublock_load(const SolveArgs &a, int f, int w, int lane, double *tri, double &rd, int &q)
 {
-    const int64_t rbeg = lane < w ? __ldg(a.Urp + f + lane) - lane - 1 : 0;
-#pragma unroll
-    for (int d = 0; d < kBR; d++)
-        tu[d] = (lane < d && d < w) ? __ldg(a.LUx + __ldg(a.Uslot + rbeg + d)) : 0.0;
+    q = lane < w ? __ldg(a.Q + f + lane) : 0;
+    double rhs = lane < w ? __ldcg(a.y + f + lane) : 0.0;
     rd = lane < w ? 1.0 / __ldg(a.LUx + __ldg(a.Udiag + f + lane)) : 1.0;
+    const int64_t rbeg = lane < w ? __ldg(a.Urp + f + lane) - lane - 1 : 0;
+    for (int d0 = 0; d0 < w; d0 += 8) {   // eight entries in flight
+        double v[8];
+#pragma unroll
+        for (int u = 0; u < 8; u++)
+            v[u] = (lane < d0 + u && d0 + u < w) ? __ldg(a.LUx + __ldg(a.Uslot + rbeg + d0 + u)) : 0.0;
+#pragma unroll
+        for (int u = 0; u < 8; u++) tri[(d0 + u) * kBR + lane] = v[u];
+    }
+    keep(rhs);
+    keep(rd);
+    asm volatile("" : "+r"(q));
+    __syncwarp();
+    return rhs;
 }
 
 // backward block finish: lane p < w holds e = the outside sum of row f+p
-__device__ __forceinline__ void ublock_solve(const SolveArgs &a, int f, int w, int lane, double e,
-                                             const double (&tu)[kBR], double rd)
+__device__ __forceinline__ void ublock_solve(const SolveArgs &a, int f, int w, int lane, double rhs, double e,
+                                             const double *tri, double rd, int q)
 {
-    double v = lane < w ? __ldcg(a.y + f + lane) - e : 0.0, zl = 0.0;
+    double v = lane < w ? rhs - e : 0.0, zl = 0.0;
+    for (int d0 = (w - 1) & ~7; d0 >= 0; d0 -= 8) {
+        double t[8], r[8];
 #pragma unroll
-    for (int d = kBR - 1; d >= 0; d--) {
-        if (d < w) {
-            const double zd = __shfl_sync(kFull, v, d) * __shfl_sync(kFull, rd, d);
-            if (lane == d) zl = zd;
-            if (lane < d) v = fma(-tu[d], zd, v);
+        for (int u = 0; u < 8; u++) {
+            t[u] = tri[(d0 + u) * kBR + lane];
+            r[u] = __shfl_sync(kFull, rd, d0 + u);
+        }
+#pragma unroll
+        for (int u = 7; u >= 0; u--) {
+            const int d = d0 + u;
+            if (d < w) {
+                const double zd = __shfl_sync(kFull, v, d) * r[u];
+                const double nv = fma(-t[u], zd, v);
+                zl = lane == d ? zd : zl;
+                v = lane < d ? nv : v;
+            }
         }
     }
     if (lane < w) {
         st_relaxed_f64(a.z + f + lane, zl);
-        a.x[__ldg(a.Q + f + lane)] = zl;
+        a.x[q] = zl;
     }
+    __syncwarp();   // the triangle is read: the warp's next block may overwrite it
 }
 
-__device__ __forceinline__ void ublock_finish(const SolveArgs &a, int f, int w, int lane, double e)
+__device__ __forceinline__ void ublock_finish(const SolveArgs &a, int f, int w, int lane, double e, double *tri)
 {
-    double tu[kBR], rd;
-    ublock_load(a, f, w, lane, tu, rd);
-    ublock_solve(a, f, w, lane, e, tu, rd);
+    double rd;
+    int q;
+    const double rhs = ublock_load(a, f, w, lane, tri, rd, q);
+    ublock_solve(a, f, w, lane, rhs, e, tri, rd, q);
 }
 
 // Batches (gblu_solve_batch): the same kernels over nsets right-hand sides
@@ -707,7 +739,7 @@ __device__ __forceinline__ SolveArgs set_view(const SolveArgs &a, int s)
 
 // level mode, first launch of a level: every row of the level stores its
 // outside sum (its inputs are final: earlier launches)
-__device__ __forceinline__ void lsolve_level_row(const SolveArgs &a, int t, int lane)
+__device__ __forceinline__ void lsolve_level_row(const SolveArgs &a, int t, int lane, double *)
 {
     const int i = __ldg(a.rows + t), b = __ldg(a.rb + i);
     double s;
@@ -715,7 +747,7 @@ __device__ __forceinline__ void lsolve_level_row(const SolveArgs &a, int t, int 
     if (lane == 0) a.ext[i] = s;
 }
 
-__device__ __forceinline__ void usolve_level_row(const SolveArgs &a, int t, int lane)
+__device__ __forceinline__ void usolve_level_row(const SolveArgs &a, int t, int lane, double *)
 {
     const int i = __ldg(a.rows + t), b = __ldg(a.rb + i);
     const int f = __ldg(a.bs + b), w = __ldg(a.bs + b + 1) - f;
@@ -725,38 +757,41 @@ __device__ __forceinline__ void usolve_level_row(const SolveArgs &a, int t, int 
 }
 
 // level mode, second launch of a level: one warp per block (a.rows = block ids)
-__device__ __forceinline__ void lsolve_finish_block(const SolveArgs &a, int t, int lane)
+__device__ __forceinline__ void lsolve_finish_block(const SolveArgs &a, int t, int lane, double *tri)
 {
     const int b = __ldg(a.rows + t), f = __ldg(a.bs + b), w = __ldg(a.bs + b + 1) - f;
-    lblock_finish(a, f, w, lane, lane < w ? __ldcg(a.ext + f + lane) : 0.0);
+    lblock_finish(a, f, w, lane, lane < w ? __ldcg(a.ext + f + lane) : 0.0, tri);
 }
 
-__device__ __forceinline__ void usolve_finish_block(const SolveArgs &a, int t, int lane)
+__device__ __forceinline__ void usolve_finish_block(const SolveArgs &a, int t, int lane, double *tri)
 {
     const int b = __ldg(a.rows + t), f = __ldg(a.bs + b), w = __ldg(a.bs + b + 1) - f;
-    ublock_finish(a, f, w, lane, lane < w ? __ldcg(a.ext + f + lane) : 0.0);
+    ublock_finish(a, f, w, lane, lane < w ? __ldcg(a.ext + f + lane) : 0.0, tri);
 }
 
 // kernels of the level launches; a batch puts the set in blockIdx.y
-#define GBLU_WARP_KERNEL(name, body)                                                             \
+// (tri: doubles of shared memory per warp)
+#define GBLU_WARP_KERNEL(name, body, tri)                                                        \
     template <bool kBatch>                                                                      \
     __global__ void __launch_bounds__(kSolveWarpsPerBlock * 32) name(SolveArgs a)               \
     {                                                                                           \
         const int t = blockIdx.x * kSolveWarpsPerBlock + (threadIdx.x >> 5), lane = threadIdx.x & 31; \
+        extern __shared__ double s_tri[];                                                       \
+        double *wt = s_tri + (threadIdx.x >> 5) * (tri);                                        \
         if (t >= a.nrows) return;                                                               \
-        if (kBatch) body(set_view(a, blockIdx.y), t, lane);                                     \
-        else body(a, t, lane);                                                                  \
+        if (kBatch) body(set_view(a, blockIdx.y), t, lane, wt);                                 \
+        else body(a, t, lane, wt);                                                              \
     }
-GBLU_WARP_KERNEL(lsolve_level_kernel, lsolve_level_row)
-GBLU_WARP_KERNEL(usolve_level_kernel, usolve_level_row)
-GBLU_WARP_KERNEL(lsolve_finish_kernel, lsolve_finish_block)
-GBLU_WARP_KERNEL(usolve_finish_kernel, usolve_finish_block)
+GBLU_WARP_KERNEL(lsolve_level_kernel, lsolve_level_row, 0)
+GBLU_WARP_KERNEL(usolve_level_kernel, usolve_level_row, 0)
+GBLU_WARP_KERNEL(lsolve_finish_kernel, lsolve_finish_block, kTriDoubles)
+GBLU_WARP_KERNEL(usolve_finish_kernel, usolve_finish_block, kTriDoubles)
 #undef GBLU_WARP_KERNEL
 
 // sync-free: a.rows[0..nrows) = rows in a topological order (blocks by
 // level, the finishing row of each block last), handed out by ticket; in a
 // batch ticket t is row ticket t / nsets of set t % nsets.  true = stop.
-__device__ __forceinline__ bool lsolve_sf_row(const SolveArgs &a, int t, int lane)
+__device__ __forceinline__ bool lsolve_sf_row(const SolveArgs &a, int t, int lane, double *tri)
 {
     const int i = __ldg(a.rows + t), b = __ldg(a.rb + i);
     const int f = __ldg(a.bs + b), w = __ldg(a.bs + b + 1) - f, q = i - f;
@@ -767,18 +802,16 @@ __device__ __forceinline__ bool lsolve_sf_row(const SolveArgs &a, int t, int lan
         return false;
     }
     // the last row finishes the block; its triangle is loaded first
-    double tv[kBR - 1];
-    lblock_load(a, f, w, lane, tv);
+    const double rhs = lblock_load(a, f, w, lane, tri);
     if (!lrow_ext(a, i, q, lane, true, s)) return true;
-    double e = s;
-    bool ok = true;
-    if (lane < w - 1) ok = await_value(a.ext, f + lane, a, 5, f + lane, e);
-    if (!__all_sync(kFull, ok)) return true;
-    lblock_solve(a, f, w, lane, e, tv);
+    double e;
+    if (!await_value(a.ext, f + lane, lane < w - 1, a, 5, f, e)) return true;
+    if (lane >= w - 1) e = s;
+    lblock_solve(a, f, w, lane, rhs, e, tri);
     return false;
 }
 
-__device__ __forceinline__ bool usolve_sf_row(const SolveArgs &a, int t, int lane)
+__device__ __forceinline__ bool usolve_sf_row(const SolveArgs &a, int t, int lane, double *tri)
 {
     const int i = __ldg(a.rows + t), b = __ldg(a.rb + i);
     const int f = __ldg(a.bs + b), w = __ldg(a.bs + b + 1) - f, q = i - f;
@@ -789,14 +822,14 @@ __device__ __forceinline__ bool usolve_sf_row(const SolveArgs &a, int t, int lan
         return false;
     }
     // the first row finishes the block; its triangle is loaded first
-    double tu[kBR], rd;
-    ublock_load(a, f, w, lane, tu, rd);
+    double rd;
+    int qx;
+    const double rhs = ublock_load(a, f, w, lane, tri, rd, qx);
     if (!urow_ext(a, i, q, w, lane, true, s)) return true;
-    double e = s;
-    bool ok = true;
-    if (lane >= 1 && lane < w) ok = await_value(a.ext, f + lane, a, 6, f + lane, e);
-    if (!__all_sync(kFull, ok)) return true;
-    ublock_solve(a, f, w, lane, e, tu, rd);
+    double e;
+    if (!await_value(a.ext, f + lane, lane >= 1 && lane < w, a, 6, f, e)) return true;
+    if (lane == 0) e = s;
+    ublock_solve(a, f, w, lane, rhs, e, tri, rd, qx);
     return false;
 }
 
@@ -804,6 +837,8 @@ __device__ __forceinline__ bool usolve_sf_row(const SolveArgs &a, int t, int lan
     template <bool kBatch>                                                                      \
     __global__ void __launch_bounds__(kSolveWarpsPerBlock * 32) name(SolveArgs a)               \
     {                                                                                           \
+        extern __shared__ double s_tri[];                                                       \
+        double *wt = s_tri + (threadIdx.x >> 5) * kTriDoubles;                                  \
         const int lane = threadIdx.x & 31;                                                      \
         const int total = kBatch ? a.nrows * a.nsets : a.nrows;                                 \
         for (;;) {                                                                              \
@@ -811,8 +846,8 @@ __device__ __forceinline__ bool usolve_sf_row(const SolveArgs &a, int t, int lan
             if (lane == 0) t = atomicAdd(&a.ctl->tick, 1);                                      \
             t = __shfl_sync(kFull, t, 0);                                                       \
             if (t >= total) break;                                                              \
-            const bool stop = kBatch ? body(set_view(a, t % a.nsets), t / a.nsets, lane)        \
-                                     : body(a, t, lane);                                        \
+            const bool stop = kBatch ? body(set_view(a, t % a.nsets), t / a.nsets, lane, wt)    \
+                                     : body(a, t, lane, wt);                                    \
             if (stop) break;                                                                    \
         }                                                                                       \
     }
@@ -828,6 +863,8 @@ template <bool kLower>
 __global__ void __launch_bounds__(kSolveWarpsPerBlock * 32)
 solve_multi_kernel(const SolveArgs *sets, const SetTask *order, int total, int32_t *ticket)
 {
+    extern __shared__ double s_tri[];
+    double *wt = s_tri + (threadIdx.x >> 5) * kTriDoubles;
     const int lane = threadIdx.x & 31;
     for (;;) {
         int t = 0;
@@ -836,7 +873,7 @@ solve_multi_kernel(const SolveArgs *sets, const SetTask *order, int total, int32
         if (t >= total) break;
         const SetTask o = order[t];
         const SolveArgs a = sets[o.set];
-        const bool stop = kLower ? lsolve_sf_row(a, o.task, lane) : usolve_sf_row(a, o.task, lane);
+        const bool stop = kLower ? lsolve_sf_row(a, o.task, lane, wt) : usolve_sf_row(a, o.task, lane, wt);
         if (stop) break;
     }
 }
@@ -979,6 +1016,15 @@ __device__ bool trail_slice(const SolveArgs &a, const TrailArgs &t, int I, doubl
     const int i0 = t.p0 + kTB * I, w = min(kTB, t.n - i0), i = i0 + lane;
     if (warp == 0 && !trail_stage(dtile, a.LUx, t, kLower, I, I, lane))   // off the critical path
         for (int idx = lane; idx < kTB * kTileLd; idx += 32) dtile[idx] = 0.0;
+    // warp 0 finishes the slice: its right-hand side and the reciprocals of
+    // its diagonal are ready before the waits, off the chain
+    double rhs = 0.0, rd = 1.0;
+    if (warp == 0 && lane < w) {
+        if (kLower) rhs = __ldg(a.b + __ldg(a.piv + i)) - __ldcg(a.ext + i);
+        else { rhs = __ldcg(a.y + i); rd = 1.0 / dtile[lane * kTileLd + lane]; }
+    }
+    keep(rhs);
+    keep(rd);
     // this warp's blocks: J(m) = first + step * m while in range
     const int first = kLower ? warp : t.nb - 1 - warp, step = kLower ? kTrailWarps : -kTrailWarps;
     auto in_range = [&](int J) { return kLower ? J < I : J > I; };
@@ -992,10 +1038,8 @@ __device__ bool trail_slice(const SolveArgs &a, const TrailArgs &t, int I, doubl
         const bool have_n = in_range(Jn) && trail_stage(nxt, a.LUx, t, kLower, I, Jn, lane);
         if (have) {
             const int j0 = t.p0 + kTB * J, wj = min(kTB, t.n - j0);
-            double vq = 0.0;
-            bool got = true;
-            if (lane < wj) got = await_value(kLower ? a.y : a.z, j0 + lane, a, kLower ? 7 : 8, i0, vq);
-            ok = __all_sync(kFull, got);
+            double vq;
+            ok = await_value(kLower ? a.y : a.z, j0 + lane, lane < wj, a, kLower ? 7 : 8, i0, vq);
             if (ok) {
 #pragma unroll
                 for (int c = 0; c < kTB; c += 4) {   // columns past wj hold zero tiles and vq = 0
@@ -1019,22 +1063,24 @@ __device__ bool trail_slice(const SolveArgs &a, const TrailArgs &t, int I, doubl
 #pragma unroll
         for (int q = 0; q < kTrailWarps; q++) sum += part[q * 32 + lane];
         if (kLower) {
-            double v = 0.0;
-            if (lane < w) v = __ldg(a.b + __ldg(a.piv + i)) - __ldcg(a.ext + i) - sum;
-            for (int c = 0; c < w - 1; c++) {
-                const double yc = __shfl_sync(kFull, v, c);
-                if (lane > c && lane < w) v = fma(-dtile[c * kTileLd + lane], yc, v);
+            double v = lane < w ? rhs - sum : 0.0;
+#pragma unroll 8
+            for (int c = 0; c < kTB - 1; c++) {   // (columns past w have zero tiles)
+                const double nv = fma(-dtile[c * kTileLd + lane], __shfl_sync(kFull, v, c), v);
+                v = lane > c && c < w - 1 ? nv : v;
             }
             if (lane < w) st_relaxed_f64(a.y + i, v);
         } else {
             double v = 0.0, zl = 0.0;
-            if (lane < w) v = __ldcg(a.y + i) - sum;
-            // reciprocals of the diagonal by every lane at once, off the chain
-            const double rd = lane < w ? 1.0 / dtile[lane * kTileLd + lane] : 1.0;
-            for (int c = w - 1; c >= 0; c--) {
-                const double zc = __shfl_sync(kFull, v, c) * __shfl_sync(kFull, rd, c);
-                if (lane == c) zl = zc;
-                if (lane < c) v = fma(-dtile[c * kTileLd + lane], zc, v);
+            if (lane < w) v = rhs - sum;
+#pragma unroll 8
+            for (int c = kTB - 1; c >= 0; c--) {
+                if (c < w) {
+                    const double zc = __shfl_sync(kFull, v, c) * __shfl_sync(kFull, rd, c);
+                    const double nv = fma(-dtile[c * kTileLd + lane], zc, v);
+                    zl = lane == c ? zc : zl;
+                    v = lane < c ? nv : v;
+                }
             }
             if (lane < w) {
                 st_relaxed_f64(a.z + i, zl);
@@ -1419,8 +1465,8 @@ int launch_lsolve(const SolveArgs &a, bool level_mode, int grid, void *stream)
         if (batch) lsolve_level_kernel<true><<<g, kSolveWarpsPerBlock * 32, 0, st>>>(a);
         else lsolve_level_kernel<false><<<g, kSolveWarpsPerBlock * 32, 0, st>>>(a);
     } else {
-        if (batch) lsolve_syncfree_kernel<true><<<grid, kSolveWarpsPerBlock * 32, 0, st>>>(a);
-        else lsolve_syncfree_kernel<false><<<grid, kSolveWarpsPerBlock * 32, 0, st>>>(a);
+        if (batch) lsolve_syncfree_kernel<true><<<grid, kSolveWarpsPerBlock * 32, kSolveSmem, st>>>(a);
+        else lsolve_syncfree_kernel<false><<<grid, kSolveWarpsPerBlock * 32, kSolveSmem, st>>>(a);
     }
     return (int)cudaGetLastError();
 }
@@ -1432,11 +1478,11 @@ int launch_solve_finish(const SolveArgs &a, bool lower, void *stream)
     const dim3 g((a.nrows + kSolveWarpsPerBlock - 1) / kSolveWarpsPerBlock, batch ? a.nsets : 1);
     cudaStream_t st = (cudaStream_t)stream;
     if (lower) {
-        if (batch) lsolve_finish_kernel<true><<<g, kSolveWarpsPerBlock * 32, 0, st>>>(a);
-        else lsolve_finish_kernel<false><<<g, kSolveWarpsPerBlock * 32, 0, st>>>(a);
+        if (batch) lsolve_finish_kernel<true><<<g, kSolveWarpsPerBlock * 32, kSolveSmem, st>>>(a);
+        else lsolve_finish_kernel<false><<<g, kSolveWarpsPerBlock * 32, kSolveSmem, st>>>(a);
     } else {
-        if (batch) usolve_finish_kernel<true><<<g, kSolveWarpsPerBlock * 32, 0, st>>>(a);
-        else usolve_finish_kernel<false><<<g, kSolveWarpsPerBlock * 32, 0, st>>>(a);
+        if (batch) usolve_finish_kernel<true><<<g, kSolveWarpsPerBlock * 32, kSolveSmem, st>>>(a);
+        else usolve_finish_kernel<false><<<g, kSolveWarpsPerBlock * 32, kSolveSmem, st>>>(a);
     }
     return (int)cudaGetLastError();
 }
@@ -1449,8 +1495,8 @@ int launch_solve_multi(const SolveArgs *lo, const SolveArgs *up, int nsets, int 
     int gx = (max_n + 255) / 256;
     gx = gx < 1 ? 1 : (gx > 64 ? 64 : gx);
     begin_multi_solve_kernel<<<dim3(gx, nsets), 256, 0, st>>>(lo, up, tickets);
-    solve_multi_kernel<true><<<grid, kSolveWarpsPerBlock * 32, 0, st>>>(lo, order_l, total_l, tickets);
-    solve_multi_kernel<false><<<grid, kSolveWarpsPerBlock * 32, 0, st>>>(up, order_u, total_u, tickets + 1);
+    solve_multi_kernel<true><<<grid, kSolveWarpsPerBlock * 32, kSolveSmem, st>>>(lo, order_l, total_l, tickets);
+    solve_multi_kernel<false><<<grid, kSolveWarpsPerBlock * 32, kSolveSmem, st>>>(up, order_u, total_u, tickets + 1);
     return (int)cudaGetLastError();
 }
 
@@ -1464,8 +1510,8 @@ int launch_usolve(const SolveArgs &a, bool level_mode, int grid, void *stream)
         if (batch) usolve_level_kernel<true><<<g, kSolveWarpsPerBlock * 32, 0, st>>>(a);
         else usolve_level_kernel<false><<<g, kSolveWarpsPerBlock * 32, 0, st>>>(a);
     } else {
-        if (batch) usolve_syncfree_kernel<true><<<grid, kSolveWarpsPerBlock * 32, 0, st>>>(a);
-        else usolve_syncfree_kernel<false><<<grid, kSolveWarpsPerBlock * 32, 0, st>>>(a);
+        if (batch) usolve_syncfree_kernel<true><<<grid, kSolveWarpsPerBlock * 32, kSolveSmem, st>>>(a);
+        else usolve_syncfree_kernel<false><<<grid, kSolveWarpsPerBlock * 32, kSolveSmem, st>>>(a);
     }
     return (int)cudaGetLastError();
 }
@@ -1525,17 +1571,22 @@ int solve_syncfree_grid(int *grid)
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     int p[4] = {0, 0, 0, 0};
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p[0], lsolve_syncfree_kernel<false>,
-                                                                  kSolveWarpsPerBlock * 32, 0);
-    if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p[1], usolve_syncfree_kernel<false>,
-                                                          kSolveWarpsPerBlock * 32, 0);
-    if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p[2], lsolve_syncfree_kernel<true>,
-                                                          kSolveWarpsPerBlock * 32, 0);
-    if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p[3], usolve_syncfree_kernel<true>,
-                                                          kSolveWarpsPerBlock * 32, 0);
+    cudaError_t e = cudaSuccess;
+    auto setup = [&](auto kernel, int *out) {
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSolveSmem);
+        if (e == cudaSuccess && out)
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, kernel, kSolveWarpsPerBlock * 32, kSolveSmem);
+    };
+    setup(lsolve_syncfree_kernel<false>, &p[0]);
+    setup(usolve_syncfree_kernel<false>, &p[1]);
+    setup(lsolve_syncfree_kernel<true>, &p[2]);
+    setup(usolve_syncfree_kernel<true>, &p[3]);
+    setup(lsolve_finish_kernel<false>, nullptr);
+    setup(usolve_finish_kernel<false>, nullptr);
+    setup(lsolve_finish_kernel<true>, nullptr);
+    setup(usolve_finish_kernel<true>, nullptr);
+    setup(solve_multi_kernel<true>, nullptr);
+    setup(solve_multi_kernel<false>, nullptr);
     if (e != cudaSuccess) return (int)e;
     per = p[0];
     for (int i = 1; i < 4; i++) per = p[i] < per ? p[i] : per;
