@@ -188,11 +188,12 @@ __global__ void __launch_bounds__(kT) block_step_kernel(BlockArgs a, int step)
             const double inv = 1.0 / s.d[k][k];
             const double l = xq * inv;
             if (tid == 0) s.inv[k] = inv;
-            if (q > k) {
-                if (g == 0) s.l[q][k] = l;
-                if (g > k) { v0 = fma(-u0, l, v0); s.d[q][g] = v0; }
-                if (g + 8 > k) { v1 = fma(-u1, l, v1); s.d[q][g + 8] = v1; }
-            }
+            const double n0 = fma(-u0, l, v0), n1 = fma(-u1, l, v1);
+            v0 = q > k && g > k ? n0 : v0;
+            v1 = q > k && g + 8 > k ? n1 : v1;
+            if (q > k && g == 0) s.l[q][k] = l;
+            if (q > k && g > k) s.d[q][g] = v0;
+            if (q > k && g + 8 > k) s.d[q][g + 8] = v1;
             __syncthreads();
         }
         for (int i = tid; i < nb * nb; i += kT) {

@@ -280,12 +280,16 @@ __device__ __forceinline__ bool panel_consume(R *X, bool in_smem, unsigned char 
                 R v[C];
 #pragma unroll
                 for (int c = 0; c < C; c++) v[c] = lane < w ? x[c * kConsWarps] : R(0);
+                // (selects, not branches: a divergent step costs several times
+                // its arithmetic)
+                const R *lp = val + max(lane, 1) - 1;
+#pragma unroll 4
                 for (int d = 0; d < w - 1; d++) {
-                    const R lv = (lane > d && lane < w) ? val[h.off[d] + lane - 1] : R(0);
+                    const R lv = lp[h.off[d]];
 #pragma unroll
                     for (int c = 0; c < C; c++) {
-                        const R m = __shfl_sync(kFull, v[c], d);
-                        if (lane > d) v[c] = fma(-lv, m, v[c]);
+                        const R nv = fma(-lv, __shfl_sync(kFull, v[c], d), v[c]);
+                        v[c] = lane > d && lane < w ? nv : v[c];
                     }
                 }
                 if (lane < w) {
@@ -622,12 +626,13 @@ __device__ __noinline__ bool col_panel(const RefactorArgsT<R> *ap, int id, unsig
                 __threadfence_block();
                 *step = s + 1;
             }
-            const R l = xq * inv;
-            if (q > s) {
-                if (c0 > s) v0 = fma(-u0, l, v0);
-                if (LD > 4 && c1 > s) v1 = fma(-u1, l, v1);
-                if (c0 == 0) sh.Lb[q * kPanelMax + s] = l;
+            const R l = xq * inv, n0 = fma(-u0, l, v0);
+            v0 = q > s && c0 > s ? n0 : v0;
+            if (LD > 4) {
+                const R n1 = fma(-u1, l, v1);
+                v1 = q > s && c1 > s ? n1 : v1;
             }
+            if (q > s && c0 == 0) sh.Lb[q * kPanelMax + s] = l;
         }
         // below the diagonal: the unscaled values
         if (q > c0) sh.D[q * kPanelMax + c0] = v0;

@@ -206,8 +206,9 @@ __device__ bool col_warp(const RefactorArgsT<R> &a, int k, R *xs, int32_t *rs, i
 #pragma unroll
             for (int d = 0; d < kWarpRun - 1; d++) {
                 if (d < w - 1) {
-                    const R mv = __shfl_sync(kFull, v, d);
-                    if (lane > d && lane < w) v = fma(-tv[d], mv, v);
+                    // (a select: a divergent step costs several times its arithmetic)
+                    const R nv = fma(-tv[d], __shfl_sync(kFull, v, d), v);
+                    v = lane > d && lane < w ? nv : v;
                 }
             }
             if (lane < w) x[t + lane] = v;
@@ -648,9 +649,11 @@ __device__ bool col_grp(const RefactorArgsT<R> &a, int k, R *xs, int32_t *rs, in
             }
             __syncwarp();
             R v = lane < w ? x[t + lane] : R(0);
-            for (int d = 0; d < w - 1; ++d) {
-                const R mv = __shfl_sync(kFull, v, d);
-                if (lane > d && lane < w) v = fma(-sh.tri[tri_off(d) + lane - d - 1], mv, v);
+#pragma unroll 4
+            for (int d = 0; d < w - 1; ++d) {   // selects, not branches
+                const R l = sh.tri[tri_off(d) + max(lane - d - 1, 0)];
+                const R nv = fma(-l, __shfl_sync(kFull, v, d), v);
+                v = lane > d && lane < w ? nv : v;
             }
             if (lane < w) x[t + lane] = v;
         }
