@@ -185,7 +185,7 @@ __global__ void __launch_bounds__(kT) block_step_kernel(BlockArgs a, int step)
         __syncthreads();
         for (int k = 0; k < nb; k++) {
             const double xq = s.d[q][k], u0 = s.d[k][g], u1 = s.d[k][g + 8];
-            const double inv = 1.0 / s.d[k][k];
+            const double inv = __drcp_rn(s.d[k][k]);   // 1 / x, correctly rounded
             const double l = xq * inv;
             if (tid == 0) s.inv[k] = inv;
             const double n0 = fma(-u0, l, v0), n1 = fma(-u1, l, v1);

@@ -132,6 +132,21 @@ __device__ __forceinline__ void stv(R *p, const R (&v)[N])
     }
 }
 
+// 1 / x, correctly rounded (as the division is)
+__device__ __forceinline__ double recip(double x) { return __drcp_rn(x); }
+__device__ __forceinline__ float recip(float x) { return __frcp_rn(x); }
+
+__device__ __forceinline__ void st_release_cta(int *p, int v)
+{
+    asm volatile("st.release.cta.shared.b32 [%0], %1;" ::"r"((unsigned)__cvta_generic_to_shared(p)), "r"(v) : "memory");
+}
+__device__ __forceinline__ int ld_acquire_cta(const int *p)
+{
+    int v;
+    asm volatile("ld.acquire.cta.shared.b32 %0, [%1];" : "=r"(v) : "r"((unsigned)__cvta_generic_to_shared(p)) : "memory");
+    return v;
+}
+
 // |x| as an integer of the same order (NaN above infinity), so that maxima
 // stay off the FP64 pipe
 __device__ __forceinline__ unsigned long long abs_key(double v)
@@ -604,7 +619,6 @@ __device__ __noinline__ bool col_panel(const RefactorArgsT<R> *ap, int id, unsig
     // they are done; the other warps follow with the L rows below the block,
     // 32 rows at a time
     const int nuk = lane < nc ? __ldg(nUp + k0 + lane) : 0;
-    volatile int *step = &sh.step;
     if (warp == 0) {
         const int q = lane & 7, c0 = lane >> 3, c1 = c0 + 4;   // this lane's entries (q, c0), (q, c1)
         R v0 = (q < nc && c0 < nc) ? X[(size_t)(nu + q) * LD + c0] : R(0);
@@ -619,13 +633,10 @@ __device__ __noinline__ bool col_panel(const RefactorArgsT<R> *ap, int id, unsig
                 sh.D[q * kPanelMax + c0] = v0;
                 if (LD > 4) sh.D[q * kPanelMax + c1] = v1;
             }
-            const R inv = R(1) / d;
+            const R inv = recip(d);
             if (lane == 0) sh.inv[s] = inv;
             __syncwarp();
-            if (lane == 0) {
-                __threadfence_block();
-                *step = s + 1;
-            }
+            if (lane == 0) st_release_cta(&sh.step, s + 1);
             const R l = xq * inv, n0 = fma(-u0, l, v0);
             v0 = q > s && c0 > s ? n0 : v0;
             if (LD > 4) {
@@ -670,7 +681,7 @@ __device__ __noinline__ bool col_panel(const RefactorArgsT<R> *ap, int id, unsig
 #pragma unroll
         for (int s = 0; s < LD; s++) {
             if (s < nc) {
-                for (long long it = 0; *step <= s && it < kBarTries; ++it) {}   // warp 0 is on its way
+                for (long long it = 0; ld_acquire_cta(&sh.step) <= s && it < kBarTries; ++it) {}   // warp 0 is on its way
                 __syncwarp();
                 const int64_t o = __shfl_sync(kFull, out, s);
                 if (in) {
@@ -704,13 +715,24 @@ __device__ __noinline__ bool col_panel(const RefactorArgsT<R> *ap, int id, unsig
     // ---- pivot checks (lane c of warp 0: column c) and publication
     if (warp == 0) {
         bool pass = true;
-        if (lane < nc) {
-            unsigned long long m = 0;
-            for (int i = 0; i < kWarps; i++) m = sh.mx[i][lane] > m ? sh.mx[i][lane] : m;
-            for (int i = lane + 1; i < nc; i++) {
-                const unsigned long long key = abs_key(sh.D[i * kPanelMax + lane]);
-                m = key > m ? key : m;
+        // column c = lane & 7: four lanes share its eight warps' maxima and
+        // the rows of the diagonal block
+        unsigned long long m = 0;
+        {
+            const int c = lane & 7, h = lane >> 3;
+            if (c < nc) {
+#pragma unroll
+                for (int i = 0; i < 2; i++) {
+                    const unsigned long long v = sh.mx[2 * h + i][c];
+                    const int r = 2 * h + i;
+                    const unsigned long long key = r > c && r < nc ? abs_key(sh.D[r * kPanelMax + c]) : 0ull;
+                    m = max(m, max(v, key));
+                }
             }
+            m = max(m, __shfl_xor_sync(kFull, m, 8));
+            m = max(m, __shfl_xor_sync(kFull, m, 16));
+        }
+        if (lane < nc) {
             pass = check_pivot(a, k0 + lane, sh.D[lane * kPanelMax + lane], key_abs(m, R(0)));
         }
         const unsigned ok = __ballot_sync(kFull, pass);
