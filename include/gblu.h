@@ -127,7 +127,8 @@ typedef struct {
     /* batches of value sets (gblu_refactorize_batch): the persistent launch
        takes the sets in groups of batch_group, all tasks of one group before
        the next group's, so that the factors being read stay in L2 (0 = as
-       many sets as fit in half of L2; >= nsets: every set at once).
+       many sets as fit in half of L2, at least 32; >= nsets: every set at
+       once).
        Default 0. */
     int batch_group;
     /* CTAs (8 warps each) per SM of the sync-free solve launches; 0 = as

@@ -390,8 +390,10 @@ int install_structure(gblu_ctx *h, Structure &&S, const std::vector<double> *val
     const int resident_warps = h->ref_blocks_per_sm[1] * h->sm_count * (kRefThreads / 32);
     const SolveSplit sp = solve_split(h->opts);
     const auto t_s = std::chrono::steady_clock::now();
-    const int panel_ctas =   // scratch panels only run with kRefSmemTwo
-        std::max(h->ref_blocks_per_sm[0], std::max(h->batch_blocks_per_sm[0], h->ref32_blocks_per_sm[0])) * h->sm_count;
+    int panel_ctas[2];
+    for (int i = 0; i < 2; i++)
+        panel_ctas[i] =
+            std::max(h->ref_blocks_per_sm[i], std::max(h->batch_blocks_per_sm[i], h->ref32_blocks_per_sm[i])) * h->sm_count;
     build_schedule(h->P, h->S, h->opts.alpha, resident_warps, panel_ctas, h->opts.sched_mode, h->opts.warp_column_max, sp,
                    h->opts.dense_min_rows, h->W, defer_solve);
     h->solve_pending = defer_solve;
@@ -410,10 +412,11 @@ int install_structure(gblu_ctx *h, Structure &&S, const std::vector<double> *val
         // one scratch per CTA that a persistent launch can hold; only while it
         // stays within kPullScratchBytes (the columns are pushed otherwise)
         const int slots = std::max(h->ref_blocks_per_sm[1], h->batch_blocks_per_sm[1]) * h->sm_count;
-        const size_t bytes = (size_t)slots * (size_t)n * (sizeof(double) + sizeof(unsigned long long));
+        const size_t ld = (size_t)h->W.pull_ld;
+        const size_t bytes = (size_t)slots * (size_t)n * (ld * sizeof(double) + sizeof(unsigned long long));
         if (bytes <= kPullScratchBytes) {
             CK(upload(h, h->pull_start, h->W.pull_start, st));
-            CK(ensure(h, h->pull_x, (size_t)slots * n));
+            CK(ensure(h, h->pull_x, (size_t)slots * n * ld));
             CK(ensure(h, h->pull_tag, (size_t)slots * n));
             CK(ensure(h, h->pull_ctr, (size_t)slots));
             CK(ensure(h, h->pull_lock, (size_t)slots));
@@ -443,8 +446,8 @@ int install_structure(gblu_ctx *h, Structure &&S, const std::vector<double> *val
     }
     h->pscratch_ctas = 0;
     if (h->W.pscratch > 0) {
-        CK(ensure(h, h->pscratch, (size_t)panel_ctas * (size_t)h->W.pscratch));
-        h->pscratch_ctas = panel_ctas;
+        h->pscratch_ctas = panel_ctas[cfg(h)];
+        CK(ensure(h, h->pscratch, (size_t)h->pscratch_ctas * (size_t)h->W.pscratch));
     }
     CK(upload(h, h->dense_s0, h->W.dense_s0, st));
     if (h->W.dense_m > 0) CK(ensure(h, h->dense, (size_t)h->W.dense_m * h->W.dense_m));
@@ -541,6 +544,7 @@ RefactorArgs refactor_args(gblu_ctx *h, const double *Ax)
         a.pull_ctr = h->pull_ctr.p;
         a.pull_lock = h->pull_lock.p;
         a.pull_slots = h->pull_slots;
+        a.pull_ld = h->W.pull_ld;
     }
     a.n = h->S.n;
     a.pan_id = h->pan_id.p;
@@ -1670,13 +1674,19 @@ int gblu_solve(gblu_handle h, const double *b_dev, double *x_dev, void *stream)
 }
 
 // sets per group of a batch's persistent launch: the option, else as many
-// sets as fit in half of L2 (their factor and A values)
+// sets as fit in half of L2 (their factor and A values), at least
+// kBatchGroup: a set's panels wait for one another, and the panels of other
+// sets fill the device meanwhile (one set per group against four: 40,000
+// unknowns 51 -> 43 ms, 57,600 unknowns 62 -> 50 ms; the bordered 141x141
+// grid, 256 sets, 8, 16, 32, 64 and 256 per group: 281, 272, 265, 269 and
+// 283 ms)
+constexpr int kBatchGroup = 32;
 static int batch_group(gblu_ctx *h, int32_t nsets)
 {
     int g = h->opts.batch_group;
     if (g <= 0) {
         const double per = 8.0 * ((double)h->S.nnz() + (double)h->P.Ai.size());
-        g = (int)std::max(1.0, 0.5 * (double)h->l2_bytes / std::max(per, 1.0));
+        g = (int)std::max((double)kBatchGroup, 0.5 * (double)h->l2_bytes / std::max(per, 1.0));
     }
     return std::min(g, (int)nsets);
 }

@@ -79,6 +79,7 @@ struct PanelDesc {
     int64_t roff;   // first of nruns runs in prun
     int32_t k0, nc, nu, nruns;
     int32_t nux, nrunsx;   // slots and runs of dependencies before the trailing block (k0 in the block)
+    int32_t pull, runp;    // wide columns: the first pull slots are taken row by row, the runs after them begin at runp
 };
 // w <= kPanelRun consecutive dependencies j0 .. at slots t .. t+w-1 in one
 // supernode of L; wm = w | (mask of the panel's columns that have any of
@@ -175,6 +176,7 @@ struct Schedule {
     // diagonal are taken that way (0: none); pull_cols = columns with > 0
     std::vector<int32_t> pull_start;
     int64_t pull_cols = 0;
+    int32_t pull_ld = 1;              // values per row of a pull scratch (kPullLd with panels of wide columns)
     // dividing threshold of the levels (alpha x resident warps); which parts
     // are built: the row-wise copies, and the whole solve part
     double thr = 0.0;
@@ -185,6 +187,7 @@ struct Schedule {
 constexpr int kPullMaxL = 64;
 constexpr int kPullMinRuns = 256;
 constexpr size_t kPullScratchBytes = (size_t)1 << 30;
+constexpr int kPullLd = 4;            // wide columns of a panel
 // trailing block: at least kBlockMin columns, at most kBlockMax (302 MB of
 // values), at least kBlockDensity of its entries in the factor
 constexpr int kBlockCols = 16, kBlockMin = 128, kBlockMax = 6144;
@@ -235,7 +238,7 @@ int64_t unsymmetric_entries(const Pattern &P);
 // The schedule of a structure; with defer_solve, only what the
 // re-factorization reads (the solve part follows by build_solve_schedule)
 void build_schedule(const Pattern &P, const Structure &S, double alpha,
-                    int resident_warps, int panel_ctas, int sched_mode, int cap_short, const SolveSplit &split,
+                    int resident_warps, const int (&panel_ctas)[2], int sched_mode, int cap_short, const SolveSplit &split,
                     int dense_min_rows, Schedule &W, bool defer_solve = false);
 void build_solve_schedule(const Structure &S, const SolveSplit &split, Schedule &W);
 // levels of the column dependency graph; with cut < n, the dependencies of
@@ -315,7 +318,7 @@ struct RefactorArgsT {
     double *pull_x = nullptr;
     unsigned long long *pull_tag = nullptr, *pull_ctr = nullptr;
     int32_t *pull_lock = nullptr;
-    int32_t pull_slots = 0, n = 0;
+    int32_t pull_slots = 0, n = 0, pull_ld = 1;
     // panels (Schedule::pan); pscratch: per CTA (blockIdx.x) pscratch_bytes
     // for the panels beyond shared memory
     const int32_t *pan_id = nullptr;

@@ -43,6 +43,8 @@ struct PanelShared {
     unsigned long long mx[kWarps][kPanelMax];    // bits of max |x| over the L rows, by warp
     unsigned pass;
     int abort;                                   // a producer gave up: everyone leaves
+    int pull_slot;                               // wide columns: the scratch in use
+    unsigned long long pull_tag;                 // and its tag
     int step, next;                              // finished columns of the diagonal block; next L row to take
 };
 
@@ -520,6 +522,156 @@ __device__ __forceinline__ void store_u_rows(const RefactorArgsT<R> &a, const Pa
     }
 }
 
+// The first p0 slots of a panel of wide columns (pull_rows, for all of the
+// panel's columns at once: an entry of L, its row's tag and the wait for a
+// value, whose latency bounds the chain, are paid once for four columns; 256
+// sets of the bordered 141x141 grid: 334 ms with single columns, 304 ms so.
+// A warp per row, with its entries' loads in parallel, took 334 ms, and with
+// them pipelined two chunks ahead 345 ms: 256 rows in flight hide more than
+// eight).  xd holds
+// kPullLd values per row.  A column without an entry that its neighbours
+// have holds a zero there.  Returns false if a wait gave up.
+template <int LD>
+__device__ __noinline__ bool pull_panel(const RefactorArgs *ap, int k0, double *X, const int32_t *rows, int len, int p0,
+                                        int epoch, bool wait, PanelShared<double> &sh)
+{
+    static_assert(LD == kPullLd, "the scratch's pitch");
+    const RefactorArgs &a = *ap;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int64_t *const Lrp = a.Lrp;
+    const int32_t *const Lcol = a.Lcol, *const Lslot = a.Lslot;
+    const double *const LUx = a.LUx;
+    bool fail = false;
+    auto timeout = [&](int site) {
+        set_status(a.ctl, GBLU_ERR_DEVICE_TIMEOUT);
+        a.ctl->where = site;
+        a.ctl->where_k = k0;
+    };
+    if (tid == 0) {
+        int slot = -1;
+        for (long long it = 0; slot < 0; ++it) {
+            const int c = (int)((blockIdx.x + it) % a.pull_slots);
+            if (atomicCAS(a.pull_lock + c, 0, 1) == 0) slot = c;
+            else if (it > a.spin_limit) { timeout(11); break; }
+        }
+        sh.pull_slot = slot;
+        if (slot >= 0) sh.pull_tag = ++a.pull_ctr[slot];
+    }
+    __syncthreads();
+    const int slot = sh.pull_slot;
+    if (slot < 0) return false;
+    double *const xd = a.pull_x + (size_t)slot * a.n * LD;
+    unsigned long long *const xt = a.pull_tag + (size_t)slot * a.n;
+    const unsigned long long tag = sh.pull_tag;
+    auto release = [&]() {
+        __syncthreads();
+        if (tid == 0) atomicExch(a.pull_lock + slot, 0);
+    };
+    auto give_up = [&](long long it, int site) -> bool {
+        if ((it & 31) == 0 && (ld_volatile(&a.ctl->interrupted) || ld_volatile(&a.ctl->status))) return true;
+        if (it > a.spin_limit) {
+            timeout(site);
+            return true;
+        }
+        if (it > 64) __nanosleep(64);
+        return false;
+    };
+    if (wait)   // the prefix's dependencies are final
+        for (int s = tid; s < p0 && !fail; s += kThreads) {
+            const int j = rows[s];
+            for (long long it = 1; ld_acquire(a.finish + j) != epoch; ++it)
+                if (give_up(it, 9)) {
+                    fail = true;
+                    break;
+                }
+        }
+    if (__syncthreads_or(fail)) {
+        release();
+        return false;
+    }
+    const double sent = __longlong_as_double((long long)kSentinel);
+    for (int s = tid; s < p0; s += kThreads) {
+        const int r = rows[s];
+#pragma unroll
+        for (int c = 0; c < LD; c++) st_relaxed_f64(xd + (size_t)r * LD + c, sent);
+        st_relaxed_u64(xt + r, tag);
+    }
+    __syncthreads();
+    for (int s = tid; s < p0 && !fail; s += kThreads) {
+        const int r = rows[s];
+        double acc[LD];
+        ldv<double, LD>(X + (size_t)s * LD, acc);
+        const int64_t e1 = __ldg(Lrp + r + 1);
+        for (int64_t e = __ldg(Lrp + r); e < e1 && !fail; e++) {
+            const int j = __ldg(Lcol + e);
+            if (ld_relaxed_u64(xt + j) != tag) continue;
+            const double l = __ldcg(LUx + __ldg(Lslot + e));
+            const double *v = xd + (size_t)j * LD;
+            unsigned long long b[LD];
+            for (long long it = 1;; ++it) {
+                bool missing = false;
+#pragma unroll
+                for (int c = 0; c < LD; c++) b[c] = ld_relaxed_u64(v + c);
+#pragma unroll
+                for (int c = 0; c < LD; c++) missing = missing || b[c] == kSentinel;
+                if (!missing) break;
+                if (give_up(it, 10)) {
+                    fail = true;
+                    break;
+                }
+            }
+            if (fail) break;
+#pragma unroll
+            for (int c = 0; c < LD; c++) acc[c] = fma(-__longlong_as_double((long long)b[c]), l, acc[c]);
+        }
+        stv<double, LD>(X + (size_t)s * LD, acc);
+#pragma unroll
+        for (int c = 0; c < LD; c++) st_relaxed_f64(xd + (size_t)r * LD + c, acc[c]);
+    }
+    if (__syncthreads_or(fail)) {
+        release();
+        return false;
+    }
+    const int jlim = rows[p0 - 1];   // the last dependency of the prefix
+    for (int s = p0 + warp; s < len; s += kWarps) {
+        const int r = rows[s];
+        const int64_t e1 = __ldg(Lrp + r + 1);
+        double part[LD];
+#pragma unroll
+        for (int c = 0; c < LD; c++) part[c] = 0.0;
+        for (int64_t e0 = __ldg(Lrp + r) + lane; e0 < e1; e0 += 32 * 4) {
+            int j[4];
+            double l[4];
+            unsigned long long tg[4];
+#pragma unroll
+            for (int u = 0; u < 4; u++) j[u] = e0 + 32 * u < e1 ? __ldg(Lcol + e0 + 32 * u) : INT_MAX;
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                const bool in = j[u] <= jlim;   // ascending: the rest is past the prefix
+                tg[u] = in ? ld_relaxed_u64(xt + j[u]) : 0ull;
+                l[u] = in ? __ldcg(LUx + __ldg(Lslot + e0 + 32 * u)) : 0.0;
+            }
+#pragma unroll
+            for (int u = 0; u < 4; u++)
+                if (j[u] <= jlim && tg[u] == tag) {
+                    const double *v = xd + (size_t)j[u] * LD;
+#pragma unroll
+                    for (int c = 0; c < LD; c++)
+                        part[c] = fma(__longlong_as_double((long long)ld_relaxed_u64(v + c)), l[u], part[c]);
+                }
+            if (j[3] > jlim) break;
+        }
+#pragma unroll
+        for (int c = 0; c < LD; c++) {
+            const double t = warp_sum(part[c]);
+            if (lane == 0) X[(size_t)s * LD + c] -= t;
+        }
+    }
+    release();
+    __syncthreads();
+    return true;
+}
+
 // One panel by the whole CTA; true = stop.  Not inlined: its registers are
 // allocated apart from the column kernels' (they share a launch bound), and
 // the argument block stays where it is (kernel parameter or global memory).
@@ -594,9 +746,17 @@ __device__ __noinline__ bool col_panel(const RefactorArgsT<R> *ap, int id, unsig
     bool go = true;
     // a panel of the trailing block: its dependencies before the block
     const bool blk = k0 >= a.tb_p;
-    const int nruns = blk ? p.nrunsx : p.nruns, nux = blk ? p.nux : nu;
+    const int nux = blk ? p.nux : nu;
+    int run0 = 0;
+    if constexpr (std::is_same<R, double>::value && LD == kPullLd) {
+        if (p.pull > 0 && a.pull_start) {   // wide columns: their prefix row by row
+            if (!pull_panel<LD>(ap, k0, X, rows, len, p.pull, epoch, wait, sh)) return true;
+            run0 = p.runp;
+        }
+    }
+    const int nruns = (blk ? p.nrunsx : p.nruns) - run0;
     if (nruns > 0) {
-        const PanelRun *runs = a.prun + p.roff;
+        const PanelRun *runs = a.prun + p.roff + run0;
         if (warp < kConsWarps)
             go = panel_consume<R, LD>(X, in_smem, smem, stage_bytes, ns, sh, bars, a.ctl, warp, lane);
         else

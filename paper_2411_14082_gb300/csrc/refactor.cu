@@ -390,13 +390,13 @@ struct PullArgs {
     int32_t *pull_lock;
     DevCtl *ctl;
     long long spin_limit;
-    int32_t pull_slots, n;
+    int32_t pull_slots, n, pull_ld;
 };
 
 __device__ __forceinline__ PullArgs pull_args(const RefactorArgsT<double> &a)
 {
     return PullArgs{a.Lrp,    a.Lcol,     a.Lslot,    a.LUx, a.finish,     a.pull_x,     a.pull_tag,
-                    a.pull_ctr, a.pull_lock, a.ctl, a.spin_limit, a.pull_slots, a.n};
+                    a.pull_ctr, a.pull_lock, a.ctl, a.spin_limit, a.pull_slots, a.n, a.pull_ld};
 }
 
 template <bool kWait>
@@ -424,7 +424,7 @@ __device__ __forceinline__ bool pull_rows(const PullArgs a, int k, double *x, co
     __syncthreads();
     const int slot = sh.pull_slot;
     if (slot < 0) return false;
-    double *xd = a.pull_x + (size_t)slot * a.n;
+    double *xd = a.pull_x + (size_t)slot * a.n * a.pull_ld;
     unsigned long long *xt = a.pull_tag + (size_t)slot * a.n;
     const unsigned long long tag = sh.pull_tag;
     auto release = [&]() {

@@ -553,9 +553,16 @@ static void build_panels(const Structure &S, int panel_ctas, bool allow_scratch,
     // link[j]: columns j and j+1 may share a panel; long chains are cut every
     // 64 columns, the units that the host threads share
     std::vector<uint8_t> link(n, 0);
+    // wide columns share a panel when their prefixes end at the same step,
+    // and while the scratches of the CTAs stay within their bound
+    auto prefix_end = [&](int32_t k) { return S.LUi[S.LUp[k] + W.pull_start[k]]; };
+    const bool pull_panels =
+        W.pull_cols > 0 && (size_t)panel_ctas * (size_t)n * ((kPullLd + 1) * sizeof(double)) <= kPullScratchBytes / 2;
     for (int32_t j = 0, run = 1; j + 1 < n; j++) {
-        link[j] = j + 1 != W.tb_p && run < 64 && W.chain[j] && !W.pull_start[j] && !W.pull_start[j + 1] && S.nU[j + 1] >= 2 &&
-               S.LUi[S.LUp[j + 1] + S.nU[j + 1] - 2] == j;
+        const bool wide = W.pull_start[j] > 0, wide1 = W.pull_start[j + 1] > 0;
+        const bool same = wide || wide1 ? pull_panels && wide && wide1 && prefix_end(j) == prefix_end(j + 1) : true;
+        link[j] = same && j + 1 != W.tb_p && run < 64 && W.chain[j] && S.nU[j + 1] >= 2 &&
+                  S.LUi[S.LUp[j + 1] + S.nU[j + 1] - 2] == j;
         run = link[j] ? run + 1 : 1;
     }
     const int64_t smem = W.smem;
@@ -614,7 +621,8 @@ static void build_panels(const Structure &S, int panel_ctas, bool allow_scratch,
                 while (k < end) {
                     const int32_t left = end - k;
                     if (left == 1) { k++; break; }   // a column of its own
-                    int nc = std::min<int32_t>(left, kPanelMax);
+                    const bool wide = W.pull_start[k] > 0;
+                    int nc = std::min<int32_t>(left, wide ? kPullLd : kPanelMax);
                     auto l_rows = [&](int c) { return S.LUp[k + c + 1] - S.LUp[k + c] - S.nU[k + c]; };
                     auto least = [&](int c) {   // the union has at least this many slots
                         int64_t mx = 0;
@@ -632,10 +640,10 @@ static void build_panels(const Structure &S, int panel_ctas, bool allow_scratch,
                         if (!ok) nc = 4;
                     }
                     if (nc <= 4) {
-                        if (!allow_scratch && !fits(least(nc), nc)) { k++; continue; }
+                        if (!allow_scratch && !wide && !fits(least(nc), nc)) { k++; continue; }
                         nu = join(k, nc);
                         slots = nu + nc + l_rows(nc - 1);
-                        if (!fits(slots, nc) && !allow_scratch) { k++; continue; }
+                        if (!fits(slots, nc) && !allow_scratch && !wide) { k++; continue; }
                     }
                     const int64_t need = slots * (8 * panel_ld(nc) + 4);
                     if (!fits(slots, nc)) pt.scratch = std::max(pt.scratch, (need + 255) / 256 * 256);
@@ -643,6 +651,7 @@ static void build_panels(const Structure &S, int panel_ctas, bool allow_scratch,
                     d.k0 = k;
                     d.nc = nc;
                     d.nu = (int32_t)nu;
+                    d.pull = wide ? (int32_t)(std::lower_bound(u.begin(), u.begin() + nu, (uint64_t)prefix_end(k) << 8) - u.begin()) : 0;
                     d.uoff = (int64_t)pt.prow.size();
                     d.poff = (int64_t)pt.ppref.size();
                     pt.prow.resize(d.uoff + nu + nc);
@@ -682,10 +691,17 @@ static void build_panels(const Structure &S, int panel_ctas, bool allow_scratch,
         of[i + 1] = of[i] + (int64_t)parts[i].ppref.size();
         W.pscratch = std::max(W.pscratch, parts[i].scratch);
     }
-    if (W.pscratch > 0 && (size_t)W.pscratch * (size_t)panel_ctas > kPanelScratchBytes && allow_scratch) {
-        build_panels(S, panel_ctas, false, W);   // long columns one at a time
+    if (W.pscratch > 0 && (size_t)W.pscratch * (size_t)panel_ctas > kPanelScratchBytes) {
+        // long columns one at a time (and wide ones, when even they do not fit)
+        if (allow_scratch) build_panels(S, panel_ctas, false, W);
+        else {
+            std::fill(W.pan_id.begin(), W.pan_id.end(), -1);
+            W.pscratch = 0;
+            W.pan.clear();
+        }
         return;
     }
+    W.pull_ld = pull_panels ? kPullLd : 1;
     W.pan.resize(op[nparts]);
     W.prow.resize(ou[nparts]);
     W.pmask.resize(ou[nparts]);
@@ -710,7 +726,7 @@ static void build_panels(const Structure &S, int panel_ctas, bool allow_scratch,
                     int w = 1;
                     unsigned mk = m[s];
                     while (w < kPanelRun && s + w < d.nu && u[s + w] == u[s + w - 1] + 1 && W.chain[u[s + w - 1]] &&
-                           u[s + w] != W.tb_p && !(d.nu - (s + w) <= kPanelRun && first[u[s + w]])) {
+                           u[s + w] != W.tb_p && s + w != d.pull && !(d.nu - (s + w) <= kPanelRun && first[u[s + w]])) {
                         mk |= m[s + w];
                         w++;
                     }
@@ -726,6 +742,8 @@ static void build_panels(const Structure &S, int panel_ctas, bool allow_scratch,
                 }
                 d.nruns = (int32_t)((int64_t)pt.prun.size() - r0);
                 d.nux = (int32_t)(std::lower_bound(u, u + d.nu, W.tb_p) - u);
+                d.runp = 0;
+                while (d.runp < d.nruns && pt.prun[r0 + d.runp].t < d.pull) d.runp++;
                 d.nrunsx = 0;
                 while (d.nrunsx < d.nruns && pt.prun[r0 + d.nrunsx].t < d.nux) d.nrunsx++;
                 d.roff = r0;
@@ -746,7 +764,7 @@ static void build_panels(const Structure &S, int panel_ctas, bool allow_scratch,
 }
 
 void build_schedule(const Pattern &P, const Structure &S, double alpha,
-                    int resident_warps, int panel_ctas, int sched_mode, int cap_short, const SolveSplit &split,
+                    int resident_warps, const int (&panel_ctas)[2], int sched_mode, int cap_short, const SolveSplit &split,
                     int dense_min_rows, Schedule &W, bool defer_solve)
 {
     const int32_t n = S.n;
@@ -875,7 +893,9 @@ void build_schedule(const Pattern &P, const Structure &S, double alpha,
     // wait most (256 sets of the bordered 141x141 grid: 354 ms against 384 ms)
     const bool three = lng > 0.5 * outside || W.pull_cols > 0;
     W.smem = three ? kRefSmemThree : kRefSmemTwo;
-    build_panels(S, panel_ctas, !three, W);
+    // panels of wide columns hold kPullLd values per row of their scratch
+    W.pull_ld = 1;
+    build_panels(S, panel_ctas[three ? 1 : 0], !three, W);
     W.tb_nux.resize(W.tb_m);
     for (int32_t c = 0; c < W.tb_m; c++) {
         const int32_t *r = S.LUi.data() + S.LUp[W.tb_p + c];
@@ -891,7 +911,7 @@ void build_schedule(const Pattern &P, const Structure &S, double alpha,
     }
     const double thr = alpha * (double)resident_warps;
     W.thr = thr;
-    bool all_short = !W.pan.empty() && W.dense_m == 0;
+    bool all_short = !W.pan.empty() && W.dense_m == 0 && W.pull_cols == 0;
     for (int32_t k = 0; k < n && all_short; k++) all_short = S.LUp[k + 1] - S.LUp[k] <= cap_short;
     // ---- EGraph levels, the dividing level (Section IV-B) and the tasks:
     // on a thread of their own, beside the slot maps and row-wise copies
