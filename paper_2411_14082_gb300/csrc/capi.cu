@@ -1070,6 +1070,17 @@ int repredict(gblu_ctx *h, const double *Ax, cudaStream_t st, const std::vector<
     return GBLU_OK;
 }
 
+// Entries of the pool that a factorization of every step starts with: room
+// for the fill that exchanged rows add to the symmetric estimate, since a
+// pool that runs out costs a whole run (4,934 unknowns with 35 voltage
+// sources fill 1.35 times the estimate: 65 ms in two runs, 32 ms in one).
+// Beyond 32M entries (384 MB) a quarter more than the estimate.
+static size_t first_pool(const Pattern &P)
+{
+    const double est = 2.0 * (double)symmetric_fill(P) + (double)P.n;
+    return (size_t)std::max(1.25 * est, std::min(2.5 * est, (double)(32 << 20)));
+}
+
 // Every step recomputed by the pivoting kernel, preferring the rows
 // prefer[k] (the definition of a factorization with preferred pivots, used
 // when a re-prediction gives up)
@@ -1086,13 +1097,8 @@ int pivot_every_step(gblu_ctx *h, const double *Ax, cudaStream_t st, const std::
     h->S = std::move(E);
     CK(upload(h, h->piv, h->S.piv, st));
     CK(upload(h, h->pinv, h->S.pinv, st));
-    // room for the fill that exchanged rows add to the symmetric estimate: a
-    // pool that runs out costs a whole run (4,934 unknowns with 35 voltage
-    // sources fill 1.3 times the estimate: 69 ms in two runs, 36 ms in one)
-    const double est = 2.0 * (double)symmetric_fill(h->P) + (double)n;
-    const size_t hint = (size_t)std::max(1.25 * est, std::min(2.5 * est, (double)(32 << 20)));
     std::vector<uint8_t> all(n, 1);
-    return run_tail(h, Ax, st, all, hint, false, true);
+    return run_tail(h, Ax, st, all, first_pool(h->P), false, true);
 }
 
 // The pivot moves of a restart on a predicted structure, from the first
@@ -1470,9 +1476,8 @@ int gblu_factorize(gblu_handle h, const double *Ax_dev, void *stream)
         h->factorized = true;
         return GBLU_OK;
     }
-    const size_t hint = (size_t)(1.25 * (double)(2 * symmetric_fill(h->P) + n));
     std::vector<uint8_t> all(n, 1);
-    CK(run_tail(h, Ax_dev, st, all, hint, false, spec));
+    CK(run_tail(h, Ax_dev, st, all, first_pool(h->P), false, spec));
     h->factorized = true;
     return GBLU_OK;
 }
