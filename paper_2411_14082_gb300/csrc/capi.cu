@@ -130,6 +130,7 @@ struct gblu_ctx {
     DBuf<int32_t> tb_nux;
     DBuf<unsigned long long> tb_words;
     int32_t pscratch_ctas = 0;
+    bool lean = false;   // without panels: their workspaces did not fit
     // re-prediction: steps whose predicted row is not the preferred one, and
     // the pivot choice read back (step, non-finite flag)
     DBuf<uint8_t> strict;
@@ -376,6 +377,24 @@ static int upload_solve(gblu_ctx *h, cudaStream_t st, bool l_rows_done)
 // row pitch of the trailing block's matrix (values)
 static size_t block_pitch(int32_t m) { return ((size_t)m + 31) & ~(size_t)31; }
 
+// Gives up the panels and the trailing block of a handle, whose workspaces
+// did not fit: the next install_structure takes the columns one at a time
+static void make_lean(gblu_ctx *h, cudaStream_t st)
+{
+    cudaStreamSynchronize(st);   // uploads from the host vectors may be in flight
+    h->lean = true;
+    release(h, h->pscratch);
+    release(h, h->tb_S);
+    release(h, h->tb_words);
+    release(h, h->tb_nux);
+    release(h, h->pull_x);
+    release(h, h->pan);
+    release(h, h->prow);
+    release(h, h->pmask);
+    release(h, h->ppref);
+    release(h, h->prun);
+}
+
 // Install a factor structure: schedule on the host, arrays on the device.
 // values (optional) are the factor values in canonical order.  With
 // defer_solve only what the re-factorization reads is built and uploaded
@@ -392,7 +411,7 @@ int install_structure(gblu_ctx *h, Structure &&S, const std::vector<double> *val
     const auto t_s = std::chrono::steady_clock::now();
     int panel_ctas[2];
     for (int i = 0; i < 2; i++)
-        panel_ctas[i] =
+        panel_ctas[i] = h->lean ? 0 :
             std::max(h->ref_blocks_per_sm[i], std::max(h->batch_blocks_per_sm[i], h->ref32_blocks_per_sm[i])) * h->sm_count;
     build_schedule(h->P, h->S, h->opts.alpha, resident_warps, panel_ctas, h->opts.sched_mode, h->opts.warp_column_max, sp,
                    h->opts.dense_min_rows, h->W, defer_solve);
@@ -416,7 +435,13 @@ int install_structure(gblu_ctx *h, Structure &&S, const std::vector<double> *val
         const size_t bytes = (size_t)slots * (size_t)n * (ld * sizeof(double) + sizeof(unsigned long long));
         if (bytes <= kPullScratchBytes) {
             CK(upload(h, h->pull_start, h->W.pull_start, st));
-            CK(ensure(h, h->pull_x, (size_t)slots * n * ld));
+            const int px = ensure(h, h->pull_x, (size_t)slots * n * ld);
+            if (px != GBLU_OK) {
+                if (h->lean) return px;
+                make_lean(h, st);
+                Structure again = std::move(h->S);
+                return install_structure(h, std::move(again), values, st, defer_solve);
+            }
             CK(ensure(h, h->pull_tag, (size_t)slots * n));
             CK(ensure(h, h->pull_ctr, (size_t)slots));
             CK(ensure(h, h->pull_lock, (size_t)slots));
@@ -432,22 +457,26 @@ int install_structure(gblu_ctx *h, Structure &&S, const std::vector<double> *val
         CK(upload(h, h->ctask_cols, h->W.ctask_cols, st));
         CK(upload(h, h->camap, h->W.camap, st));
     }
-    CK(upload(h, h->pan, h->W.pan, st));
     CK(upload(h, h->pan_id, h->W.pan_id, st));
-    CK(upload(h, h->prow, h->W.prow, st));
-    CK(upload(h, h->pmask, h->W.pmask, st));
-    CK(upload(h, h->ppref, h->W.ppref, st));
-    CK(upload(h, h->prun, h->W.prun, st));
-    if (h->W.tb_m > 0) {
-        const size_t m = (size_t)h->W.tb_m;
+    h->pscratch_ctas = h->W.pscratch > 0 ? panel_ctas[cfg(h)] : 0;
+    const size_t m = (size_t)h->W.tb_m;
+    int room = upload(h, h->pan, h->W.pan, st);
+    if (room == GBLU_OK) room = upload(h, h->prow, h->W.prow, st);
+    if (room == GBLU_OK) room = upload(h, h->pmask, h->W.pmask, st);
+    if (room == GBLU_OK) room = upload(h, h->ppref, h->W.ppref, st);
+    if (room == GBLU_OK) room = upload(h, h->prun, h->W.prun, st);
+    if (m > 0 && room == GBLU_OK) {
         CK(upload(h, h->tb_nux, h->W.tb_nux, st));
-        CK(ensure(h, h->tb_S, m * block_pitch(h->W.tb_m)));
-        CK(ensure(h, h->tb_words, 2 * m + block_steps(h->W.tb_m)));
+        room = ensure(h, h->tb_S, m * block_pitch(h->W.tb_m));
+        if (room == GBLU_OK) room = ensure(h, h->tb_words, 2 * m + block_steps(h->W.tb_m));
     }
-    h->pscratch_ctas = 0;
-    if (h->W.pscratch > 0) {
-        h->pscratch_ctas = panel_ctas[cfg(h)];
-        CK(ensure(h, h->pscratch, (size_t)h->pscratch_ctas * (size_t)h->W.pscratch));
+    if (h->W.pscratch > 0 && room == GBLU_OK)
+        room = ensure(h, h->pscratch, (size_t)h->pscratch_ctas * (size_t)h->W.pscratch);
+    if (room != GBLU_OK) {
+        if (room != GBLU_ERR_NOMEM || h->lean) return room;
+        make_lean(h, st);
+        Structure again = std::move(h->S);
+        return install_structure(h, std::move(again), values, st, defer_solve);
     }
     CK(upload(h, h->dense_s0, h->W.dense_s0, st));
     if (h->W.dense_m > 0) CK(ensure(h, h->dense, (size_t)h->W.dense_m * h->W.dense_m));
@@ -1354,6 +1383,7 @@ int gblu_analyze(gblu_handle h, int32_t n, const int32_t *Ap, const int32_t *Ai,
     CK(upload(h, h->Aslot, P.Aslot, st));
     CK(ensure(h, h->partial, (size_t)3 * h->res_blocks));
     CU(cudaStreamSynchronize(st));
+    h->lean = false;
     h->analyzed = true;
     return GBLU_OK;
 }
@@ -2247,6 +2277,32 @@ int gblu_get_opts(gblu_handle h, gblu_opts *o)
     if (!h || !o) return fail(GBLU_ERR_INVALID_INPUT, "null pointer");
     *o = h->opts;
     return GBLU_OK;
+}
+
+// for callers with a memory budget (the server): the handle without its
+// panels' workspaces and without the room behind its factors
+int gblu_handle_lean(gblu_handle h, void *stream)
+{
+    CK(check_handle(h));
+    DeviceGuard g(h->device);
+    cudaStream_t st = (cudaStream_t)stream;
+    make_lean(h, st);
+    const size_t nnz = (size_t)h->S.nnz();
+    if (nnz > 0 && (h->rows.cap > nnz || h->vals.cap > nnz)) {
+        DBuf<int32_t> nr;
+        DBuf<double> nv;
+        if (ensure(h, nr, nnz) == GBLU_OK && ensure(h, nv, nnz) == GBLU_OK) {
+            CU(cudaMemcpyAsync(nr.p, h->rows.p, nnz * sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
+            CU(cudaMemcpyAsync(nv.p, h->vals.p, nnz * sizeof(double), cudaMemcpyDeviceToDevice, st));
+            CU(cudaStreamSynchronize(st));
+            std::swap(nr, h->rows);
+            std::swap(nv, h->vals);
+        }
+        release(h, nr);
+        release(h, nv);
+    }
+    Structure S = h->S;
+    return install_structure(h, std::move(S), nullptr, st);
 }
 
 int gblu_set_opts(gblu_handle h, const gblu_opts *o, void *stream)

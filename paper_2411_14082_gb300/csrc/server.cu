@@ -40,6 +40,9 @@
 
 #include "gblu.h"
 
+// capi.cu: a factorized handle rebuilt without panels and their workspaces
+extern "C" int gblu_handle_lean(gblu_handle h, void *stream);
+
 namespace {
 
 using Clock = std::chrono::steady_clock;
@@ -442,13 +445,20 @@ int gblu_server_add_pattern(gblu_server s, int32_t n, const int32_t *Ap, const i
     // of the batched refactor; intermediate vectors and sums of the solve
     const int64_t per_set = 8 * (p->nnz_a + p->lu_stride + 2 * (int64_t)n + 4) + 44 * (int64_t)n + 1024;
     int64_t avail;
-    {
+    auto fit = [&]() {
         std::lock_guard<std::mutex> lk(s->mu);
         // the handle, plus the single-precision workspace (float factors,
         // widened copy, refinement vectors) grown below
         avail = s->budget - s->reserved - hs.device_bytes - (12 * p->lu_stride + 32 * (int64_t)n);
+        p->slots = (int32_t)std::min<int64_t>(s->max_batch, avail > 0 ? avail / per_set : 0);
+    };
+    fit();
+    if (p->slots < 1) {   // without the panels' workspaces, which are only faster
+        if (gblu_handle_lean(p->h, p->st) == GBLU_OK) {
+            gblu_get_stats(p->h, &hs);
+            fit();
+        }
     }
-    p->slots = (int32_t)std::min<int64_t>(s->max_batch, avail > 0 ? avail / per_set : 0);
     if (p->slots < 1) {
         cudaFree(Ax0);
         return bail(sfail(GBLU_ERR_NOMEM, "server: pattern needs %lld + %lld bytes per set, %lld left in the budget",

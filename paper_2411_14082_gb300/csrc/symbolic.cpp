@@ -535,8 +535,8 @@ void build_solve_schedule(const Structure &S, const SolveSplit &split, Schedule 
 // Panels of the re-factorization (Schedule::pan): the columns of each
 // supernode of L whose neighbours also depend on one another, cut from the
 // lowest up.  kPanelMax columns while they have at most kPanelWideRows rows
-// below them and their union fits in a CTA's shared memory (1,167 slots),
-// else four, in shared memory (2,204 slots) or in a scratch of the CTA
+// below them and their union fits in a CTA's shared memory (1,197 slots),
+// else four, in shared memory (2,261 slots) or in a scratch of the CTA
 // (allow_scratch).  Wide columns and the dense
 // tail stay single.
 static void build_panels(const Structure &S, int panel_ctas, bool allow_scratch, Schedule &W)
@@ -549,7 +549,7 @@ static void build_panels(const Structure &S, int panel_ctas, bool allow_scratch,
     W.prun.clear();
     W.pan_id.assign(n, -1);
     W.pscratch = 0;
-    if (W.dense_m > 0 || n == 0) return;
+    if (W.dense_m > 0 || n == 0 || panel_ctas == 0) return;
     // link[j]: columns j and j+1 may share a panel; long chains are cut every
     // 64 columns, the units that the host threads share
     std::vector<uint8_t> link(n, 0);
@@ -846,7 +846,8 @@ void build_schedule(const Pattern &P, const Structure &S, double alpha,
     // have one pattern, so L's entries tell) without wide columns ----
     W.tb_p = n;
     W.tb_m = 0;
-    if (S.symmetric && W.dense_m == 0 && W.pull_cols == 0) {
+    const bool panels = panel_ctas[0] > 0;   // else the column kernels alone
+    if (panels && S.symmetric && W.dense_m == 0 && W.pull_cols == 0) {
         int64_t held = 0;
         for (int32_t p = n - 1; p >= 0 && n - p <= kBlockMax; p--) {
             held += S.LUp[p + 1] - S.LUp[p] - S.nU[p];
@@ -891,11 +892,11 @@ void build_schedule(const Pattern &P, const Structure &S, double alpha,
     // long columns, which are taken one at a time there (200x200x4 mesh: 74
     // ms against 87 ms with panels in scratches), and wide columns, which
     // wait most (256 sets of the bordered 141x141 grid: 354 ms against 384 ms)
-    const bool three = lng > 0.5 * outside || W.pull_cols > 0;
+    const bool three = lng > 0.5 * outside || W.pull_cols > 0 || !panels;
     W.smem = three ? kRefSmemThree : kRefSmemTwo;
     // panels of wide columns hold kPullLd values per row of their scratch
     W.pull_ld = 1;
-    build_panels(S, panel_ctas[three ? 1 : 0], !three, W);
+    build_panels(S, panel_ctas[three ? 1 : 0], !three, W);   // (none for 0 CTAs)
     W.tb_nux.resize(W.tb_m);
     for (int32_t c = 0; c < W.tb_m; c++) {
         const int32_t *r = S.LUi.data() + S.LUp[W.tb_p + c];

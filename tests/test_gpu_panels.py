@@ -110,3 +110,32 @@ def test_failed_check_inside_a_panel(col):
     assert np.array_equal(s.export_factors()["piv"], lu.piv)
     b = np.ones(n)
     assert O.residual(n, Ap, Ai, v, s.solve(dev(b)).cpu().numpy(), b) <= 1e-12
+
+
+def test_server_budget_without_room_for_panel_scratches():
+    """A budget that holds the factors but not the CTAs' scratches: the
+    pattern is taken without panels and gives the same bits."""
+    m, k, tail = 64, 45, 4   # dense blocks of m, a border of 4: one scratch panel
+    n = m * k + tail
+    rng = np.random.default_rng(5)
+    cols = [np.r_[(j // m) * m:(j // m) * m + m, n - tail:n] if j < m * k else np.arange(n) for j in range(n)]
+    Ap = np.r_[0, np.cumsum([len(c) for c in cols])].astype(np.int32)
+    Ai = np.concatenate(cols).astype(np.int32)
+    Ax = rng.uniform(-1.0, 1.0, len(Ai)) / n
+    Ax[Ai == np.repeat(np.arange(n), np.diff(Ap))] = 1.0
+    q = np.arange(n, dtype=np.int32)
+    s = gblu.Solver(DEV)
+    s.analyze(n, Ap, Ai, q)
+    s.factorize(dev(Ax))
+    full = s.stats()["device_bytes"]
+    v, b = Ax * rng.uniform(0.9, 1.0, len(Ax)), rng.uniform(-1.0, 1.0, n)
+    s.refactorize(dev(v))
+    want = s.solve(dev(b)).cpu().numpy()
+    budget = full - (10 << 20)
+    srv = gblu.Server(DEV, hbm_budget=budget, max_batch=1)
+    pid, slots = srv.add_pattern(n, Ap, Ai, q, Ax)
+    assert slots == 1 and srv.pattern_info(pid)["footprint_bytes"] <= budget
+    x = np.zeros(n)
+    srv.wait(srv.submit(pid, v, b, x))
+    srv.close()
+    assert np.array_equal(x, want)
