@@ -337,16 +337,35 @@ __device__ __forceinline__ bool panel_consume(R *X, bool in_smem, unsigned char 
     return true;
 }
 
+// Waits until the copies that producer warp p has started (fills of them) have
+// landed.  Only an aborted panel needs it: otherwise the consumers have waited
+// for every stage.  A copy in flight lands without anyone's help, so the limit
+// is a backstop.
+__device__ __forceinline__ void drain_slot(PanelBars &bars, int p, int fills, DevCtl *ctl)
+{
+    if (fills == 0) return;
+    const unsigned addr = smem_u32(&bars.full[p]), parity = (unsigned)(fills - 1) & 1u;
+    unsigned done = 0;
+    for (long long it = 0; !done && it < kBarTries; ++it)
+        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                     : "=r"(done)
+                     : "r"(addr), "r"(parity)
+                     : "memory");
+    if (!done) set_status(ctl, GBLU_ERR_DEVICE_TIMEOUT);
+}
+
 // the producers' part: warp p < ns fills slot p of the ring, stages p, p + ns,
 // ... (a slot belongs to one warp: a barrier's parity tells two successive
 // phases apart, so each phase has to be waited for in turn); false = gave up
-// (sh.abort set)
+// (sh.abort set).  Either way the last fill's copies may still be in flight:
+// fills = how many were started (drain_slot).
 template <typename R>
 __device__ __forceinline__ bool panel_produce(const RefactorArgsT<R> &a, const PanelRun *runs, int nruns,
                                               const int32_t *rows, int nu, int len, int k0, unsigned char *ring,
                                               int cap, int stage_bytes, int ns, PanelShared<R> &sh, PanelBars &bars,
-                                              int epoch, bool wait, int p, int lane)
+                                              int epoch, bool wait, int p, int lane, int &fills)
 {
+    fills = 0;
     if (p >= ns) return true;
     const R *const LUx = a.LUx;
     const int32_t *const LUi = a.LUi, *const nUp = a.nU, *const finish = a.finish;
@@ -361,19 +380,8 @@ __device__ __forceinline__ bool panel_produce(const RefactorArgsT<R> &a, const P
     RunWindow rw;
     rw.load(runs, 0, nruns, cap, 0, lane);
     int ready = 0;   // dependencies [0, ready) are known to be final
-    int fills = 0;
     auto give_up = [&]() -> bool {
         if (lane == 0) *abort = 1;
-        // this warp's copies in flight land before the CTA moves on
-        if (fills > 0) {
-            const unsigned addr = smem_u32(&bars.full[p]), parity = (unsigned)(fills - 1) & 1u;
-            unsigned done = 0;
-            for (long long it = 0; !done && it < kBarTries; ++it)
-                asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                             : "=r"(done)
-                             : "r"(addr), "r"(parity)
-                             : "memory");
-        }
         return false;
     };
     for (int s = p;; s += ns) {
@@ -755,15 +763,24 @@ __device__ __noinline__ bool col_panel(const RefactorArgsT<R> *ap, int id, unsig
         }
     }
     const int nruns = (blk ? p.nrunsx : p.nruns) - run0;
+    int fills = 0;
     if (nruns > 0) {
         const PanelRun *runs = a.prun + p.roff + run0;
         if (warp < kConsWarps)
             go = panel_consume<R, LD>(X, in_smem, smem, stage_bytes, ns, sh, bars, a.ctl, warp, lane);
         else
             go = panel_produce<R>(a, runs, nruns, rows, nux, len, k0, smem, cap, stage_bytes, ns, sh, bars, epoch, wait,
-                                  warp - kConsWarps, lane);
+                                  warp - kConsWarps, lane, fills);
     }
-    if (__syncthreads_or(!go)) return true;
+    if (__syncthreads_or(!go)) {
+        // the one way out of an aborted panel.  Every producer waits for its
+        // own copies, also one that had started its last stage when another
+        // gave up: the CTA's next panel re-initializes the barriers and fills
+        // the ring's memory, and a CTA must not exit before they land.
+        if (warp >= kConsWarps) drain_slot(bars, warp - kConsWarps, fills, a.ctl);
+        __syncthreads();
+        return true;
+    }
 
     const int64_t lup = lane < nc ? __ldg(LUp + k0 + lane) : 0;   // lane c: column c
     if (blk) {   // the block's rows go to the dense matrix
