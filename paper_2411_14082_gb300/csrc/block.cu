@@ -16,9 +16,10 @@
 // device.  Every value gets the same multiply-adds in the same (ascending)
 // order as in the column kernels: the factors are the same bits.
 // The last launch checks every pivot against its column's largest candidate,
-// stores the block's entries in the factor's columns and publishes them; a
-// failed check sets `interrupted`, and the caller re-factorizes column by
-// column to find the first failing step.
+// stores the entries of the columns that pass in the factor's columns and
+// publishes them.  The columns before the first failing one were computed
+// from passing pivots alone, so first_bad is exact; the failing columns stay
+// unpublished, and the restart computes them again.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -256,7 +257,9 @@ __global__ void __launch_bounds__(256) block_finish_kernel(BlockArgs a)
 {
     const int c = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
     if (c >= a.m) return;
-    if (ld_volatile(&a.ctl->interrupted) || ld_volatile(&a.ctl->status)) return;
+    // a check that failed before the block (one in the block is not a reason
+    // to leave: every column is judged by itself)
+    if (ld_volatile(&a.ctl->first_bad) < a.p || ld_volatile(&a.ctl->status)) return;
     const int k = a.p + c;
     const double d = __ldcg(a.S + (int64_t)c * a.ld + c);
     const double m = __longlong_as_double((long long)__ldcg(a.colmax + c));

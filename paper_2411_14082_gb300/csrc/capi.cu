@@ -592,8 +592,8 @@ RefactorArgs refactor_args(gblu_ctx *h, const double *Ax)
 // the launches of one checked re-factorization; ep = the epoch the kernels
 // store in the ready flags, or -1: read it from the control block (graph
 // replay, where the epoch changes between launches of the same graph)
-// block: the trailing block densely (block.cu).  A check that fails then
-// only says that some check fails.
+// block: the trailing block densely (block.cu), stopping at a failed check
+// whatever the caller's mode.
 int issue_refactor(gblu_ctx *h, const double *Ax, cudaStream_t st, int ep, bool block = false)
 {
     KL(launch_begin_refactor(h->ctl, st));
@@ -671,28 +671,25 @@ int issue_refactor(gblu_ctx *h, const double *Ax, cudaStream_t st, int ep, bool 
 // column by column (a forced failure, a re-prediction's strict columns)
 static bool block_applies(const gblu_ctx *h) { return h->W.tb_m > 0 && h->force_col < 0 && !h->strict_on; }
 
+int restart_on_structure(gblu_ctx *h, const double *Ax, cudaStream_t st, bool no_stop, int *interrupted);
+
 // A deferred install's solve part is finished on the host while the
 // re-factorization runs.
 int run_refactor(gblu_ctx *h, const double *Ax, cudaStream_t st, int *interrupted)
 {
-    if (block_applies(h)) {
-        h->epoch++;
-        CK(issue_refactor(h, Ax, st, h->epoch, true));
-        CK(finish_install(h, st));
-        CK(read_ctl(h, st));
-        CK(status_code(h));
-        if (!h->hctl->interrupted) {
-            *interrupted = 0;
-            h->last_first_bad = -1;
-            return GBLU_OK;
-        }
-        // a check failed: column by column, in the caller's mode
-    }
+    const bool block = block_applies(h);
     h->epoch++;
-    CK(issue_refactor(h, Ax, st, h->epoch));
+    CK(issue_refactor(h, Ax, st, h->epoch, block));
     CK(finish_install(h, st));
     CK(read_ctl(h, st));
     CK(status_code(h));
+    // a no-stop caller wants the column that failed unnormalized and
+    // first_bad exact: the pass with the block stopped, and the columns that
+    // it did not finish follow
+    if (block && h->no_stop && h->hctl->interrupted) {
+        int any = 0;
+        CK(restart_on_structure(h, Ax, st, true, &any));
+    }
     *interrupted = h->hctl->interrupted;
     h->last_first_bad = h->hctl->interrupted ? h->hctl->first_bad : -1;
     return GBLU_OK;
@@ -2136,16 +2133,8 @@ int gblu_step(gblu_handle h, const double *Ax_dev, const double *b_dev, double *
     h->last_first_bad = h->hctl->interrupted ? h->hctl->first_bad : -1;
     if (!h->hctl->interrupted) return GBLU_OK;
     // the check failed: the solve of the replay is void; restart, solve again
-    // (with a trailing block, the first failing step is not known yet)
-    int rc = GBLU_OK;
-    if (block_applies(h)) {
-        h->n_refactor--;
-        rc = gblu_refactorize(h, h->stage_ax.p, stream, nullptr);
-        if (rc == GBLU_REPIVOTED) rc = GBLU_OK;
-    } else {
-        h->n_repivot++;
-        rc = run_restart(h, h->stage_ax.p, st);
-    }
+    h->n_repivot++;
+    const int rc = run_restart(h, h->stage_ax.p, st);
     if (rc != GBLU_OK) {
         h->factorized = false;
         return rc;

@@ -1,0 +1,62 @@
+"""A check that fails on a structure with a trailing block: one pass with the
+block finds the first failing step, and the restart goes on from the columns
+that passed, through gblu_refactorize and through a replayed gblu_step."""
+import numpy as np
+import pytest
+
+from oracle import oracle as O
+from paper_2411_14082_gb300 import gblu
+from tests.factor_compare import compare_factors
+from tests.test_gpu_panel_abort import band, dev, with_failing_pivot
+
+pytestmark = pytest.mark.gpu
+
+DEV = 0
+
+
+def solver(sys_):
+    n, Ap, Ai, Ax0, Q = sys_
+    s = gblu.Solver(DEV)
+    s.analyze(n, Ap, Ai, Q)
+    s.factorize(dev(Ax0))
+    return s
+
+
+def launches(s, call):
+    before = s.stats()["kernel_launches"]
+    out = call()
+    return s.stats()["kernel_launches"] - before, out
+
+
+# 200 dense last rows and columns, the block, behind too few columns for any
+# to be a wide one
+@pytest.mark.parametrize("k", [100, 220, 390])
+def test_a_failed_check_costs_one_pass_with_the_block(k):
+    n, Ap, Ai, Ax0, Q = band(400, 30, 200, 3)
+    for r, c in ((k, k + 1), (k + 1, k)):   # steps k and k + 1 exchange rows and no other step moves
+        Ax0[Ap[c] + int(np.searchsorted(Ai[Ap[c]:Ap[c + 1]], r))] = 0.9
+    sys_ = n, Ap, Ai, Ax0, Q
+    rng = np.random.default_rng(2)
+    lu0 = O.factorize(n, Ap, Ai, Ax0, Q, 1e-3)
+    v = Ax0 * rng.uniform(0.98, 1.02, len(Ax0))
+    w = with_failing_pivot(n, Ap, Ai, v, Q, lu0, k)
+    lu = O.refactorize(lu0, Ap, Ai, w)
+    assert np.nonzero(lu.piv != lu0.piv)[0].tolist() == [k, k + 1]
+    b = rng.uniform(-1.0, 1.0, n)
+    g, p = solver(sys_), solver(sys_)
+    ok_pass, (_, rep) = launches(p, lambda: p.refactorize(dev(v)))
+    assert not rep and ok_pass > 13   # a block of 200 columns takes 13 launches of its own
+    solve, _ = launches(p, lambda: p.solve(dev(b)))
+    replay, (_, rep) = launches(g, lambda: g.step(dev(v), dev(b)))
+    assert not rep and replay == ok_pass + solve
+    bad_pass, (_, rep) = launches(p, lambda: p.refactorize(dev(w)))
+    assert rep and p.stats()["last_first_bad"] == k
+    bad_step, (x, rep) = launches(g, lambda: g.step(dev(w), dev(b)))
+    assert rep and g.stats()["last_first_bad"] == k
+    # the failed replay stands for the first pass; what the restart adds is
+    # the same through both calls
+    assert bad_step - replay - solve == bad_pass - ok_pass
+    for s in (g, p):
+        compare_factors(s.export_factors(), lu, 1e-10)
+        assert s.stats()["n_repivot"] == 1 and s.stats()["n_refactor"] == 2
+    assert O.residual(n, Ap, Ai, w, x.cpu().numpy(), b) <= 1e-12
