@@ -874,8 +874,8 @@ int run_tail(gblu_ctx *h, const double *Ax, cudaStream_t st, const std::vector<u
             if (!bits_smem) CU(cudaMemsetAsync(h->sbits.p, 0, (size_t)slots * words * sizeof(unsigned), st));
             t.seq = h->seq.p;
         }
-        if (pool_full) {
-            pool *= 2;
+        if (pool_full) {   // twice what was tried: all that the buffers hold
+            pool = 2 * std::max(pool, std::min(h->rows.cap, h->vals.cap) - (size_t)nnz);
             CK(upload(h, h->seq, seq, st));
             continue;
         }
