@@ -377,8 +377,8 @@ static int upload_solve(gblu_ctx *h, cudaStream_t st, bool l_rows_done)
 // row pitch of the trailing block's matrix (values)
 static size_t block_pitch(int32_t m) { return ((size_t)m + 31) & ~(size_t)31; }
 
-// Gives up the panels and the trailing block of a handle, whose workspaces
-// did not fit: the next install_structure takes the columns one at a time
+// Gives up the panels and the trailing block of a handle: the next
+// install_structure takes the columns one at a time.
 static void make_lean(gblu_ctx *h, cudaStream_t st)
 {
     cudaStreamSynchronize(st);   // uploads from the host vectors may be in flight
@@ -393,6 +393,26 @@ static void make_lean(gblu_ctx *h, cudaStream_t st)
     release(h, h->pmask);
     release(h, h->ppref);
     release(h, h->prun);
+    release(h, h->ctask_ptr);
+    release(h, h->ctask_cols);
+    release(h, h->camap);
+}
+
+// Frees the factors' buffers if they hold room for a pool behind the nnz
+// entries of a structure; the next install_structure allocates those alone.
+// alive: their first nnz values are the factors, which go to *kept.
+static int drop_spare(gblu_ctx *h, size_t nnz, bool alive, std::vector<double> *kept, cudaStream_t st, bool *dropped)
+{
+    *dropped = h->rows.cap > nnz || h->vals.cap > nnz;
+    if (!*dropped) return GBLU_OK;
+    if (alive) {
+        kept->resize(nnz);
+        CU(cudaMemcpyAsync(kept->data(), h->vals.p, nnz * sizeof(double), cudaMemcpyDeviceToHost, st));
+    }
+    CU(cudaStreamSynchronize(st));
+    release(h, h->rows);
+    release(h, h->vals);
+    return GBLU_OK;
 }
 
 // Install a factor structure: schedule on the host, arrays on the device.
@@ -400,8 +420,7 @@ static void make_lean(gblu_ctx *h, cudaStream_t st)
 // defer_solve only what the re-factorization reads is built and uploaded
 // (nothing synchronizes); finish_install adds the rest, on the host while
 // the stream runs the re-factorization.
-int install_structure(gblu_ctx *h, Structure &&S, const std::vector<double> *values, cudaStream_t st,
-                      bool defer_solve = false)
+static int try_install(gblu_ctx *h, Structure &&S, const std::vector<double> *values, cudaStream_t st, bool defer_solve)
 {
     h->S = std::move(S);
     h->struct_version++;
@@ -435,13 +454,7 @@ int install_structure(gblu_ctx *h, Structure &&S, const std::vector<double> *val
         const size_t bytes = (size_t)slots * (size_t)n * (ld * sizeof(double) + sizeof(unsigned long long));
         if (bytes <= kPullScratchBytes) {
             CK(upload(h, h->pull_start, h->W.pull_start, st));
-            const int px = ensure(h, h->pull_x, (size_t)slots * n * ld);
-            if (px != GBLU_OK) {
-                if (h->lean) return px;
-                make_lean(h, st);
-                Structure again = std::move(h->S);
-                return install_structure(h, std::move(again), values, st, defer_solve);
-            }
+            CK(ensure(h, h->pull_x, (size_t)slots * n * ld));
             CK(ensure(h, h->pull_tag, (size_t)slots * n));
             CK(ensure(h, h->pull_ctr, (size_t)slots));
             CK(ensure(h, h->pull_lock, (size_t)slots));
@@ -460,24 +473,17 @@ int install_structure(gblu_ctx *h, Structure &&S, const std::vector<double> *val
     CK(upload(h, h->pan_id, h->W.pan_id, st));
     h->pscratch_ctas = h->W.pscratch > 0 ? panel_ctas[cfg(h)] : 0;
     const size_t m = (size_t)h->W.tb_m;
-    int room = upload(h, h->pan, h->W.pan, st);
-    if (room == GBLU_OK) room = upload(h, h->prow, h->W.prow, st);
-    if (room == GBLU_OK) room = upload(h, h->pmask, h->W.pmask, st);
-    if (room == GBLU_OK) room = upload(h, h->ppref, h->W.ppref, st);
-    if (room == GBLU_OK) room = upload(h, h->prun, h->W.prun, st);
-    if (m > 0 && room == GBLU_OK) {
+    CK(upload(h, h->pan, h->W.pan, st));
+    CK(upload(h, h->prow, h->W.prow, st));
+    CK(upload(h, h->pmask, h->W.pmask, st));
+    CK(upload(h, h->ppref, h->W.ppref, st));
+    CK(upload(h, h->prun, h->W.prun, st));
+    if (m > 0) {
         CK(upload(h, h->tb_nux, h->W.tb_nux, st));
-        room = ensure(h, h->tb_S, m * block_pitch(h->W.tb_m));
-        if (room == GBLU_OK) room = ensure(h, h->tb_words, 2 * m + block_steps(h->W.tb_m));
+        CK(ensure(h, h->tb_S, m * block_pitch(h->W.tb_m)));
+        CK(ensure(h, h->tb_words, 2 * m + block_steps(h->W.tb_m)));
     }
-    if (h->W.pscratch > 0 && room == GBLU_OK)
-        room = ensure(h, h->pscratch, (size_t)h->pscratch_ctas * (size_t)h->W.pscratch);
-    if (room != GBLU_OK) {
-        if (room != GBLU_ERR_NOMEM || h->lean) return room;
-        make_lean(h, st);
-        Structure again = std::move(h->S);
-        return install_structure(h, std::move(again), values, st, defer_solve);
-    }
+    if (h->W.pscratch > 0) CK(ensure(h, h->pscratch, (size_t)h->pscratch_ctas * (size_t)h->W.pscratch));
     CK(upload(h, h->dense_s0, h->W.dense_s0, st));
     if (h->W.dense_m > 0) CK(ensure(h, h->dense, (size_t)h->W.dense_m * h->W.dense_m));
     CK(upload(h, h->piv, h->S.piv, st));
@@ -516,6 +522,33 @@ int install_structure(gblu_ctx *h, Structure &&S, const std::vector<double> *val
     return GBLU_OK;
 }
 
+int install_structure(gblu_ctx *h, Structure &&S, const std::vector<double> *values, cudaStream_t st,
+                      bool defer_solve = false)
+{
+    int rc = try_install(h, std::move(S), values, st, defer_solve);
+    // without room: once more without the pool behind the factors, then
+    // without what only makes the re-factorization faster
+    std::vector<double> kept;
+    for (int step = 0; step < 2 && rc == GBLU_ERR_NOMEM; step++) {
+        cudaStreamSynchronize(st);
+        if (step == 0) {
+            bool dropped = false;
+            const bool alive = !values && !defer_solve;
+            CK(drop_spare(h, (size_t)h->S.nnz(), alive, &kept, st, &dropped));
+            if (!dropped) continue;
+            if (alive) values = &kept;
+        } else {
+            if (h->lean) break;
+            make_lean(h, st);
+        }
+        Structure again = std::move(h->S);
+        rc = try_install(h, std::move(again), values, st, defer_solve);
+    }
+    // uploads from `kept` are stream-ordered copies of pageable memory
+    if (!kept.empty()) CU(cudaStreamSynchronize(st));
+    return rc;
+}
+
 // The solve part of a deferred install_structure: built on the host (while
 // the stream may still run a re-factorization, which does not read it),
 // then uploaded behind the work on the stream.
@@ -528,8 +561,21 @@ int finish_install(gblu_ctx *h, cudaStream_t st)
     h->t_tail[2] += std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t_s).count();
     // its uploads wait behind the stream's work, so their time is the
     // caller's (the re-factorization's), not tail_upload_ms
-    CK(upload_solve(h, st, l_rows_done));
     h->solve_pending = false;
+    const int rc = upload_solve(h, st, l_rows_done);
+    if (rc != GBLU_ERR_NOMEM) return rc;
+    // without room: the whole structure once more (install_structure gives
+    // up what it can) around the values and ready flags that the
+    // re-factorization leaves
+    std::vector<double> vals((size_t)h->S.nnz());
+    std::vector<int32_t> fin(h->S.n);
+    CU(cudaMemcpyAsync(vals.data(), h->vals.p, vals.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
+    CU(cudaMemcpyAsync(fin.data(), h->finish.p, fin.size() * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+    CU(cudaStreamSynchronize(st));
+    Structure again = std::move(h->S);
+    CK(install_structure(h, std::move(again), &vals, st));
+    CU(cudaMemcpyAsync(h->finish.p, fin.data(), fin.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st));
+    CU(cudaStreamSynchronize(st));
     return GBLU_OK;
 }
 
@@ -695,13 +741,17 @@ int run_refactor(gblu_ctx *h, const double *Ax, cudaStream_t st, int *interrupte
     return GBLU_OK;
 }
 
+struct PoolHint { size_t want = 0, least = 0; };   // entries (run_tail)
+
 // Factorization with threshold pivoting of the steps in rmask (Algorithm 5;
 // Algorithm 1 when rmask holds every step); the other steps keep their
 // current columns.  Rebuilds the structure and the schedule afterwards.
 // speculate: passes predict that every step takes its preferred row;
 // keep_if_same: a restart, whose structure stays when every pivot is kept.
-int run_tail(gblu_ctx *h, const double *Ax, cudaStream_t st, const std::vector<uint8_t> &rmask,
-             size_t pool_hint, bool keep_if_same, bool speculate)
+// The pool starts with room for hint.want entries, or for hint.least where
+// the device has no room for those.
+static int try_tail(gblu_ctx *h, const double *Ax, cudaStream_t st, const std::vector<uint8_t> &rmask, PoolHint hint,
+                    bool keep_if_same, bool speculate)
 {
     const Pattern &P = h->P;
     const int32_t n = P.n;
@@ -749,9 +799,9 @@ int run_tail(gblu_ctx *h, const double *Ax, cudaStream_t st, const std::vector<u
     if (!bits_smem) CK(ensure(h, h->sbits, (size_t)slots * words));
     // pool after the canonical columns
     // speculative restarts may write a column once per pass
-    size_t pool = std::max<size_t>(pool_hint, (size_t)std::max<int64_t>((speculate ? 4 : 2) * restart_len,
-                                                                        (int64_t)P.Ai.size())) +
-                  (size_t)n;
+    const size_t floor = (size_t)std::max<int64_t>((speculate ? 4 : 2) * restart_len, (int64_t)P.Ai.size());
+    size_t pool = std::max(hint.want, floor) + (size_t)n;
+    const size_t least = std::max(hint.least, floor) + (size_t)n;
     using TClock = std::chrono::steady_clock;
     auto ms_since = [](TClock::time_point t) {
         return std::chrono::duration<double, std::milli>(TClock::now() - t).count();
@@ -764,8 +814,15 @@ int run_tail(gblu_ctx *h, const double *Ax, cudaStream_t st, const std::vector<u
             // grow, keeping the canonical region
             DBuf<int32_t> nr;
             DBuf<double> nv;
-            CK(ensure(h, nr, need));
-            CK(ensure(h, nv, need));
+            int room = ensure(h, nr, need);
+            if (room == GBLU_OK) room = ensure(h, nv, need);
+            if (room != GBLU_OK) {
+                release(h, nr);
+                if (attempt > 0 || pool <= least) return room;
+                pool = least;
+                attempt--;
+                continue;
+            }
             if (nnz > 0) {
                 CU(cudaMemcpyAsync(nr.p, h->rows.p, nnz * sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
                 CU(cudaMemcpyAsync(nv.p, h->vals.p, nnz * sizeof(double), cudaMemcpyDeviceToDevice, st));
@@ -988,6 +1045,22 @@ int run_tail(gblu_ctx *h, const double *Ax, cudaStream_t st, const std::vector<u
     return GBLU_OK;
 }
 
+int run_tail(gblu_ctx *h, const double *Ax, cudaStream_t st, const std::vector<uint8_t> &rmask, PoolHint hint,
+             bool keep_if_same, bool speculate)
+{
+    const int rc = try_tail(h, Ax, st, rmask, hint, keep_if_same, speculate);
+    const size_t before = h->device_bytes;
+    if (rc != GBLU_ERR_NOMEM || h->lean) return rc;
+    // without room beside the panels of the installed structure: without them
+    make_lean(h, st);
+    if (h->device_bytes == before) return rc;
+    if (h->S.nnz() > 0) {
+        Structure again = std::move(h->S);
+        CK(install_structure(h, std::move(again), nullptr, st));
+    }
+    return try_tail(h, Ax, st, rmask, hint, keep_if_same, speculate);
+}
+
 // Restart (Section IV-C): every column that did not finish in this
 // re-factorization, and all of its column-elimination-tree ancestors, is
 // recomputed with pivoting.
@@ -1096,15 +1169,15 @@ int repredict(gblu_ctx *h, const double *Ax, cudaStream_t st, const std::vector<
     return GBLU_OK;
 }
 
-// Entries of the pool that a factorization of every step starts with: room
-// for the fill that exchanged rows add to the symmetric estimate, since a
-// pool that runs out costs a whole run (4,934 unknowns with 35 voltage
-// sources fill 1.35 times the estimate: 65 ms in two runs, 32 ms in one).
-// Beyond 32M entries (384 MB) a quarter more than the estimate.
-static size_t first_pool(const Pattern &P)
+// The pool that a factorization of every step starts with: room for the fill
+// that exchanged rows add to the symmetric estimate, since a pool that runs
+// out costs a whole run (4,934 unknowns with 35 voltage sources fill 1.35
+// times the estimate: 65 ms in two runs, 32 ms in one).  Beyond 32M entries
+// (384 MB), or without room for that many, a quarter more than the estimate.
+static PoolHint first_pool(const Pattern &P)
 {
-    const double est = 2.0 * (double)symmetric_fill(P) + (double)P.n;
-    return (size_t)std::max(1.25 * est, std::min(2.5 * est, (double)(32 << 20)));
+    const double est = 2.0 * (double)symmetric_fill(P) + (double)P.n, least = 1.25 * est;
+    return {(size_t)std::max(least, std::min(2.5 * est, (double)(32 << 20))), (size_t)least};
 }
 
 // Every step recomputed by the pivoting kernel, preferring the rows
@@ -1177,7 +1250,7 @@ int run_restart(gblu_ctx *h, const double *Ax, cudaStream_t st)
     std::vector<uint8_t> finished(n), rmask(n);
     for (int32_t k = 0; k < n; k++) finished[k] = fin[k] == h->epoch;
     gblu_restart_set(n, h->P.cetree.data(), finished.data(), rmask.data());
-    return run_tail(h, Ax, st, rmask, 0, true, true);
+    return run_tail(h, Ax, st, rmask, PoolHint{}, true, true);
 }
 
 int check_handle(gblu_ctx *h)
@@ -1483,7 +1556,7 @@ int gblu_factorize(gblu_handle h, const double *Ax_dev, void *stream)
             std::vector<uint8_t> finished(n), rmask(n);
             for (int32_t k = 0; k < n; k++) finished[k] = fin[k] == h->epoch;
             gblu_restart_set(n, h->P.cetree.data(), finished.data(), rmask.data());
-            CK(run_tail(h, Ax_dev, st, rmask, 0, true, true));
+            CK(run_tail(h, Ax_dev, st, rmask, PoolHint{}, true, true));
             h->first_mode = 2;
         } else if (repred && h->hctl->first_bad != INT_MAX) {
             h->last_first_bad = h->hctl->first_bad;
@@ -2276,22 +2349,13 @@ int gblu_handle_lean(gblu_handle h, void *stream)
     DeviceGuard g(h->device);
     cudaStream_t st = (cudaStream_t)stream;
     make_lean(h, st);
-    const size_t nnz = (size_t)h->S.nnz();
-    if (nnz > 0 && (h->rows.cap > nnz || h->vals.cap > nnz)) {
-        DBuf<int32_t> nr;
-        DBuf<double> nv;
-        if (ensure(h, nr, nnz) == GBLU_OK && ensure(h, nv, nnz) == GBLU_OK) {
-            CU(cudaMemcpyAsync(nr.p, h->rows.p, nnz * sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
-            CU(cudaMemcpyAsync(nv.p, h->vals.p, nnz * sizeof(double), cudaMemcpyDeviceToDevice, st));
-            CU(cudaStreamSynchronize(st));
-            std::swap(nr, h->rows);
-            std::swap(nv, h->vals);
-        }
-        release(h, nr);
-        release(h, nv);
-    }
-    Structure S = h->S;
-    return install_structure(h, std::move(S), nullptr, st);
+    std::vector<double> kept;
+    bool dropped = false;
+    CK(drop_spare(h, (size_t)h->S.nnz(), true, &kept, st, &dropped));
+    Structure S = std::move(h->S);
+    const int rc = install_structure(h, std::move(S), dropped ? &kept : nullptr, st);
+    CU(cudaStreamSynchronize(st));   // kept is in use
+    return rc;
 }
 
 int gblu_set_opts(gblu_handle h, const gblu_opts *o, void *stream)
