@@ -2341,17 +2341,33 @@ int gblu_get_opts(gblu_handle h, gblu_opts *o)
     return GBLU_OK;
 }
 
-// for callers with a memory budget (the server): the handle without its
-// panels' workspaces and without the room behind its factors
-int gblu_handle_lean(gblu_handle h, void *stream)
+// for callers with a memory budget (the server): the bytes that a factorized
+// handle could give up, behind its factors (*pool) and as panels' workspaces
+int gblu_handle_spare(gblu_handle h, int64_t *pool, int64_t *panels)
+{
+    CK(check_handle(h));
+    const int64_t nnz = std::max<int64_t>(h->S.nnz(), 1);
+    *pool = 4 * std::max<int64_t>((int64_t)h->rows.cap - nnz, 0) + 8 * std::max<int64_t>((int64_t)h->vals.cap - nnz, 0);
+    *panels = 0;
+    if (h->lean) return GBLU_OK;
+    auto add = [&](const auto &b) { *panels += (int64_t)(b.cap * sizeof(*b.p)); };
+    add(h->pscratch); add(h->tb_S); add(h->tb_words); add(h->tb_nux); add(h->pan); add(h->prow); add(h->pmask);
+    add(h->ppref); add(h->prun); add(h->ctask_ptr); add(h->ctask_cols); add(h->camap);
+    if (h->W.pull_ld > 0) *panels += (int64_t)(h->pull_x.cap / h->W.pull_ld * (h->W.pull_ld - 1) * sizeof(double));
+    return GBLU_OK;
+}
+
+// ... without the pool behind its factors and, with lean, without its panels
+int gblu_handle_shrink(gblu_handle h, int lean, void *stream)
 {
     CK(check_handle(h));
     DeviceGuard g(h->device);
     cudaStream_t st = (cudaStream_t)stream;
-    make_lean(h, st);
+    if (lean) make_lean(h, st);
     std::vector<double> kept;
     bool dropped = false;
     CK(drop_spare(h, (size_t)h->S.nnz(), true, &kept, st, &dropped));
+    if (!lean && !dropped) return GBLU_OK;
     Structure S = std::move(h->S);
     const int rc = install_structure(h, std::move(S), dropped ? &kept : nullptr, st);
     CU(cudaStreamSynchronize(st));   // kept is in use

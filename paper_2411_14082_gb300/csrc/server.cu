@@ -40,8 +40,9 @@
 
 #include "gblu.h"
 
-// capi.cu: a factorized handle rebuilt without panels and their workspaces
-extern "C" int gblu_handle_lean(gblu_handle h, void *stream);
+// capi.cu: what a factorized handle could give up, and the handle without it
+extern "C" int gblu_handle_spare(gblu_handle h, int64_t *pool, int64_t *panels);
+extern "C" int gblu_handle_shrink(gblu_handle h, int lean, void *stream);
 
 namespace {
 
@@ -98,6 +99,8 @@ struct Pattern {
     std::thread worker;
     int64_t batches = 0, requests = 0, repivots = 0;
     int32_t max_batch_seen = 0;
+    bool shrink = false;   // asked to give up what its handle can do without,
+    int64_t spare = 0;     // this many bytes when the pattern was added
 };
 
 }  // namespace
@@ -132,6 +135,17 @@ void free_pattern(Pattern *p)
     if (p->st) cudaStreamDestroy(p->st);
     p->Ax_d = p->LU_d = p->b_d = p->x_d = p->res_d = p->res_h = nullptr;
     p->st = nullptr;
+}
+
+// the handle without the pool behind its factors and without its panels
+// (by the thread that uses the handle); false: it cannot serve any more
+bool shrink_handle(Pattern *p, gblu_stats *hs)
+{
+    int64_t pool = 0, panels = 0;
+    gblu_handle_spare(p->h, &pool, &panels);
+    const bool ok = pool + panels == 0 || gblu_handle_shrink(p->h, 1, p->st) == GBLU_OK;
+    gblu_get_stats(p->h, hs);
+    return ok;
 }
 
 int64_t server_buffer_bytes(const Pattern *p)
@@ -276,11 +290,18 @@ void run_batch(gblu_server_s *s, Pattern *p, std::vector<Request *> &batch)
             p->LU_d = nullptr;
             const int64_t old = p->footprint;
             p->lu_stride = hs.nnz_l + hs.nnz_u;
-            std::lock_guard<std::mutex> lk(s->mu);
-            // keep within the budget by dropping slots if needed (at least one)
-            while (p->slots > 1 &&
-                   s->reserved - old + hs.device_bytes + server_buffer_bytes(p) > s->budget)
-                p->slots--;
+            std::unique_lock<std::mutex> lk(s->mu);
+            auto over = [&] {
+                return s->reserved - old + hs.device_bytes + server_buffer_bytes(p) > s->budget;
+            };
+            // keep within the budget: without what the handle can give up,
+            // then by dropping slots (at least one stays)
+            if (p->slots > 1 && over()) {
+                lk.unlock();
+                shrink_handle(p, &hs);
+                lk.lock();
+            }
+            while (p->slots > 1 && over()) p->slots--;
             if (cudaMalloc(&p->LU_d, (size_t)p->slots * p->lu_stride * sizeof(double)) != cudaSuccess) {
                 cudaGetLastError();
                 p->slots = 0;   // the pattern cannot serve further requests
@@ -316,7 +337,21 @@ void worker_loop(gblu_server_s *s, Pattern *p)
     for (;;) {
         {
             std::unique_lock<std::mutex> lk(s->mu);
-            p->cv.wait(lk, [&] { return s->stop || !p->queue.empty(); });
+            p->cv.wait(lk, [&] { return s->stop || p->shrink || !p->queue.empty(); });
+            if (p->shrink) {   // another pattern needs the room
+                lk.unlock();
+                gblu_stats hs{};
+                const bool ok = shrink_handle(p, &hs);
+                lk.lock();
+                if (!ok) p->slots = 0;   // the pattern cannot serve further requests
+                const int64_t old = p->footprint;
+                p->footprint = hs.device_bytes + server_buffer_bytes(p);
+                s->reserved += p->footprint - old;
+                p->shrink = false;
+                p->spare = 0;
+                s->cv_done.notify_all();
+                continue;
+            }
             if (p->queue.empty()) return;   // stopping and drained
             batch.clear();
             const size_t cap = (size_t)std::max(p->slots, 0);
@@ -444,20 +479,57 @@ int gblu_server_add_pattern(gblu_server s, int32_t n, const int32_t *Ap, const i
     // handle growth per batch set: ready flags, control block and arguments
     // of the batched refactor; intermediate vectors and sums of the solve
     const int64_t per_set = 8 * (p->nnz_a + p->lu_stride + 2 * (int64_t)n + 4) + 44 * (int64_t)n + 1024;
-    int64_t avail;
-    auto fit = [&]() {
-        std::lock_guard<std::mutex> lk(s->mu);
-        // the handle, plus the single-precision workspace (float factors,
-        // widened copy, refinement vectors) grown below
-        avail = s->budget - s->reserved - hs.device_bytes - (12 * p->lu_stride + 32 * (int64_t)n);
-        p->slots = (int32_t)std::min<int64_t>(s->max_batch, avail > 0 ? avail / per_set : 0);
+    // sets that fit beside the handle when it gives up `less` bytes, with the
+    // single-precision workspace (float factors, widened copy, refinement
+    // vectors) grown below
+    int64_t avail = 0;
+    auto sets = [&](int64_t less) {
+        avail = s->budget - s->reserved - (hs.device_bytes - less) - (12 * p->lu_stride + 32 * (int64_t)n);
+        return (int32_t)std::min<int64_t>(s->max_batch, avail > 0 ? avail / per_set : 0);
     };
-    fit();
-    if (p->slots < 1) {   // without the panels' workspaces, which are only faster
-        if (gblu_handle_lean(p->h, p->st) == GBLU_OK) {
+    // A budget holds as many sets as without the pool behind the factors and
+    // the panels, which are only faster.  A pattern that would not fit at all
+    // takes those of the earlier ones too.
+    auto fit = [&]() {
+        std::unique_lock<std::mutex> lk(s->mu);
+        p->slots = sets(0);
+        int64_t pool = 0, panels = 0;
+        for (int lean = 0; lean < 2 && p->slots < s->max_batch; lean++) {
+            gblu_handle_spare(p->h, &pool, &panels);
+            if (sets(pool + (lean ? panels : 0)) <= p->slots) continue;
+            lk.unlock();
+            const int r = gblu_handle_shrink(p->h, lean, p->st);
             gblu_get_stats(p->h, &hs);
-            fit();
+            lk.lock();
+            if (r != GBLU_OK) return r;
+            p->slots = sets(0);
         }
+        return GBLU_OK;
+    };
+    rc = fit();
+    if (rc == GBLU_OK && p->slots < 1) {
+        std::unique_lock<std::mutex> lk(s->mu);
+        int64_t pool = 0, panels = 0;
+        gblu_handle_spare(p->h, &pool, &panels);
+        int64_t spare = pool + panels;
+        for (auto &q : s->patterns) spare += q->spare;
+        if (sets(spare) >= 1) {
+            for (auto &q : s->patterns) {
+                q->shrink = true;
+                q->cv.notify_all();
+            }
+            s->cv_done.wait(lk, [&] {
+                for (auto &q : s->patterns)
+                    if (q->shrink) return false;
+                return true;
+            });
+            lk.unlock();
+            rc = fit();
+        }
+    }
+    if (rc != GBLU_OK) {
+        cudaFree(Ax0);
+        return bail_h(rc);
     }
     if (p->slots < 1) {
         cudaFree(Ax0);
@@ -486,6 +558,9 @@ int gblu_server_add_pattern(gblu_server s, int32_t n, const int32_t *Ap, const i
     if (rc != GBLU_OK) return bail_h(rc);
     gblu_get_stats(p->h, &hs);
     p->footprint = hs.device_bytes + server_buffer_bytes(p.get());
+    int64_t pool = 0, panels = 0;
+    gblu_handle_spare(p->h, &pool, &panels);
+    p->spare = pool + panels;
     Pattern *pp = p.get();
     {
         std::lock_guard<std::mutex> lk(s->mu);
