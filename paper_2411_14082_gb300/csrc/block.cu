@@ -79,15 +79,10 @@ __device__ __forceinline__ unsigned long long abs_bits(double v)
     return (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
 }
 
-// launch `step`: update by block step-1 (none for step 0) and factor block step
-__global__ void __launch_bounds__(kT) block_step_kernel(BlockArgs a, int step)
+// task t of launch `step`
+__device__ __forceinline__ void block_task(const BlockArgs &a, int step, int t, StepShared &s)
 {
-    __shared__ StepShared s;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (tid == 0) s.ticket = ld_volatile(&a.ctl->interrupted) ? -1 : atomicAdd(a.ticket + step, 1);
-    __syncthreads();
-    int t = s.ticket;
-    if (t < 0) return;   // a check failed before the block
     const int kd = step > 0 ? kB : 0;             // depth of the update
     const int kb = (step - 1) * kB;               // first column of block step-1
     const int o = step * kB;                      // first column of block step
@@ -251,12 +246,29 @@ __global__ void __launch_bounds__(kT) block_step_kernel(BlockArgs a, int step)
     }
 }
 
-// pivot checks, the block's entries into the factor's columns, ready flags:
-// one warp per column
-__global__ void __launch_bounds__(256) block_finish_kernel(BlockArgs a)
+// launch `step`: update by block step-1 (none for step 0) and factor block
+// step; tasks are handed out in order (a diagonal block is never waited for
+// before a running CTA has it), one per CTA or, where max_sms leaves fewer
+// CTAs than tasks, several
+__global__ void __launch_bounds__(kT) block_step_kernel(BlockArgs a, int step, int tasks)
 {
-    const int c = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-    if (c >= a.m) return;
+    __shared__ StepShared s;
+    for (;;) {
+        // (a check that failed before the block: nothing to do)
+        if (threadIdx.x == 0) s.ticket = ld_volatile(&a.ctl->interrupted) ? tasks : atomicAdd(a.ticket + step, 1);
+        __syncthreads();
+        const int t = s.ticket;
+        if (t >= tasks) return;
+        block_task(a, step, t, s);
+        if ((int)gridDim.x == tasks) return;
+        __syncthreads();
+    }
+}
+
+// pivot checks, the block's entries into the factor's columns, ready flags:
+// column c by one warp
+__device__ __forceinline__ void finish_column(const BlockArgs &a, int c, int lane)
+{
     // a check that failed before the block (one in the block is not a reason
     // to leave: every column is judged by itself)
     if (ld_volatile(&a.ctl->first_bad) < a.p || ld_volatile(&a.ctl->status)) return;
@@ -277,9 +289,20 @@ __global__ void __launch_bounds__(256) block_finish_kernel(BlockArgs a)
     if (lane == 0) st_release(a.finish + k, a.epoch < 0 ? ld_volatile(&a.ctl->epoch) : a.epoch);
 }
 
+__global__ void __launch_bounds__(256) block_finish_kernel(BlockArgs a)
+{
+    const int step = (int)((gridDim.x * blockDim.x) >> 5);
+    for (int c = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); c < a.m; c += step) finish_column(a, c, threadIdx.x & 31);
+}
+
 }  // namespace
 
 int block_steps(int m) { return (m + kB - 1) / kB; }
+
+int block_setup(int *ctas_per_sm)
+{
+    return (int)cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas_per_sm, block_step_kernel, kT, 0);
+}
 
 // launches of the block's LU (after the panels' launch on the same stream)
 int launch_block_lu(const BlockArgs &a, void *stream, long long *launches)
@@ -289,11 +312,12 @@ int launch_block_lu(const BlockArgs &a, void *stream, long long *launches)
     for (int b = 0; b < steps; b++) {
         const int rest = std::max(a.m - (b + 1) * kB, 0), ne = (rest + kEdge - 1) / kEdge;
         const int tiles = b > 0 ? ((rest + kTR - 1) / kTR) * ((rest + kTC - 1) / kTC) : 0;
-        block_step_kernel<<<1 + 2 * ne + tiles, kT, 0, st>>>(a, b);
+        const int tasks = 1 + 2 * ne + tiles;
+        block_step_kernel<<<std::min(tasks, a.max_ctas), kT, 0, st>>>(a, b, tasks);
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return (int)e;
     }
-    block_finish_kernel<<<(a.m + 7) / 8, 256, 0, st>>>(a);
+    block_finish_kernel<<<std::min((a.m + 7) / 8, a.max_ctas), 256, 0, st>>>(a);
     *launches += steps + 1;
     return (int)cudaGetLastError();
 }

@@ -84,7 +84,7 @@ struct gblu_ctx {
     int l2_bytes = 0;
     // re-factorization CTAs that fit on an SM, with kRefSmemTwo and kRefSmemThree
     int ref_blocks_per_sm[2] = {0, 0}, batch_blocks_per_sm[3] = {0, 0, 0}, ref32_blocks_per_sm[2] = {0, 0};
-    int solve_grid = 0, res_blocks = 0, trail_per_sm = 0;
+    int solve_grid = 0, res_blocks = 0, trail_per_sm = 0, block_per_sm = 0;
     bool f32_valid = false, f32_widened = false;   // single-precision factors of the last call
     int32_t force_col = -1;                        // forced check failure of the next refactorization
     double t_tail[4] = {0, 0, 0, 0};               // last tail run: kernel, repack, schedule, upload (ms)
@@ -687,6 +687,7 @@ int issue_refactor(gblu_ctx *h, const double *Ax, cudaStream_t st, int ep, bool 
         b.ticket = (int32_t *)(h->tb_words.p + m);      // one word per step: ticket, flag
         b.flag = b.ticket + block_steps((int)m);
         b.inv = (double *)(h->tb_words.p + m + block_steps((int)m));
+        b.max_ctas = sms_used(h) < h->sm_count ? pgrid(h, h->block_per_sm) : INT_MAX;
         long long nl = 0;
         const int e = launch_block_lu(b, st, &nl);
         h->launches += nl;
@@ -1327,6 +1328,7 @@ int gblu_create(gblu_handle *out, int device, const gblu_opts *o)
     int trail_per_sm = 0;
     if (e == cudaSuccess && r == 0) r = trail_setup(&trail_per_sm);
     if (e == cudaSuccess && r == 0) r = dense_setup(GBLU_DENSE_MAX_ROWS);
+    if (e == cudaSuccess && r == 0) r = block_setup(&h->block_per_sm);
     if (e == cudaSuccess && r == 0) r = tail_setup();
     if (e != cudaSuccess || r != 0 || h->ref_blocks_per_sm[0] < 1 || h->batch_blocks_per_sm[0] < 1) {
         const char *msg = cudaGetErrorString(e != cudaSuccess ? e : (cudaError_t)r);

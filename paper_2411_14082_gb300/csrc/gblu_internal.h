@@ -454,8 +454,10 @@ struct BlockArgs {
     int32_t *ticket, *flag;         // one per step, zeroed
     unsigned long long *colmax;     // bits of max |x| over each column's L rows, zeroed
     double *inv;                    // reciprocals of the diagonal
+    int max_ctas;                   // CTAs of a launch at most (the max_sms option)
 };
 int block_steps(int m);
+int block_setup(int *ctas_per_sm);
 int launch_block_lu(const BlockArgs &a, void *stream, long long *launches);
 constexpr int kDenseNb = 8;         // panel width
 int dense_setup(int max_rows);

@@ -1,8 +1,11 @@
 """A check that fails on a structure with a trailing block: one pass with the
 block finds the first failing step, and the restart goes on from the columns
 that passed, through gblu_refactorize and through a replayed gblu_step."""
+import time
+
 import numpy as np
 import pytest
+import torch
 
 from oracle import oracle as O
 from paper_2411_14082_gb300 import gblu
@@ -60,3 +63,28 @@ def test_a_failed_check_costs_one_pass_with_the_block(k):
         compare_factors(s.export_factors(), lu, 1e-10)
         assert s.stats()["n_repivot"] == 1 and s.stats()["n_refactor"] == 2
     assert O.residual(n, Ap, Ai, w, x.cpu().numpy(), b) <= 1e-12
+
+
+def test_the_block_keeps_to_max_sms():
+    """With one SM's share of CTAs the block's launches take several tasks per
+    CTA: the same bits, at a small part of the device's speed (the block is
+    all of the arithmetic here, and 152 SMs share it otherwise)."""
+    sys_ = band(1400, 1399, 0, 3)
+    n, Ap, Ai, Ax0, _ = sys_
+    s = solver(sys_)
+    v = dev(Ax0 * np.random.default_rng(2).uniform(0.98, 1.02, len(Ax0)))
+
+    def run():
+        s.refactorize(v)
+        torch.cuda.synchronize()
+        t0 = time.perf_counter()
+        s.refactorize(v)
+        torch.cuda.synchronize()
+        return time.perf_counter() - t0, s.export_factors()
+
+    t_all, want = run()
+    s.set_opts(max_sms=1)
+    t_one, got = run()
+    for k in want:
+        assert np.array_equal(want[k], got[k]), k
+    assert t_one > 8 * t_all
