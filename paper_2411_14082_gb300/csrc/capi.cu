@@ -431,7 +431,7 @@ static int try_install(gblu_ctx *h, Structure &&S, const std::vector<double> *va
     int panel_ctas[2];
     for (int i = 0; i < 2; i++)
         panel_ctas[i] = h->lean ? 0 :
-            std::max(h->ref_blocks_per_sm[i], std::max(h->batch_blocks_per_sm[i], h->ref32_blocks_per_sm[i])) * h->sm_count;
+            std::max(h->ref_blocks_per_sm[i], h->batch_blocks_per_sm[i]) * h->sm_count;
     build_schedule(h->P, h->S, h->opts.alpha, resident_warps, panel_ctas, h->opts.sched_mode, h->opts.warp_column_max, sp,
                    h->opts.dense_min_rows, h->W, defer_solve);
     h->solve_pending = defer_solve;
@@ -2526,7 +2526,7 @@ int gblu_refactorize_f32(gblu_handle h, const double *Ax_dev, void *stream, int3
     a.cap_short = d.cap_short; a.cap_long = d.cap_long; a.eps = d.eps; a.spin_limit = d.spin_limit;
     a.ctl = d.ctl;
     a.pan_id = d.pan_id; a.pan = d.pan; a.prow = d.prow; a.ppref = d.ppref; a.pmask = d.pmask; a.prun = d.prun;
-    a.smem_bytes = d.smem_bytes; a.pscratch = d.pscratch; a.pscratch_bytes = d.pscratch_bytes; a.pscratch_ctas = d.pscratch_ctas;
+    a.smem_bytes = cfg(h) == 0 ? kRefSmemTwo32 : kRefSmemThree32; a.pscratch = d.pscratch; a.pscratch_bytes = d.pscratch_bytes; a.pscratch_ctas = d.pscratch_ctas;
     const std::vector<int32_t> &ltp = h->W.level_task_ptr;
     const int32_t div = h->W.div_level;
     for (int32_t l = 0; l < div; l++) {
@@ -2538,7 +2538,9 @@ int gblu_refactorize_f32(gblu_handle h, const double *Ax_dev, void *stream, int3
     if (ltp[div] < ntask) {
         a.task_begin = ltp[div];
         a.ntasks = ntask - ltp[div];
-        KL(launch_refactor_tasks_f32(a, true, pgrid(h, h->ref32_blocks_per_sm[cfg(h)]), h->epoch, st));
+        int grid = pgrid(h, h->ref32_blocks_per_sm[cfg(h)]);
+        if (h->pscratch_ctas > 0) grid = std::min(grid, h->pscratch_ctas);   // a scratch for each
+        KL(launch_refactor_tasks_f32(a, true, grid, h->epoch, st));
     }
     // the pivots in double: a pivot that single precision cannot place
     // clearly on the passing side of the threshold fails here, and the

@@ -506,6 +506,12 @@ constexpr int kRefCapLong = 8 * kRefCapShort;  // per CTA (long columns), 60 KB
 // dynamic shared memory of a re-factorization CTA: two CTAs per SM, or three
 // (and a larger L1) where most of the work is in columns beyond panels
 constexpr int kRefSmemTwo = 100 * 1024, kRefSmemThree = 65 * 1024;
+// the same with single-precision values: the panels are sized for doubles, so
+// about half the room holds their work vectors and ring, three CTAs fit on an
+// SM in both, and the rest stays L1 (re-factorization of the 57,600-unknown
+// mesh with 100 KB and with 56 KB: 10.5 and 9.1 ms; of the 160,000-unknown
+// mesh with 65 KB and with 40 KB: 40.9 and 40.6 ms)
+constexpr int kRefSmemTwo32 = 56 * 1024, kRefSmemThree32 = kRefCapLong * (int)(sizeof(float) + sizeof(int32_t));
 // of a launch without panels: the column kernels' work vectors alone
 constexpr int kRefSmemColumns = kRefCapLong * (int)(sizeof(double) + sizeof(int32_t));
 // stage ring of a panel: four stages of kStageCap values (work vector in

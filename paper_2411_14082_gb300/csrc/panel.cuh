@@ -184,6 +184,14 @@ constexpr int kStagePad = 4;
 __host__ __device__ constexpr int stage_bytes_of(int cap, int elem) { return kHeadBytes + kStageRows * 4 + cap * elem; }
 static_assert(4 * stage_bytes_of(kStageCap, 8) == kPanelRing, "kPanelRing");
 static_assert(kStageCap / kPanelRun - kStagePad >= 32, "a stage holds 32 rows of the widest run");
+// a panel whose work vector fits beside the ring in doubles fits in floats
+constexpr bool fits_in_floats(int smem, int smem32)
+{
+    const int room = smem - kPanelRing, room32 = smem32 - 4 * stage_bytes_of(kStageCap, 4);
+    return room / (4 * 8 + 4) * (4 * 4 + 4) <= room32 && room / (8 * 8 + 4) * (8 * 4 + 4) <= room32 &&
+           3 * stage_bytes_of(kStageCapBig, 4) <= smem32 && kRefCapLong * 8 <= smem32;
+}
+static_assert(fits_in_floats(kRefSmemTwo, kRefSmemTwo32) && fits_in_floats(kRefSmemThree, kRefSmemThree32), "smem32");
 
 // rows of a stage for a run of w dependencies
 __device__ __forceinline__ int stage_rows(int cap, int w)
@@ -706,7 +714,8 @@ __device__ __noinline__ bool col_panel(const RefactorArgsT<R> *ap, int id, unsig
     // the stage ring, then work vector and rows in shared memory; or, with
     // larger stages, the rows alone and the work vector in this CTA's
     // scratch; or both there
-    const bool in_smem = (long long)len * (long long)(LD * sizeof(R) + 4) <= smem_bytes - kPanelRing;
+    const bool in_smem = (long long)len * (long long)(LD * sizeof(R) + 4) <=
+                         smem_bytes - 4 * stage_bytes_of(kStageCap, (int)sizeof(R));
     const int cap = in_smem ? kStageCap : kStageCapBig, ns = in_smem ? 4 : 3;
     const int stage_bytes = stage_bytes_of(cap, (int)sizeof(R));
     unsigned char *area = smem + ns * stage_bytes;

@@ -1137,11 +1137,11 @@ int launch_refactor_multi(const RefactorArgs *sets_dev, int nsets, const SetTask
 int refactor_setup_f32(int *blocks_per_sm)
 {
     cudaError_t e = cudaSuccess;
-    e = allow_smem(refactor_task_kernel<float, true, false, false>, kRefSmemTwo, e);
-    e = allow_smem(refactor_task_kernel<float, false, false, false>, kRefSmemTwo, e);
+    e = allow_smem(refactor_task_kernel<float, true, false, false>, kRefSmemTwo32, e);
+    e = allow_smem(refactor_task_kernel<float, false, false, false>, kRefSmemTwo32, e);
     for (int i = 0; i < 2 && e == cudaSuccess; i++)
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm[i], refactor_task_kernel<float, true, false, false>,
-                                                          kThreads, i == 0 ? kRefSmemTwo : kRefSmemThree);
+                                                          kThreads, i == 0 ? kRefSmemTwo32 : kRefSmemThree32);
     return (int)e;
 }
 
