@@ -628,6 +628,7 @@ RefactorArgs refactor_args(gblu_ctx *h, const double *Ax)
     a.ppref = h->ppref.p;
     a.pmask = h->pmask.p;
     a.prun = h->prun.p;
+    a.panels = h->W.pan.empty() ? 0 : 1;
     a.smem_bytes = h->W.smem;
     a.pscratch = h->pscratch.p;
     a.pscratch_bytes = h->W.pscratch;
@@ -1818,7 +1819,7 @@ static RefactorArgs batch_args(gblu_ctx *h, bool columns)
         a.task_ptr = h->ctask_ptr.p;
         a.task_cols = h->ctask_cols.p;
         a.amap = h->camap.p;
-        a.pan_id = nullptr;
+        a.panels = 0;
         a.smem_bytes = kRefSmemColumns;
         a.pscratch_ctas = 0;
     }
@@ -2526,7 +2527,7 @@ int gblu_refactorize_f32(gblu_handle h, const double *Ax_dev, void *stream, int3
     a.cap_short = d.cap_short; a.cap_long = d.cap_long; a.eps = d.eps; a.spin_limit = d.spin_limit;
     a.ctl = d.ctl;
     a.pan_id = d.pan_id; a.pan = d.pan; a.prow = d.prow; a.ppref = d.ppref; a.pmask = d.pmask; a.prun = d.prun;
-    a.smem_bytes = cfg(h) == 0 ? kRefSmemTwo32 : kRefSmemThree32; a.pscratch = d.pscratch; a.pscratch_bytes = d.pscratch_bytes; a.pscratch_ctas = d.pscratch_ctas;
+    a.panels = d.panels; a.smem_bytes = cfg(h) == 0 ? kRefSmemTwo32 : kRefSmemThree32; a.pscratch = d.pscratch; a.pscratch_bytes = d.pscratch_bytes; a.pscratch_ctas = d.pscratch_ctas;
     const std::vector<int32_t> &ltp = h->W.level_task_ptr;
     const int32_t div = h->W.div_level;
     for (int32_t l = 0; l < div; l++) {

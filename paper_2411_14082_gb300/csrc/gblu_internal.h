@@ -326,6 +326,7 @@ struct RefactorArgsT {
     const int32_t *prow = nullptr, *ppref = nullptr;
     const uint8_t *pmask = nullptr;
     const PanelRun *prun = nullptr;
+    int32_t panels = 0;             // some task is a panel
     int32_t smem_bytes = 0;         // dynamic shared memory of a CTA
     unsigned char *pscratch = nullptr;
     int64_t pscratch_bytes = 0;
@@ -504,7 +505,7 @@ constexpr int kRefThreads = 256;       // 8 warps per refactor CTA
 constexpr int kRefCapShort = 640;      // work-vector entries per warp (short columns)
 constexpr int kRefCapLong = 8 * kRefCapShort;  // per CTA (long columns), 60 KB
 // dynamic shared memory of a re-factorization CTA: two CTAs per SM, or three
-// (and a larger L1) where most of the work is in columns beyond panels
+// (and a larger L1) where there are no panels or wide columns among them
 constexpr int kRefSmemTwo = 100 * 1024, kRefSmemThree = 65 * 1024;
 // the same with single-precision values: the panels are sized for doubles, so
 // about half the room holds their work vectors and ring, three CTAs fit on an

@@ -885,7 +885,10 @@ __device__ __forceinline__ bool run_task(const RefactorArgsT<R> &a, const Refact
 // Tasks [task_begin, task_begin + ntasks): dealt to the CTAs in cluster mode
 // (persistent == 0; one each, or several where panels use the CTAs'
 // scratches, of which there are pscratch_ctas), taken by ticket in pipeline mode (persistent == 1).
-template <typename R, bool kWait, bool kDense, bool kPull>
+// kPanel = false: a task list without panels.  The column kernels are slower
+// in a kernel that also holds the panels' code, even if no task is a panel
+// (10,000-unknown grid with a dense tail 4.70 ms, without that code 4.49 ms).
+template <typename R, bool kWait, bool kDense, bool kPull, bool kPanel>
 __global__ void __launch_bounds__(kThreads, 3) refactor_task_kernel(const __grid_constant__ RefactorArgsT<R> a, int epoch, int persistent)
 {
     // a replayed graph passes -1: the epoch was written to the control block
@@ -906,7 +909,7 @@ __global__ void __launch_bounds__(kThreads, 3) refactor_task_kernel(const __grid
         const int t = s_t, quit = s_quit;
         __syncthreads();
         if (t >= a.ntasks || quit) break;
-        if (run_task<R, kWait, kDense, kPull, true>(a, &a, a.task_begin + t, xs, rs, epoch, s_sh, s_bars)) break;
+        if (run_task<R, kWait, kDense, kPull, kPanel>(a, &a, a.task_begin + t, xs, rs, epoch, s_sh, s_bars)) break;
     }
 }
 
@@ -947,7 +950,6 @@ __device__ __forceinline__ int group_task(long long t, int ntasks, int nsets, in
     return task;
 }
 
-// kPanel = false: a task list without panels (the column kernels alone)
 template <bool kWait, bool kPull, bool kPanel>
 __global__ void __launch_bounds__(kThreads, 3)
 refactor_batch_kernel(const RefactorArgs *sets, int nsets, int task_begin, int ntasks, int epoch, int persistent,
@@ -1038,16 +1040,29 @@ static cudaError_t allow_smem(K kernel, size_t sm, cudaError_t e)
     return e == cudaSuccess ? cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) : e;
 }
 
+// fn(kernel) for every instantiation that launch_tasks uses
+template <typename R, class F>
+static void for_task_kernels(F &&fn)
+{
+    fn(refactor_task_kernel<R, true, false, false, true>);
+    fn(refactor_task_kernel<R, false, false, false, true>);
+    fn(refactor_task_kernel<R, true, false, false, false>);
+    fn(refactor_task_kernel<R, false, false, false, false>);
+    if constexpr (std::is_same<R, double>::value) {
+        fn(refactor_task_kernel<R, true, true, false, true>);
+        fn(refactor_task_kernel<R, false, true, false, true>);
+        fn(refactor_task_kernel<R, true, true, false, false>);
+        fn(refactor_task_kernel<R, false, true, false, false>);
+        fn(refactor_task_kernel<R, true, false, true, true>);
+        fn(refactor_task_kernel<R, false, false, true, true>);
+    }
+}
+
 int refactor_setup(int *blocks_per_sm, int *batch_blocks_per_sm)
 {
     const size_t sm = kRefSmemTwo;
     cudaError_t e = cudaSuccess;
-    e = allow_smem(refactor_task_kernel<double, true, false, false>, sm, e);
-    e = allow_smem(refactor_task_kernel<double, false, false, false>, sm, e);
-    e = allow_smem(refactor_task_kernel<double, true, true, false>, sm, e);
-    e = allow_smem(refactor_task_kernel<double, false, true, false>, sm, e);
-    e = allow_smem(refactor_task_kernel<double, true, false, true>, sm, e);
-    e = allow_smem(refactor_task_kernel<double, false, false, true>, sm, e);
+    for_task_kernels<double>([&](auto kernel) { e = allow_smem(kernel, sm, e); });
     e = allow_smem(refactor_batch_kernel<true, false, true>, sm, e);
     e = allow_smem(refactor_batch_kernel<false, false, true>, sm, e);
     e = allow_smem(refactor_batch_kernel<true, true, true>, sm, e);
@@ -1066,9 +1081,9 @@ int refactor_setup(int *blocks_per_sm, int *batch_blocks_per_sm)
         auto fit = [&](int &out, auto kernel) {
             if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&out, kernel, kThreads, bytes);
         };
-        fit(b[0], refactor_task_kernel<double, true, false, false>);
-        fit(b[1], refactor_task_kernel<double, true, true, false>);
-        fit(b[2], refactor_task_kernel<double, true, false, true>);
+        fit(b[0], refactor_task_kernel<double, true, false, false, true>);
+        fit(b[1], refactor_task_kernel<double, true, true, false, true>);
+        fit(b[2], refactor_task_kernel<double, true, false, true, true>);
         fit(b[3], refactor_batch_kernel<true, false, true>);
         fit(b[4], refactor_batch_kernel<true, true, true>);
         blocks_per_sm[i] = std::min(b[0], std::min(b[1], b[2]));
@@ -1091,7 +1106,7 @@ int launch_refactor_batch(const RefactorArgs *sets_dev, const RefactorArgs &a0, 
     cudaStream_t st = (cudaStream_t)stream;
     if (group < 1 || group > nsets) group = nsets;
     if (pipeline) {
-        if (!a0.pan_id)
+        if (!a0.panels && !a0.pull_start)
             refactor_batch_kernel<true, false, false><<<grid, kThreads, a0.smem_bytes, st>>>(
                 sets_dev, nsets, a0.task_begin, a0.ntasks, epoch, 1, ticket, nullptr, group);
         else if (a0.pull_start)
@@ -1104,7 +1119,7 @@ int launch_refactor_batch(const RefactorArgs *sets_dev, const RefactorArgs &a0, 
         // a level launch has no waits: one group holding every set
         const long long blocks = (long long)a0.ntasks * nsets;
         if (blocks > INT_MAX) return (int)cudaErrorInvalidValue;
-        if (!a0.pan_id)
+        if (!a0.panels && !a0.pull_start)
             refactor_batch_kernel<false, false, false><<<level_grid(a0, blocks), kThreads, a0.smem_bytes, st>>>(
                 sets_dev, nsets, a0.task_begin, a0.ntasks, epoch, 0, ticket, nullptr, nsets);
         else if (a0.pull_start)
@@ -1137,39 +1152,49 @@ int launch_refactor_multi(const RefactorArgs *sets_dev, int nsets, const SetTask
 int refactor_setup_f32(int *blocks_per_sm)
 {
     cudaError_t e = cudaSuccess;
-    e = allow_smem(refactor_task_kernel<float, true, false, false>, kRefSmemTwo32, e);
-    e = allow_smem(refactor_task_kernel<float, false, false, false>, kRefSmemTwo32, e);
+    for_task_kernels<float>([&](auto kernel) { e = allow_smem(kernel, kRefSmemTwo32, e); });
     for (int i = 0; i < 2 && e == cudaSuccess; i++)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm[i], refactor_task_kernel<float, true, false, false>,
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm[i], refactor_task_kernel<float, true, false, false, true>,
                                                           kThreads, i == 0 ? kRefSmemTwo32 : kRefSmemThree32);
     return (int)e;
+}
+
+// the tasks of a, by the kernel that has what they need and no more: waits
+// (pipeline mode), a dense tail or trailing block, wide columns, panels
+template <typename R, bool kWait>
+static int launch_tasks(const RefactorArgsT<R> &a, unsigned grid, int epoch, cudaStream_t st)
+{
+    auto go = [&](auto kernel) { kernel<<<grid, kThreads, a.smem_bytes, st>>>(a, epoch, kWait ? 1 : 0); };
+    if constexpr (std::is_same<R, double>::value) {
+        if (a.dense_p < INT_MAX) {
+            if (a.panels) go(refactor_task_kernel<R, kWait, true, false, true>);
+            else go(refactor_task_kernel<R, kWait, true, false, false>);
+            return (int)cudaGetLastError();
+        }
+        if (a.pull_start) {
+            go(refactor_task_kernel<R, kWait, false, true, true>);
+            return (int)cudaGetLastError();
+        }
+    }
+    if (a.panels) go(refactor_task_kernel<R, kWait, false, false, true>);
+    else go(refactor_task_kernel<R, kWait, false, false, false>);
+    return (int)cudaGetLastError();
 }
 
 int launch_refactor_tasks_f32(const RefactorArgsT<float> &a, bool pipeline, int grid, int epoch, void *stream)
 {
     if (a.ntasks <= 0) return 0;
     cudaStream_t st = (cudaStream_t)stream;
-    if (pipeline) refactor_task_kernel<float, true, false, false><<<grid, kThreads, a.smem_bytes, st>>>(a, epoch, 1);
-    else refactor_task_kernel<float, false, false, false><<<level_grid(a, a.ntasks), kThreads, a.smem_bytes, st>>>(a, epoch, 0);
-    return (int)cudaGetLastError();
+    return pipeline ? launch_tasks<float, true>(a, grid, epoch, st)
+                    : launch_tasks<float, false>(a, level_grid(a, a.ntasks), epoch, st);
 }
 
 int launch_refactor_tasks(const RefactorArgs &a, bool pipeline, int grid, int epoch, void *stream)
 {
     if (a.ntasks <= 0) return 0;
     cudaStream_t st = (cudaStream_t)stream;
-    const bool dense = a.dense_p < INT_MAX;   // a dense tail is in use
-    if (pipeline) {
-        if (dense) refactor_task_kernel<double, true, true, false><<<grid, kThreads, a.smem_bytes, st>>>(a, epoch, 1);
-        else if (a.pull_start) refactor_task_kernel<double, true, false, true><<<grid, kThreads, a.smem_bytes, st>>>(a, epoch, 1);
-        else refactor_task_kernel<double, true, false, false><<<grid, kThreads, a.smem_bytes, st>>>(a, epoch, 1);
-    } else {
-        if (dense) refactor_task_kernel<double, false, true, false><<<level_grid(a, a.ntasks), kThreads, a.smem_bytes, st>>>(a, epoch, 0);
-        else if (a.pull_start)
-            refactor_task_kernel<double, false, false, true><<<level_grid(a, a.ntasks), kThreads, a.smem_bytes, st>>>(a, epoch, 0);
-        else refactor_task_kernel<double, false, false, false><<<level_grid(a, a.ntasks), kThreads, a.smem_bytes, st>>>(a, epoch, 0);
-    }
-    return (int)cudaGetLastError();
+    return pipeline ? launch_tasks<double, true>(a, grid, epoch, st)
+                    : launch_tasks<double, false>(a, level_grid(a, a.ntasks), epoch, st);
 }
 
 }  // namespace gblu

@@ -889,14 +889,21 @@ void build_schedule(const Pattern &P, const Structure &S, double alpha,
         lng += v[2];
     }
     // Two CTAs per SM hold the larger panels; three, with a larger L1, suit
-    // long columns, which are taken one at a time there (200x200x4 mesh: 74
-    // ms against 87 ms with panels in scratches), and wide columns, which
-    // wait most (256 sets of the bordered 141x141 grid: 354 ms against 384 ms)
-    const bool three = lng > 0.5 * outside || W.pull_cols > 0 || !panels;
+    // the column kernels and wide columns, which wait most (256 sets of the
+    // bordered 141x141 grid: 354 ms against 384 ms).  Where most of the flops
+    // outside the block are in long columns, every column is taken by the
+    // column kernels, in a kernel without the panels' code.  Meshes a x a x 4,
+    // re-factorization with panels / without, ms (share: of those flops):
+    //   a (share)   120 (.02)    135 (.24)    150 (.53)    170 (.72)    200 (.79)
+    //   double     15.9 / 18.4  23.0 / 22.6  31.8 / 28.8  48.8 / 44.0  81.5 / 67.1
+    //   single     10.3 / 13.9  13.3 / 15.5  18.4 / 20.3  26.0 / 26.2  44.5 / 39.3
+    // so the line lies between where the two precisions cross.
+    const bool long_cols = lng > 0.5 * outside && W.pull_cols == 0;
+    const bool three = long_cols || W.pull_cols > 0 || !panels || W.dense_m > 0;
     W.smem = three ? kRefSmemThree : kRefSmemTwo;
     // panels of wide columns hold kPullLd values per row of their scratch
     W.pull_ld = 1;
-    build_panels(S, panel_ctas[three ? 1 : 0], !three, W);   // (none for 0 CTAs)
+    build_panels(S, long_cols ? 0 : panel_ctas[three ? 1 : 0], !three, W);   // (none for 0 CTAs)
     W.tb_nux.resize(W.tb_m);
     for (int32_t c = 0; c < W.tb_m; c++) {
         const int32_t *r = S.LUi.data() + S.LUp[W.tb_p + c];
