@@ -612,7 +612,9 @@ typedef struct {
     /* wide columns of the installed structure (at most 64 L entries, at
        least 256 supernode runs among the dependencies): the re-factorization
        applies all but their last run of dependencies row by row through the
-       rows of L (0 when the per-CTA scratch would exceed 1 GiB) */
+       rows of L (0 when the per-CTA scratch would exceed 1 GiB, and on a
+       predicted structure whose wide columns all have fewer than 512 runs
+       and hold under 1% of the operations) */
     int64_t wide_cols;
     /* structure re-predictions of the last restart or first factorization
        on a predicted structure: each is one pivot exchange found by the

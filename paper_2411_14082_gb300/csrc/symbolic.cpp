@@ -820,9 +820,9 @@ void build_schedule(const Pattern &P, const Structure &S, double alpha,
     // starts); none in the dense tail ----
     W.pull_start.assign(n, 0);
     {
-        std::atomic<int64_t> cnt{0};
-        parallel_ranges(n, S.LUp.data(), [&](int32_t k0, int32_t k1, int) {
-            int64_t c = 0;
+        struct Part { int64_t cols = 0; int32_t runs = 0; double flops = 0; } wide[kHostThreads];
+        parallel_ranges(n, S.LUp.data(), [&](int32_t k0, int32_t k1, int t) {
+            Part p;
             for (int32_t k = k0; k < k1 && k < W.dense_p; k++) {
                 const int64_t b = S.LUp[k];
                 const int32_t nd = S.nU[k] - 1, nl = (int32_t)(S.LUp[k + 1] - b) - S.nU[k];
@@ -832,14 +832,41 @@ void build_schedule(const Pattern &P, const Structure &S, double alpha,
                 int32_t runs = 1;
                 for (int32_t i = 1; i < nd; i++) runs += !linked(i);
                 if (runs < kPullMinRuns) continue;
-                int32_t p = nd - 1;
-                while (p > 0 && linked(p)) p--;
-                W.pull_start[k] = p;
-                c += p > 0;
+                int32_t e = nd - 1;
+                while (e > 0 && linked(e)) e--;
+                W.pull_start[k] = e;
+                p.cols += e > 0;
+                p.runs = std::max(p.runs, runs);
+                for (int32_t i = 0; i < nd; i++) p.flops += 2.0 * (double)(S.LUp[u[i] + 1] - S.LUp[u[i]] - S.nU[u[i]]);
             }
-            cnt += c;
+            wide[t] = p;
         });
-        W.pull_cols = cnt.load();
+        Part all;
+        for (const Part &p : wide) {
+            all.cols += p.cols;
+            all.runs = std::max(all.runs, p.runs);
+            all.flops += p.flops;
+        }
+        W.pull_cols = all.cols;
+        // A predicted structure keeps its trailing block (no wide columns
+        // beside it) when its wide columns barely are such: the last columns
+        // of any structure have few L entries, and some of them just reach
+        // the runs (200x200x4 mesh in the generator's order: five columns of
+        // 257 to 279 runs, 0.2% of the flops, against which the block of
+        // 2,721 columns stood: 81.0 -> 71.4 ms).  The rails of a
+        // grid have more runs, or hold more: 3,608 unknowns with eight rails,
+        // 408 to 439 runs and 13% of the flops.
+        if (S.symmetric && W.pull_cols > 0 && all.runs < 2 * kPullMinRuns) {
+            double flops = 0;   // L and U^T have one pattern
+            for (int32_t k = 0; k < n; k++) {
+                const double nl = (double)(S.LUp[k + 1] - S.LUp[k] - S.nU[k]);
+                flops += 2.0 * nl * nl;
+            }
+            if (all.flops < 0.01 * flops) {
+                std::fill(W.pull_start.begin(), W.pull_start.end(), 0);
+                W.pull_cols = 0;
+            }
+        }
     }
     // ---- trailing block: the longest [p, n) in which the factor holds at
     // least kBlockDensity of the entries; of predicted structures (L and U^T

@@ -88,3 +88,42 @@ def test_the_block_keeps_to_max_sms():
     for k in want:
         assert np.array_equal(want[k], got[k]), k
     assert t_one > 8 * t_all
+
+
+def bordered_blocks(tail, wide, blocks=300):
+    """`blocks` dense 2 x 2 blocks and `tail` dense last columns: the last
+    `wide` of them touch every block (a run of dependencies each), the others
+    one block in turn."""
+    n = 2 * blocks + tail
+    rng = np.random.default_rng(9)
+    a = np.zeros((n, n), bool)
+    for j in range(blocks):
+        a[2 * j:2 * j + 2, 2 * j:2 * j + 2] = True
+        a[2 * j:2 * j + 2, n - wide:] = True
+        a[2 * j:2 * j + 2, 2 * blocks + j % (tail - wide)] = True
+    a |= a.T
+    a[2 * blocks:, 2 * blocks:] = True
+    cols, rows = np.nonzero(a.T)
+    Ap = np.r_[0, np.cumsum(np.bincount(cols, minlength=n))].astype(np.int32)
+    Ax = np.where(rows == cols, 1.0, rng.uniform(-1.0, 1.0, len(rows)) / n)
+    return n, Ap, rows.astype(np.int32), Ax, np.arange(n, dtype=np.int32)
+
+
+@pytest.mark.parametrize("wide,taken", [(3, 0), (40, 40)])
+def test_columns_that_are_barely_wide_leave_the_block(wide, taken):
+    """Three last columns of 301 runs, 0.7% of the flops, do not count as wide
+    ones and the block of 700 columns (44 steps) is factored densely; forty
+    hold more and count.  Both ways the factors are the oracle's, and the
+    batch's route gives the same bits."""
+    sys_ = bordered_blocks(700, wide)
+    n, Ap, Ai, Ax0, Q = sys_
+    s = solver(sys_)
+    assert s.stats()["wide_cols"] == taken
+    v = Ax0 * np.random.default_rng(2).uniform(0.98, 1.02, len(Ax0))
+    passes, (_, rep) = launches(s, lambda: s.refactorize(dev(v)))
+    assert not rep and (passes > 44) == (taken == 0)
+    lu = O.refactorize(O.factorize(n, Ap, Ai, Ax0, Q, 1e-3), Ap, Ai, v)
+    compare_factors(s.export_factors(), lu, 1e-10)
+    b = dev(np.random.default_rng(4).uniform(-1.0, 1.0, n))
+    LU, failed = s.refactorize_batch(dev(v[None]))
+    assert not failed.any() and torch.equal(s.solve_batch(LU, b[None])[0], s.solve(b))
