@@ -525,6 +525,7 @@ static int try_install(gblu_ctx *h, Structure &&S, const std::vector<double> *va
 int install_structure(gblu_ctx *h, Structure &&S, const std::vector<double> *values, cudaStream_t st,
                       bool defer_solve = false)
 {
+    HostTeamScope team;
     int rc = try_install(h, std::move(S), values, st, defer_solve);
     // without room: once more without the pool behind the factors, then
     // without what only makes the re-factorization faster
@@ -1116,6 +1117,7 @@ constexpr int kMaxRepredict = 6;
 int repredict(gblu_ctx *h, const double *Ax, cudaStream_t st, const std::vector<int32_t> &prefer, int32_t k,
               bool *solved)
 {
+    HostTeamScope team;
     *solved = false;
     h->repredictions = 0;
     // a forced failure (gblu_refactorize_forced) belongs to the first pass
@@ -1475,6 +1477,7 @@ int gblu_factorize(gblu_handle h, const double *Ax_dev, void *stream)
 {
     NvtxRange nvtx_range("gblu_factorize");
     CK(check_handle(h));
+    HostTeamScope team;
     h->last_repivot = false;
     if (!Ax_dev) return fail(GBLU_ERR_INVALID_INPUT, "null Ax_dev");
     DeviceGuard g(h->device);

@@ -235,6 +235,18 @@ int64_t symmetric_fill(const Pattern &P, double *flops = nullptr);
 void symmetric_structure(const Pattern &P, Structure &S, const std::vector<int32_t> *piv = nullptr);
 // off-diagonal entries of A whose transposed position is not an entry of A
 int64_t unsymmetric_entries(const Pattern &P);
+// Within a scope the parallel parts of the host work run on one set of
+// threads, started by the first and joined at the scope's end (a scope inside
+// another adds nothing; each calling thread has its own)
+struct HostTeam;
+struct HostTeamScope {
+    HostTeam *own = nullptr;
+    HostTeamScope();
+    ~HostTeamScope();
+    HostTeamScope(const HostTeamScope &) = delete;
+    HostTeamScope &operator=(const HostTeamScope &) = delete;
+};
+
 // The schedule of a structure; with defer_solve, only what the
 // re-factorization reads (the solve part follows by build_solve_schedule)
 void build_schedule(const Pattern &P, const Structure &S, double alpha,

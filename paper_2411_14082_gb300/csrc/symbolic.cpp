@@ -3,7 +3,10 @@
 // device code and no CUDA calls in this file.
 #include <algorithm>
 #include <atomic>
+#include <condition_variable>
 #include <cstring>
+#include <functional>
+#include <mutex>
 #include <numeric>
 #include <thread>
 
@@ -170,6 +173,142 @@ int64_t symmetric_fill(const Pattern &P, double *flops)
     return total;
 }
 
+constexpr int kHostThreads = 16;
+static int team_size() { return (int)std::max(1u, std::min((unsigned)kHostThreads, std::thread::hardware_concurrency())); }
+
+// The host threads of one call (HostTeamScope): started by its first parallel
+// part and joined at its end.  A first factorization has about 20 such parts,
+// and starting 15 threads takes 0.56 ms in a process that holds a CUDA context
+// (0.26 ms without): more than many of the parts.  First factorization of the
+// meshes of 12,960 and 51,840 unknowns: 21.3 -> 14.6 and 39.6 -> 32.6 ms.
+struct HostTeam {
+    const int nt = team_size();
+    std::vector<std::thread> th;
+    std::mutex mu;
+    std::condition_variable go, done;
+    const std::function<void(int)> *job = nullptr;
+    uint64_t round = 0;
+    int left = 0;
+    bool stop = false;
+
+    ~HostTeam()
+    {
+        {
+            std::lock_guard<std::mutex> lk(mu);
+            stop = true;
+        }
+        go.notify_all();
+        for (std::thread &x : th) x.join();
+    }
+
+    // fn(t) for t = 0 .. nt-1, t = 0 by the calling thread
+    void run(const std::function<void(int)> &fn)
+    {
+        {
+            std::lock_guard<std::mutex> lk(mu);
+            job = &fn;
+            left = nt - 1;
+            round++;
+        }
+        if (th.empty())
+            for (int t = 1; t < nt; t++) th.emplace_back([this, t] { work(t); });
+        else
+            go.notify_all();
+        fn(0);
+        std::unique_lock<std::mutex> lk(mu);
+        done.wait(lk, [this] { return left == 0; });
+    }
+
+    void work(int t)
+    {
+        uint64_t seen = 0;
+        for (;;) {
+            const std::function<void(int)> *fn;
+            {
+                std::unique_lock<std::mutex> lk(mu);
+                go.wait(lk, [&] { return stop || round != seen; });
+                if (stop) return;
+                seen = round;
+                fn = job;
+            }
+            (*fn)(t);
+            std::lock_guard<std::mutex> lk(mu);
+            if (--left == 0) done.notify_one();
+        }
+    }
+};
+
+static thread_local HostTeam *host_team = nullptr;
+
+HostTeamScope::HostTeamScope()
+{
+    if (!host_team) host_team = own = new HostTeam;
+}
+
+HostTeamScope::~HostTeamScope()
+{
+    if (!own) return;
+    host_team = nullptr;
+    delete own;
+}
+
+// fn(t) on the threads of the scope this is called in, or of a scope of its
+// own (a part inside another part, a thread started by the call)
+static void on_team(const std::function<void(int)> &fn)
+{
+    HostTeamScope scope;
+    HostTeam *team = host_team;
+    host_team = nullptr;   // busy
+    team->run(fn);
+    host_team = team;
+}
+
+// fn(k0, k1, t) on up to kHostThreads host threads t over index ranges
+// [k0, k1) of about equal weight (ptr: n+1 ascending offsets, the weight of
+// index k is ptr[k+1] - ptr[k]); small inputs run on the calling thread
+template <class T, class F>
+static void parallel_ranges(int32_t n, const T *ptr, F &&fn)
+{
+    const int nt = team_size();
+    const int64_t total = n > 0 ? (int64_t)ptr[n] - (int64_t)ptr[0] : 0;
+    if (nt == 1 || total < (1 << 20)) {
+        fn(0, n, 0);
+        return;
+    }
+    int32_t cut[kHostThreads + 1] = {0};
+    for (int t = 1; t <= nt; t++) {
+        int32_t k1 = n;
+        if (t < nt) {
+            const T target = (T)((int64_t)ptr[0] + total * t / nt);
+            k1 = (int32_t)(std::lower_bound(ptr, ptr + n + 1, target) - ptr);
+        }
+        cut[t] = std::min(std::max(k1, cut[t - 1]), n);
+    }
+    on_team([&](int t) {
+        if (cut[t + 1] > cut[t]) fn(cut[t], cut[t + 1], t);
+    });
+}
+
+// fn(k0, k1, t) over chunks [k0, k1) of `chunk` indices, taken in turn by
+// up to kHostThreads host threads t as each finishes its previous chunk (for
+// work whose cost per index is not known in advance)
+template <class F>
+static void parallel_chunks(int32_t n, int32_t chunk, F &&fn)
+{
+    if (team_size() == 1 || n <= chunk) {
+        if (n > 0) fn(0, n, 0);
+        return;
+    }
+    std::atomic<int64_t> next{0};
+    on_team([&](int t) {
+        for (;;) {
+            const int64_t k0 = next.fetch_add(chunk);
+            if (k0 >= n) break;
+            fn((int32_t)k0, (int32_t)std::min<int64_t>(n, k0 + chunk), t);
+        }
+    });
+}
+
 // Partition point and trapezoid slices of one triangular factor (Section
 // V-A).  count_from[p] = entries of the trailing block [p, n) (suffix sums of
 // the per-column (lower) or per-row (upper) strict counts); rowlen[i] = all
@@ -181,60 +320,6 @@ int64_t symmetric_fill(const Pattern &P, double *flops)
 // kept if it holds min_entries entries.  The rows [P0, n) are cut into
 // `slices` pieces of equal entry counts (at most max_piece rows each).
 // Returns n when no block qualifies.
-// fn(k0, k1, t) on up to kHostThreads host threads t over index ranges
-// [k0, k1) of about equal weight (ptr: n+1 ascending offsets, the weight of
-// index k is ptr[k+1] - ptr[k]); small inputs run on the calling thread
-constexpr int kHostThreads = 16;
-
-template <class T, class F>
-static void parallel_ranges(int32_t n, const T *ptr, F &&fn)
-{
-    const int nt = (int)std::max(1u, std::min((unsigned)kHostThreads, std::thread::hardware_concurrency()));
-    const int64_t total = n > 0 ? (int64_t)ptr[n] - (int64_t)ptr[0] : 0;
-    if (nt == 1 || total < (1 << 20)) {
-        fn(0, n, 0);
-        return;
-    }
-    std::vector<std::thread> th;
-    int32_t k0 = 0;
-    for (int t = 1; t <= nt; t++) {
-        int32_t k1 = n;
-        if (t < nt) {
-            const T target = (T)((int64_t)ptr[0] + total * t / nt);
-            k1 = (int32_t)(std::lower_bound(ptr, ptr + n + 1, target) - ptr);
-        }
-        k1 = std::min(std::max(k1, k0), n);
-        if (k1 > k0) th.emplace_back(fn, k0, k1, t - 1);
-        k0 = k1;
-    }
-    for (std::thread &x : th) x.join();
-}
-
-// fn(k0, k1, t) over chunks [k0, k1) of `chunk` indices, taken in turn by
-// up to kHostThreads host threads t as each finishes its previous chunk (for
-// work whose cost per index is not known in advance)
-template <class F>
-static void parallel_chunks(int32_t n, int32_t chunk, F &&fn)
-{
-    const int nt = (int)std::max(1u, std::min((unsigned)kHostThreads, std::thread::hardware_concurrency()));
-    if (nt == 1 || n <= chunk) {
-        if (n > 0) fn(0, n, 0);
-        return;
-    }
-    std::atomic<int64_t> next{0};
-    auto run = [&](int t) {
-        for (;;) {
-            const int64_t k0 = next.fetch_add(chunk);
-            if (k0 >= n) break;
-            fn((int32_t)k0, (int32_t)std::min<int64_t>(n, k0 + chunk), t);
-        }
-    };
-    std::vector<std::thread> th;
-    for (int t = 1; t < nt; t++) th.emplace_back(run, t);
-    run(0);
-    for (std::thread &x : th) x.join();
-}
-
 static int32_t dense_split(int32_t n, const std::vector<int64_t> &count_from, const std::vector<int64_t> &rowlen,
                            const SolveSplit &sp, std::vector<int32_t> &cut)
 {
@@ -532,6 +617,30 @@ void build_solve_schedule(const Structure &S, const SolveSplit &split, Schedule 
     W.solve_ready = true;
 }
 
+// How many of the ascending rows r[0 .. cnt) are consecutive columns of the
+// chain that r[0] is in
+static inline int32_t chain_part(const int32_t *r, int32_t cnt, const std::vector<int32_t> &chain_end)
+{
+    const int32_t most = std::min(cnt, chain_end[r[0]] + 1 - r[0]);
+    if (r[most - 1] == r[0] + most - 1) return most;   // ascending: none is missing
+    int32_t len = 1;
+    while (r[len] == r[0] + len) len++;
+    return len;
+}
+
+// the run of w dependencies j0 .. at slots t ..
+static inline PanelRun panel_run(const Structure &S, int32_t t, int32_t j0, int w, unsigned mask)
+{
+    const int32_t jl = j0 + w - 1;
+    PanelRun r;
+    r.t = t;
+    r.wm = (int32_t)((unsigned)w | (mask << 8));
+    r.lbl = S.LUp[jl] + S.nU[jl];
+    r.nR = (int32_t)(S.LUp[jl + 1] - r.lbl);
+    r.j0 = j0;
+    return r;
+}
+
 // Panels of the re-factorization (Schedule::pan): the columns of each
 // supernode of L whose neighbours also depend on one another, cut from the
 // lowest up.  kPanelMax columns while they have at most kPanelWideRows rows
@@ -539,7 +648,12 @@ void build_solve_schedule(const Structure &S, const SolveSplit &split, Schedule 
 // else four, in shared memory (2,261 slots) or in a scratch of the CTA
 // (allow_scratch).  Wide columns and the dense
 // tail stay single.
-static void build_panels(const Structure &S, int panel_ctas, bool allow_scratch, Schedule &W)
+//
+// The columns' U rows are taken by intervals, the part of a chain of linked
+// columns that a column depends on (from its first such row to the chain's
+// end, as a rule): unions, runs and counts cost an interval, not a row.
+static void build_panels(const Structure &S, const std::vector<int32_t> &chain_end, int panel_ctas, bool allow_scratch,
+                         Schedule &W)
 {
     const int32_t n = S.n;
     W.pan.clear();
@@ -571,10 +685,9 @@ static void build_panels(const Structure &S, int panel_ctas, bool allow_scratch,
     };
     struct Part {
         std::vector<PanelDesc> pan;
-        std::vector<int32_t> prow, ppref;
-        std::vector<uint8_t> pmask;
+        std::vector<int32_t> ppref;
         std::vector<PanelRun> prun;
-        int64_t scratch = 0;
+        int64_t scratch = 0, rows = 0;   // rows (and masks) written from its columns' U entries on
     };
     // small structures stay on this thread
     auto in_chunks = [&](int32_t m, int32_t chunk, auto &&fn) {
@@ -583,30 +696,71 @@ static void build_panels(const Structure &S, int panel_ctas, bool allow_scratch,
     };
     const int32_t chunk = 128, nparts = (n + chunk - 1) / chunk;
     std::vector<Part> parts(nparts);
+    // the unions' rows and masks, each part's in as much room as its columns
+    // have U entries: nothing is copied as they grow, and pages that stay
+    // unused cost nothing (with the intervals: mesh of 51,840 unknowns, 16
+    // threads, 2.2 -> 1.4 ms)
+    std::vector<int64_t> at(nparts + 1, 0);
+    for (int32_t i = 0; i < nparts; i++) {
+        at[i + 1] = at[i];
+        // (a panel that begins in a part may end a few columns after it)
+        const int32_t e = std::min(n, (i + 1) * chunk + kPanelMax);
+        for (int32_t k = i * chunk; k < e; k++) at[i + 1] += S.nU[k];
+    }
+    BigVec<int32_t> rows;
+    BigVec<uint8_t> masks;
+    rows.resize(at[nparts]);
+    masks.resize(at[nparts]);
     std::vector<uint8_t> first(n, 0);   // column k begins a panel
+    struct Rows { int32_t a, b; uint32_t mask; };   // rows [a, b) of the union, in the columns of mask
     in_chunks(n, chunk, [&](int32_t c0, int32_t c1, int) {
-        std::vector<uint64_t> u, v;   // union rows: row << 8 | mask of the columns that have it
-        // the union of the U rows above k of columns k .. k+nc-1; its size
+        std::vector<Rows> u, v;
+        int32_t above[kPanelMax];   // U rows above the panel, per column
+        auto add = [&](int32_t a, int32_t b, uint32_t mask) {
+            if (!v.empty() && v.back().b == a && v.back().mask == mask && W.chain[a - 1]) v.back().b = b;
+            else v.push_back({a, b, mask});
+        };
+        // u = the union of the U rows above k of columns k .. k+nc-1; its size
         auto join = [&](int32_t k, int nc) -> int64_t {
-            int64_t most = 0, nu = 0;
-            for (int c = 0; c < nc; c++) most += S.nU[k + c];
-            if ((int64_t)u.size() < most) { u.resize(most); v.resize(most); }
+            u.clear();
             for (int c = 0; c < nc; c++) {
                 const int32_t *r = S.LUi.data() + S.LUp[k + c];
-                const int32_t *re = std::lower_bound(r, r + S.nU[k + c], k);
-                const uint64_t bit = (uint64_t)1 << c, *p = u.data(), *pe = p + nu;
-                uint64_t *o = v.data();
-                while (p < pe && r < re) {
-                    const int32_t a = (int32_t)(*p >> 8), b = *r;
-                    *o++ = a <= b ? (*p | (a == b ? bit : 0)) : (((uint64_t)b << 8) | bit);
-                    p += a <= b;
-                    r += b <= a;
+                const int32_t cnt = (int32_t)(std::lower_bound(r, r + S.nU[k + c], k) - r);
+                const uint32_t bit = 1u << c;
+                above[c] = cnt;
+                v.clear();
+                size_t p = 0;
+                int32_t pa = u.empty() ? 0 : u[0].a;   // what is left of u[p] begins at pa
+                for (int32_t i = 0; i < cnt;) {
+                    int32_t a = r[i];
+                    const int32_t b = a + chain_part(r + i, cnt - i, chain_end);
+                    i += b - a;
+                    while (p < u.size() && u[p].b <= a) {
+                        add(pa, u[p].b, u[p].mask);
+                        if (++p < u.size()) pa = u[p].a;
+                    }
+                    while (a < b) {
+                        if (p == u.size() || b <= pa) {
+                            add(a, b, bit);
+                            break;
+                        }
+                        if (a < pa) add(a, pa, bit);
+                        else if (pa < a) add(pa, a, u[p].mask);
+                        a = pa = std::max(a, pa);
+                        const int32_t e = std::min(b, u[p].b);
+                        add(a, e, u[p].mask | bit);
+                        a = pa = e;
+                        if (pa == u[p].b && ++p < u.size()) pa = u[p].a;
+                    }
                 }
-                while (p < pe) *o++ = *p++;
-                while (r < re) *o++ = ((uint64_t)*r++ << 8) | bit;
-                nu = o - v.data();
+                while (p < u.size()) {
+                    add(pa, u[p].b, u[p].mask);
+                    if (++p < u.size()) pa = u[p].a;
+                }
                 u.swap(v);
             }
+            int64_t nu = 0;
+            for (const Rows &x : u) nu += x.b - x.a;
             return nu;
         };
         // one call has every part when it runs serially
@@ -651,30 +805,57 @@ static void build_panels(const Structure &S, int panel_ctas, bool allow_scratch,
                     d.k0 = k;
                     d.nc = nc;
                     d.nu = (int32_t)nu;
-                    d.pull = wide ? (int32_t)(std::lower_bound(u.begin(), u.begin() + nu, (uint64_t)prefix_end(k) << 8) - u.begin()) : 0;
-                    d.uoff = (int64_t)pt.prow.size();
+                    if (wide)
+                        for (const Rows &x : u) d.pull += std::max(0, std::min(x.b, prefix_end(k)) - x.a);
+                    d.uoff = pt.rows;
                     d.poff = (int64_t)pt.ppref.size();
-                    pt.prow.resize(d.uoff + nu + nc);
-                    pt.pmask.resize(d.uoff + nu + nc);
+                    d.roff = (int64_t)pt.prun.size();
+                    pt.rows += nu + nc;
                     pt.ppref.resize(d.poff + (nu + 31) / 32 * nc);
-                    int32_t *row = pt.prow.data() + d.uoff, *pref = pt.ppref.data() + d.poff;
-                    uint8_t *msk = pt.pmask.data() + d.uoff;
-                    int32_t cnt[kPanelMax] = {};
-                    for (int64_t s = 0; s < nu; s++) {
-                        if (s % 32 == 0)
-                            for (int c = 0; c < nc; c++) *pref++ = cnt[c];
-                        row[s] = (int32_t)(u[s] >> 8);
-                        msk[s] = (uint8_t)u[s];
-                        for (int c = 0; c < nc; c++) cnt[c] += (int32_t)(u[s] >> c) & 1;
-                    }
-                    for (int q = 0; q < nc; q++) {   // diagonal-block rows
-                        unsigned mk = 0;
-                        for (int c = 0; c < nc; c++) {
-                            const int32_t *r = S.LUi.data() + S.LUp[k + c];
-                            if (q >= c || std::binary_search(r, r + S.nU[k + c], k + q)) mk |= 1u << c;
+                    int32_t *row = rows.data() + at[b / chunk] + d.uoff, *pref = pt.ppref.data() + d.poff;
+                    uint8_t *msk = masks.data() + at[b / chunk] + d.uoff;
+                    int32_t cnt[kPanelMax] = {}, s = 0, next = 0;   // next slot with prefix counts
+                    PanelRun run{};
+                    int w = 0;
+                    unsigned mk = 0;
+                    auto flush = [&]() {
+                        if (w > 0) pt.prun.push_back(panel_run(S, run.t, run.j0, w, mk));
+                        w = 0;
+                        mk = 0;
+                    };
+                    for (const Rows &x : u) {
+                        const int32_t len = x.b - x.a;
+                        std::iota(row + s, row + s + len, x.a);
+                        std::memset(msk + s, (int)x.mask, len);
+                        for (; next < s + len; next += 32)
+                            for (int c = 0; c < nc; c++) *pref++ = cnt[c] + ((x.mask >> c) & 1u ? next - s : 0);
+                        for (int c = 0; c < nc; c++) cnt[c] += (x.mask >> c) & 1u ? len : 0;
+                        for (int32_t r = x.a; r < x.b;) {
+                            const int32_t t = s + (r - x.a);
+                            if (w == 0 || w == kPanelRun || r != run.j0 + w || !W.chain[r - 1] || r == W.tb_p || t == d.pull) {
+                                flush();
+                                run.t = t;
+                                run.j0 = r;
+                            }
+                            int32_t take = std::min({x.b - r, kPanelRun - w, chain_end[r] + 1 - r});
+                            if (W.tb_p > r) take = std::min(take, W.tb_p - r);
+                            if (d.pull > t) take = std::min(take, d.pull - t);
+                            w += take;
+                            mk |= x.mask;
+                            r += take;
                         }
+                        s += len;
+                    }
+                    flush();
+                    d.nruns = (int32_t)((int64_t)pt.prun.size() - d.roff);
+                    // diagonal-block rows
+                    for (int q = 0; q < nc; q++) {
                         row[nu + q] = k + q;
-                        msk[nu + q] = (uint8_t)mk;
+                        msk[nu + q] = (uint8_t)((2u << q) - 1u);   // column q's diagonal, L rows of the columns before
+                    }
+                    for (int c = 1; c < nc; c++) {
+                        const int32_t *r = S.LUi.data() + S.LUp[k + c];
+                        for (int32_t i = above[c]; i + 1 < S.nU[k + c]; i++) msk[nu + (r[i] - k)] |= (uint8_t)(1u << c);
                     }
                     first[k] = 1;
                     pt.pan.push_back(d);
@@ -687,13 +868,13 @@ static void build_panels(const Structure &S, int panel_ctas, bool allow_scratch,
     std::vector<int64_t> op(nparts + 1, 0), ou(nparts + 1, 0), of(nparts + 1, 0), orr(nparts + 1, 0);
     for (int32_t i = 0; i < nparts; i++) {
         op[i + 1] = op[i] + (int64_t)parts[i].pan.size();
-        ou[i + 1] = ou[i] + (int64_t)parts[i].prow.size();
+        ou[i + 1] = ou[i] + parts[i].rows;
         of[i + 1] = of[i] + (int64_t)parts[i].ppref.size();
         W.pscratch = std::max(W.pscratch, parts[i].scratch);
     }
     if (W.pscratch > 0 && (size_t)W.pscratch * (size_t)panel_ctas > kPanelScratchBytes) {
         // long columns one at a time (and wide ones, when even they do not fit)
-        if (allow_scratch) build_panels(S, panel_ctas, false, W);
+        if (allow_scratch) build_panels(S, chain_end, panel_ctas, false, W);
         else {
             std::fill(W.pan_id.begin(), W.pan_id.end(), -1);
             W.pscratch = 0;
@@ -706,23 +887,29 @@ static void build_panels(const Structure &S, int panel_ctas, bool allow_scratch,
     W.prow.resize(ou[nparts]);
     W.pmask.resize(ou[nparts]);
     W.ppref.resize(of[nparts]);
-    // The arrays of the parts in one, and the runs: up to kPanelRun linked
-    // dependencies; the last kPanelRun dependencies, which may still be in
-    // progress when the panel meets them, are cut where a panel of theirs
-    // begins, so that a run waits for no more columns than it needs
+    // The arrays of the parts in one, and the last runs: the last kPanelRun
+    // dependencies, which may still be in progress when the panel meets
+    // them, are cut where a panel of theirs begins, so that a run waits for no
+    // more columns than it needs
     in_chunks(nparts, 4, [&](int32_t i0, int32_t i1, int) {
         for (int32_t i = i0; i < i1; i++) {
             Part &pt = parts[i];
-            std::copy(pt.prow.begin(), pt.prow.end(), W.prow.begin() + ou[i]);
-            std::copy(pt.pmask.begin(), pt.pmask.end(), W.pmask.begin() + ou[i]);
+            std::copy(rows.begin() + at[i], rows.begin() + at[i] + pt.rows, W.prow.begin() + ou[i]);
+            std::copy(masks.begin() + at[i], masks.begin() + at[i] + pt.rows, W.pmask.begin() + ou[i]);
             std::copy(pt.ppref.begin(), pt.ppref.end(), W.ppref.begin() + of[i]);
+            std::vector<PanelRun> runs;
+            runs.reserve(pt.prun.size() + pt.prun.size() / 4);
             for (size_t p = 0; p < pt.pan.size(); p++) {
                 PanelDesc &d = W.pan[op[i] + (int64_t)p];
                 d = pt.pan[p];
-                const int32_t *u = pt.prow.data() + d.uoff;
-                const uint8_t *m = pt.pmask.data() + d.uoff;
-                const int64_t r0 = (int64_t)pt.prun.size();
-                for (int32_t s = 0; s < d.nu;) {
+                const int32_t *u = rows.data() + at[i] + d.uoff;
+                const uint8_t *m = masks.data() + at[i] + d.uoff;
+                const PanelRun *r = pt.prun.data() + d.roff, *re = r + d.nruns;
+                const int64_t r0 = (int64_t)runs.size();
+                int32_t s = 0;
+                while (r < re && r->t + (r->wm & 0xff) <= d.nu - kPanelRun) runs.push_back(*r++);
+                if (r < re) s = r->t;
+                while (r < re && s < d.nu) {
                     int w = 1;
                     unsigned mk = m[s];
                     while (w < kPanelRun && s + w < d.nu && u[s + w] == u[s + w - 1] + 1 && W.chain[u[s + w - 1]] &&
@@ -730,27 +917,24 @@ static void build_panels(const Structure &S, int panel_ctas, bool allow_scratch,
                         mk |= m[s + w];
                         w++;
                     }
-                    const int32_t jl = u[s + w - 1];
-                    PanelRun r;
-                    r.t = s;
-                    r.wm = (int32_t)(w | (mk << 8));
-                    r.lbl = S.LUp[jl] + S.nU[jl];
-                    r.nR = (int32_t)(S.LUp[jl + 1] - r.lbl);
-                    r.j0 = u[s];
-                    pt.prun.push_back(r);
+                    runs.push_back(panel_run(S, s, u[s], w, mk));
                     s += w;
                 }
-                d.nruns = (int32_t)((int64_t)pt.prun.size() - r0);
+                auto before = [&](int32_t slot) {   // runs of the panel that begin before it
+                    return (int32_t)(std::lower_bound(runs.begin() + r0, runs.end(), slot,
+                                                      [](const PanelRun &x, int32_t t) { return x.t < t; }) -
+                                     (runs.begin() + r0));
+                };
+                d.nruns = (int32_t)((int64_t)runs.size() - r0);
                 d.nux = (int32_t)(std::lower_bound(u, u + d.nu, W.tb_p) - u);
-                d.runp = 0;
-                while (d.runp < d.nruns && pt.prun[r0 + d.runp].t < d.pull) d.runp++;
-                d.nrunsx = 0;
-                while (d.nrunsx < d.nruns && pt.prun[r0 + d.nrunsx].t < d.nux) d.nrunsx++;
+                d.runp = before(d.pull);
+                d.nrunsx = before(d.nux);
                 d.roff = r0;
                 d.uoff += ou[i];
                 d.poff += of[i];
                 W.pan_id[d.k0] = (int32_t)(op[i] + (int64_t)p);
             }
+            pt.prun.swap(runs);
         }
     });
     for (int32_t i = 0; i < nparts; i++) orr[i + 1] = orr[i] + (int64_t)parts[i].prun.size();
@@ -767,6 +951,7 @@ void build_schedule(const Pattern &P, const Structure &S, double alpha,
                     int resident_warps, const int (&panel_ctas)[2], int sched_mode, int cap_short, const SolveSplit &split,
                     int dense_min_rows, Schedule &W, bool defer_solve)
 {
+    HostTeamScope team;
     const int32_t n = S.n;
     W.rowwise_ready = false;
     W.solve_ready = false;
@@ -814,6 +999,8 @@ void build_schedule(const Pattern &P, const Structure &S, double alpha,
             W.chain[j] = std::equal(S.LUi.begin() + a + 1, S.LUi.begin() + ae, S.LUi.begin() + b) ? 1 : 0;
         }
     });
+    std::vector<int32_t> chain_end(n);   // last column of the chain of linked columns that j is in
+    for (int32_t j = n - 1; j >= 0; j--) chain_end[j] = W.chain[j] ? chain_end[j + 1] : j;
     // ---- wide columns: at most kPullMaxL L entries and at least kPullMinRuns
     // supernode runs among the dependencies.  All but the last chain of linked
     // dependencies are taken row by row (pull_start = where that chain
@@ -894,11 +1081,13 @@ void build_schedule(const Pattern &P, const Structure &S, double alpha,
             const int64_t b = S.LUp[k], e = b + S.nU[k] - 1;
             const int32_t lim = k < W.tb_p ? n : W.tb_p;
             double f = 0, o = 0;
-            for (int64_t i = b; i < e; i++) {
-                const int32_t j = S.LUi[i];
-                const double v = 2.0 * (double)(S.LUp[j + 1] - S.LUp[j] - S.nU[j]);
-                f += v;
-                if (j < lim) o += v;
+            for (int64_t i = b; i < e;) {   // L(:, j) loses a row per column of a chain
+                const int32_t j = S.LUi[i], len = chain_part(S.LUi.data() + i, (int32_t)(e - i), chain_end);
+                const int64_t nl = S.LUp[j + 1] - S.LUp[j] - S.nU[j];
+                const int32_t in = std::min(len, std::max(lim - j, 0));
+                f += (double)(len * (2 * nl - len + 1));
+                o += (double)(in * (2 * nl - in + 1));
+                i += len;
             }
             fl += f;
             outside += o;
@@ -930,7 +1119,7 @@ void build_schedule(const Pattern &P, const Structure &S, double alpha,
     W.smem = three ? kRefSmemThree : kRefSmemTwo;
     // panels of wide columns hold kPullLd values per row of their scratch
     W.pull_ld = 1;
-    build_panels(S, long_cols ? 0 : panel_ctas[three ? 1 : 0], !three, W);   // (none for 0 CTAs)
+    build_panels(S, chain_end, long_cols ? 0 : panel_ctas[three ? 1 : 0], !three, W);   // (none for 0 CTAs)
     W.tb_nux.resize(W.tb_m);
     for (int32_t c = 0; c < W.tb_m; c++) {
         const int32_t *r = S.LUi.data() + S.LUp[W.tb_p + c];
@@ -1045,10 +1234,18 @@ void build_schedule(const Pattern &P, const Structure &S, double alpha,
             const PanelDesc *d = in_pan[k] >= 0 ? &W.pan[in_pan[k]] : nullptr;
             for (int32_t p = P.Ap[c]; p < P.Ap[c + 1]; p++) {
                 const int32_t s = S.pinv[P.Ai[p]];
+                int32_t at = -1;
+                if (d && !all_short && s < d->k0 + d->nc) {   // the slot in the panel, if the column has the row
+                    const int32_t *u = W.prow.data() + d->uoff;
+                    const int64_t q = s < d->k0 ? std::lower_bound(u, u + d->nu, s) - u : d->nu + (s - d->k0);
+                    if (u[q] == s && ((W.pmask[d->uoff + q] >> (k - d->k0)) & 1)) at = (int32_t)q;
+                    W.amap[p] = at;
+                    continue;
+                }
                 const int32_t *it = std::lower_bound(col, col + len, s);
-                int32_t at = (it != col + len && *it == s) ? (int32_t)(it - col) : -1;
+                at = (it != col + len && *it == s) ? (int32_t)(it - col) : -1;
                 if (all_short) W.camap[p] = at;
-                if (d && at >= 0) {   // the slot in the panel
+                if (d && at >= 0) {
                     const int32_t *u = W.prow.data() + d->uoff;
                     if (s < d->k0) at = (int32_t)(std::lower_bound(u, u + d->nu, s) - u);
                     else if (s < d->k0 + d->nc) at = d->nu + (s - d->k0);
