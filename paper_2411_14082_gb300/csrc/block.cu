@@ -14,7 +14,9 @@
 // chain of the factorization is one launch per 16 columns instead of a
 // hand-off between CTAs per panel; the update is spread over the whole
 // device.  Every value gets the same multiply-adds in the same (ascending)
-// order as in the column kernels: the factors are the same bits.
+// order as in the column kernels: finite factors are the same bits (the
+// zeros outside the pattern make NaN of infinite values, which fails the
+// column's check; the restart then judges it without them).
 // The last launch checks every pivot against its column's largest candidate,
 // stores the entries of the columns that pass in the factor's columns and
 // publishes them.  The columns before the first failing one were computed

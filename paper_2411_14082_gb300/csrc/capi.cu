@@ -716,8 +716,9 @@ int issue_refactor(gblu_ctx *h, const double *Ax, cudaStream_t st, int ep, bool 
     return GBLU_OK;
 }
 
-// the trailing block is factored densely unless the checks have to be made
-// column by column (a forced failure, a re-prediction's strict columns)
+// the single-matrix double-precision re-factorization factors the trailing
+// block densely unless the checks have to be made column by column (a forced
+// failure, a re-prediction's strict columns)
 static bool block_applies(const gblu_ctx *h) { return h->W.tb_m > 0 && h->force_col < 0 && !h->strict_on; }
 
 int restart_on_structure(gblu_ctx *h, const double *Ax, cudaStream_t st, bool no_stop, int *interrupted);

@@ -68,7 +68,6 @@ struct Structure {
     int64_t nnz() const { return LUp.empty() ? 0 : LUp.back(); }
 };
 
-// Everything derived from a Structure that the kernels use.
 // Panels of the re-factorization: up to kPanelMax consecutive columns
 // k0 .. k0+nc-1 of one supernode of L, computed together by one CTA on the
 // union of their patterns (slots): nu rows above k0, ascending, then the nc
@@ -91,13 +90,17 @@ struct alignas(8) PanelRun {
 constexpr int kPanelRun = 16;
 constexpr int kPanelWideRows = 256;   // most L rows below a panel of more than four columns
 constexpr int kPanelMax = 8;
-// columns of more entries count as long (Schedule::smem)
+// columns of more entries count as long (build_schedule, where the share of
+// the operations in them from which there are no panels was measured with
+// this value; four such columns are beyond the 2,261 slots of a panel in
+// shared memory whatever they share)
 constexpr int32_t kLongColumn = 3200;
 // sets * sqrt(n) from which a batch takes short columns one per warp
 constexpr double kColumnBatch = 1800.0;
 // row stride of a panel's work vector
 constexpr int panel_ld(int nc) { return nc <= 4 ? 4 : 8; }
 
+// Everything derived from a Structure that the kernels use.
 struct Schedule {
     // refactor: EGraph levels (Section II-B) and dual-mode split
     std::vector<int32_t> level_ptr;   // n_levels+1
@@ -119,9 +122,11 @@ struct Schedule {
     BigVec<PanelRun> prun;
     int64_t pscratch = 0;
     int32_t smem = 0;                 // dynamic shared memory of the CTAs
-    // trailing block factored densely (block.cu): columns [tb_p, n), tb_m of
-    // them (0: none); every one is in a panel; tb_nux[c] = entries of column
-    // tb_p + c in rows before the block
+    // trailing block factored densely (block.cu) by the single-matrix
+    // double-precision re-factorization (batches and single precision take
+    // its columns like the others): columns [tb_p, n), tb_m of them (0: none),
+    // in panels or alone; tb_nux[c] = entries of column tb_p + c in rows
+    // before the block
     int32_t tb_p = 0, tb_m = 0;
     std::vector<int32_t> tb_nux;
     std::vector<int32_t> amap;        // A slot -> position inside its column (in a panel: its slot)

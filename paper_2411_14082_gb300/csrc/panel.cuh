@@ -21,9 +21,11 @@
 // together.
 //
 // Each value gets the same fused multiply-adds in the same order as when
-// its column is computed alone, so the factors are the same bits.  A column
+// its column is computed alone, so finite factors are the same bits.  A column
 // without an entry that its neighbours have holds a zero there, and
-// subtracts zero times a value.
+// subtracts zero times a value: an infinite L (a subnormal pivot, or one that
+// passed with a tolerance below the reciprocal of the largest double) makes
+// NaN there, also in columns that do not depend on it.
 #pragma once
 
 namespace gblu {
@@ -174,7 +176,7 @@ __device__ __forceinline__ unsigned long long warp_max_key(unsigned long long k)
 // values of rows i of the stage at val[off[d] + i] (row pitch sp)
 struct StageHead {
     int t, w, mask, i0, i1;   // run; rectangle rows [i0, i1) of the stage (those before i0: the triangle's)
-    int first, last, sp;      // first stage of its run, last stage of the panel
+    int first, last, pad;     // first stage of its run, last stage of the panel
     int off[kPanelRun];
 };
 static_assert(sizeof(StageHead) == 96, "StageHead");
@@ -484,7 +486,6 @@ __device__ __forceinline__ bool panel_produce(const RefactorArgsT<R> &a, const P
             h.i1 = n;
             h.first = e0 == 0;
             h.last = rw.base + q == nruns - 1 && e0 + S >= nE;
-            h.sp = sp;
         }
         __syncwarp();
         if (lane == 0)

@@ -127,3 +127,39 @@ def test_columns_that_are_barely_wide_leave_the_block(wide, taken):
     b = dev(np.random.default_rng(4).uniform(-1.0, 1.0, n))
     LU, failed = s.refactorize_batch(dev(v[None]))
     assert not failed.any() and torch.equal(s.solve_batch(LU, b[None])[0], s.solve(b))
+
+
+def test_wide_panels_whose_columns_lack_some_rows_of_their_neighbours():
+    """Wide columns that touch different nine tenths of the blocks: panels of
+    them hold zeros where a column has no entry."""
+    n, Ap, Ai, Ax0, Q = bordered_blocks(200, 40, blocks=400)
+    rng = np.random.default_rng(12)
+    cols = np.repeat(np.arange(n), np.diff(Ap))
+    keep = np.ones(len(Ai), bool)
+    for c in range(n - 40, n):   # drop a block's two entries and the two across the diagonal
+        for j in rng.choice(400, 40, replace=False):
+            keep &= ~(((cols == c) & (Ai // 2 == j)) | ((Ai == c) & (cols // 2 == j)))
+    Ap = np.r_[0, np.cumsum(np.bincount(cols[keep], minlength=n))].astype(np.int32)
+    sys_ = n, Ap, Ai[keep], Ax0[keep], Q
+    s = solver(sys_)
+    assert s.stats()["wide_cols"] == 40
+    v = sys_[3] * np.random.default_rng(2).uniform(0.98, 1.02, len(sys_[3]))
+    _, rep = s.refactorize(dev(v))
+    lu = O.refactorize(O.factorize(*sys_[:4], Q, 1e-3), Ap, sys_[2], v)
+    assert not rep and lu.n_rejected == 0
+    compare_factors(s.export_factors(), lu, 1e-10)
+    b = dev(np.random.default_rng(4).uniform(-1.0, 1.0, n))
+    LU, failed = s.refactorize_batch(dev(np.tile(v, (5, 1))))
+    x = s.solve_batch(LU, b.expand(5, n).contiguous())
+    assert not failed.any() and bool((x == s.solve(b)).all())
+
+
+@pytest.mark.parametrize("n,half,tail", [(2, 1, 0), (9, 8, 0), (33, 32, 0), (129, 128, 0), (200, 20, 3)])
+def test_batches_large_enough_for_the_column_list_equal_the_panels(n, half, tail):
+    """A batch takes short columns one per warp from 1,800 / sqrt(n) sets."""
+    sys_ = band(n, half, tail, 7)
+    s = solver(sys_)
+    v = dev(sys_[3] * np.random.default_rng(2).uniform(0.98, 1.02, len(sys_[3])))
+    one, _ = s.refactorize_batch(v[None])
+    many, failed = s.refactorize_batch(v.expand(int(1800 / n ** 0.5) + 2, len(v)).contiguous())
+    assert not failed.any() and bool((many == one[0]).all())
