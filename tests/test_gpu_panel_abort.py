@@ -101,3 +101,40 @@ def test_single_precision_after_a_given_up_panel(k):
         assert s.refactorize_f32(dev(w))
         assert not s.refactorize_f32(dev(v))
         assert torch.equal(s.solve_refined(dev(v), b, max_iter=0, tol=1.0)[0], want)
+
+
+@pytest.mark.parametrize("name", ["band", "mesh", "rails"])
+def test_failing_handles_of_one_launch_leave_the_others_alone(name):
+    """The same in a launch over several handles: those whose check fails
+    restart alone, the others give what they give alone."""
+    n, Ap, Ai, Ax0, Q = system(name)
+    lu0 = O.factorize(n, Ap, Ai, Ax0, Q, 1e-3)
+    rng = np.random.default_rng(9)
+    vals = [Ax0 * rng.uniform(0.98, 1.02, len(Ax0)) for _ in range(6)]
+    bad = {1: n // 3, 4: 2 * n // 3}
+    for i, k in bad.items():
+        vals[i] = with_failing_pivot(n, Ap, Ai, vals[i], Q, lu0, k)
+    b = dev(rng.uniform(-1.0, 1.0, n))
+    Ax = [dev(v) for v in vals]
+    solvers = []
+    for _ in vals:
+        s = gblu.Solver(DEV)
+        s.analyze(n, Ap, Ai, Q)
+        s.factorize(dev(Ax0))
+        solvers.append(s)
+    want = {}
+    for i, s in enumerate(solvers):
+        if i not in bad:
+            assert not s.refactorize(Ax[i])[1]
+            want[i] = s.solve(b).clone()
+    for _ in range(10):
+        for i in bad:
+            solvers[i].factorize(dev(Ax0))
+        rep = gblu.refactorize_multi(solvers, Ax)
+        assert [i for i, r in enumerate(rep) if r] == sorted(bad)
+        for i, s in enumerate(solvers):
+            x = s.solve(b)
+            if i in bad:
+                assert O.residual(n, Ap, Ai, vals[i], x.cpu().numpy(), b.cpu().numpy()) <= 1e-12
+            else:
+                assert torch.equal(x, want[i])
