@@ -88,8 +88,8 @@ def hbm_roofline(bytes_alg, seconds, traffic=None):
 # (dram__bytes_read.sum + dram__bytes_write.sum over its launches); valid only
 # for the kernel source it was taken on
 REFACTOR_TRAFFIC = {
-    "rc_mesh_200x200x4/library": {"refactor_cu_sha256": "e68bae915649a44f1500d1c55a4d0193e90295ea8f5eb6f02019de0ad691508c",
-                                  "bytes": 19.104e9 + 964.9e6},
+    "rc_mesh_200x200x4/library": {"refactor_cu_sha256": "c8d82ffb37ee8890a210dfe8c7220584fc32129754001b6ade6d2268a06b8d90",
+                                  "bytes": 12.802e9 + 981.3e6},
 }
 
 

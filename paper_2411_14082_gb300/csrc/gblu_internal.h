@@ -194,7 +194,11 @@ constexpr int kPullMinRuns = 256;
 constexpr size_t kPullScratchBytes = (size_t)1 << 30;
 constexpr int kPullLd = 4;            // wide columns of a panel
 // trailing block: at least kBlockMin columns, at most kBlockMax (302 MB of
-// values), at least kBlockDensity of its entries in the factor
+// values), at least kBlockDensity of its entries in the factor (the zeros
+// among them cost operations, a larger block takes more off the column
+// kernels' chain: meshes of 48,000, 90,000 and 160,000 unknowns with 85%
+// 12.5, 30.3, 73.1 ms, with 92% 12.0, 29.2, 68.9, with 96% 12.0, 28.7, 66.9,
+// with 98.5% 11.9, 28.5, 66.2)
 constexpr int kBlockCols = 16, kBlockMin = 128, kBlockMax = 6144;
 constexpr double kBlockDensity = 0.96;
 constexpr size_t kPanelScratchBytes = (size_t)1 << 30;
