@@ -532,7 +532,8 @@ constexpr int kRefSmemTwo = 100 * 1024, kRefSmemThree = 65 * 1024;
 // about half the room holds their work vectors and ring, three CTAs fit on an
 // SM in both, and the rest stays L1 (re-factorization of the 57,600-unknown
 // mesh with 100 KB and with 56 KB: 10.5 and 9.1 ms; of the 160,000-unknown
-// mesh with 65 KB and with 40 KB: 40.9 and 40.6 ms)
+// mesh with 65 KB and with 40 KB: 40.9 and 40.6 ms with panels, 39.2 without,
+// as it runs now)
 constexpr int kRefSmemTwo32 = 56 * 1024, kRefSmemThree32 = kRefCapLong * (int)(sizeof(float) + sizeof(int32_t));
 // of a launch without panels: the column kernels' work vectors alone
 constexpr int kRefSmemColumns = kRefCapLong * (int)(sizeof(double) + sizeof(int32_t));
