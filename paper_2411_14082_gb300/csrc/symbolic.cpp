@@ -201,8 +201,9 @@ struct HostTeam {
         for (std::thread &x : th) x.join();
     }
 
-    // fn(t) for t = 0 .. nt-1, t = 0 by the calling thread
-    void run(const std::function<void(int)> &fn)
+    // fn(t) for t = 0 .. nt-1, t = 0 by the calling thread (an exception ends
+    // the process, as it does on the other threads, which still run fn)
+    void run(const std::function<void(int)> &fn) noexcept
     {
         {
             std::lock_guard<std::mutex> lk(mu);
