@@ -120,7 +120,7 @@ struct gblu_ctx {
     // panels of the re-factorization and the scratch of those beyond shared memory
     DBuf<PanelDesc> pan;
     DBuf<int32_t> pan_id, prow, ppref;
-    DBuf<int32_t> ctask_ptr, ctask_cols, camap;   // tasks without panels (Schedule::ctask_ptr)
+    DBuf<int32_t> ctask_ptr, ctask_cols, camap, cpan_id;   // a batch's second task list (Schedule::ctask_ptr)
     DBuf<uint8_t> pmask;
     DBuf<PanelRun> prun;
     DBuf<unsigned char> pscratch;
@@ -396,6 +396,7 @@ static void make_lean(gblu_ctx *h, cudaStream_t st)
     release(h, h->ctask_ptr);
     release(h, h->ctask_cols);
     release(h, h->camap);
+    release(h, h->cpan_id);
 }
 
 // Frees the factors' buffers if they hold room for a pool behind the nnz
@@ -469,6 +470,7 @@ static int try_install(gblu_ctx *h, Structure &&S, const std::vector<double> *va
         CK(upload(h, h->ctask_ptr, h->W.ctask_ptr, st));
         CK(upload(h, h->ctask_cols, h->W.ctask_cols, st));
         CK(upload(h, h->camap, h->W.camap, st));
+        if (!h->W.cpan_id.empty()) CK(upload(h, h->cpan_id, h->W.cpan_id, st));
     }
     CK(upload(h, h->pan_id, h->W.pan_id, st));
     h->pscratch_ctas = h->W.pscratch > 0 ? panel_ctas[cfg(h)] : 0;
@@ -1361,7 +1363,7 @@ void gblu_destroy(gblu_handle h)
         release(h, h->piv); release(h, h->pinv); release(h, h->vals);
         release(h, h->pan); release(h, h->pan_id); release(h, h->prow); release(h, h->ppref); release(h, h->pmask);
         release(h, h->prun); release(h, h->pscratch); release(h, h->tb_S); release(h, h->tb_nux); release(h, h->tb_words);
-        release(h, h->ctask_ptr); release(h, h->ctask_cols); release(h, h->camap);
+        release(h, h->ctask_ptr); release(h, h->ctask_cols); release(h, h->camap); release(h, h->cpan_id);
         release(h, h->Lrp); release(h, h->Urp); release(h, h->Lcol); release(h, h->Lslot);
         release(h, h->Ucol); release(h, h->Uslot); release(h, h->Udiag);
         release(h, h->lsv_rows); release(h, h->usv_rows); release(h, h->lbs); release(h, h->ubs);
@@ -1809,8 +1811,19 @@ static int batch_group(gblu_ctx *h, int32_t nsets)
 // the two took equal time on grids: 528 unknowns at 80 sets, 1,147 at 55
 // (96 sets: 1.04 ms against 1.45 ms; 8 sets: 0.69 ms against 0.36 ms), 3,300
 // at 30, 7,200 at 20.
+// A small batch of a structure with wide columns takes those alone instead
+// of four to a panel while each has about a CTA of its own: a panel's prefix
+// solve takes longer than a column's, and saves nothing where CTAs are idle.
+// Grids of 60x60 to 119x119 with 8, 20 and 40 rails, refactor and solve: up
+// to one wave (456 CTAs) alone is 1.10 to 1.42 times as fast (100x100, 40
+// rails, 8 sets: 6.95 ms in panels, 4.88 alone, 5.89 without any panels), at
+// 480 to 512 columns 0.97 to 1.08 times (119x119, 20 rails, 24 sets: 14.7 and
+// 13.8 ms), at 640 0.95 to 1.08 times, at 960 0.82 to 0.85 times.
 static bool columns_batch(const gblu_ctx *h, int32_t nsets)
 {
+    if (h->W.pull_cols > 0)
+        return !h->W.ctask_ptr.empty() && h->pull_slots > 0 &&
+               4 * nsets * h->W.pull_cols <= 5 * (int64_t)pgrid(h, h->batch_blocks_per_sm[cfg(h)]);
     return !h->W.ctask_ptr.empty() && (double)nsets * std::sqrt((double)h->S.n) > kColumnBatch;
 }
 
@@ -1823,9 +1836,13 @@ static RefactorArgs batch_args(gblu_ctx *h, bool columns)
         a.task_ptr = h->ctask_ptr.p;
         a.task_cols = h->ctask_cols.p;
         a.amap = h->camap.p;
-        a.panels = 0;
-        a.smem_bytes = kRefSmemColumns;
-        a.pscratch_ctas = 0;
+        if (h->W.pull_cols > 0) {   // panels but for the wide columns
+            a.pan_id = h->cpan_id.p;
+        } else {
+            a.panels = 0;
+            a.smem_bytes = kRefSmemColumns;
+            a.pscratch_ctas = 0;
+        }
     }
     return a;
 }
@@ -1849,7 +1866,7 @@ static int issue_batch(gblu_ctx *h, int32_t nsets, const RefactorArgs *args_dev,
         a0.task_begin = ltp[div];
         a0.ntasks = ntask - ltp[div];
         KL(launch_refactor_batch(args_dev, a0, nsets, true,
-                                 pgrid(h, h->batch_blocks_per_sm[columns ? 2 : cfg(h)]), epoch,
+                                 pgrid(h, h->batch_blocks_per_sm[columns && h->W.pull_cols == 0 ? 2 : cfg(h)]), epoch,
                                  h->bticket.p, st, batch_group(h, nsets)));
     }
     return GBLU_OK;
@@ -2360,6 +2377,7 @@ int gblu_handle_spare(gblu_handle h, int64_t *pool, int64_t *panels)
     auto add = [&](const auto &b) { *panels += (int64_t)(b.cap * sizeof(*b.p)); };
     add(h->pscratch); add(h->tb_S); add(h->tb_words); add(h->tb_nux); add(h->pan); add(h->prow); add(h->pmask);
     add(h->ppref); add(h->prun); add(h->ctask_ptr); add(h->ctask_cols); add(h->camap);
+    add(h->cpan_id);
     if (h->W.pull_ld > 0) *panels += (int64_t)(h->pull_x.cap / h->W.pull_ld * (h->W.pull_ld - 1) * sizeof(double));
     return GBLU_OK;
 }

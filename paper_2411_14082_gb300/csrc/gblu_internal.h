@@ -130,9 +130,12 @@ struct Schedule {
     int32_t tb_p = 0, tb_m = 0;
     std::vector<int32_t> tb_nux;
     std::vector<int32_t> amap;        // A slot -> position inside its column (in a panel: its slot)
-    // the same tasks without panels, for large batches of a structure whose
-    // columns are all short (empty otherwise): one warp per column
-    std::vector<int32_t> ctask_ptr, ctask_cols, clevel_task_ptr, camap;
+    // a second task list for batches (empty where there is none): without
+    // panels, one warp per column, for large batches of a structure whose
+    // columns are all short; or with the wide columns that are longer than a
+    // warp takes alone instead of in panels, for small batches of a structure
+    // with panels of them (cpan_id: pan_id for that list)
+    std::vector<int32_t> ctask_ptr, ctask_cols, clevel_task_ptr, camap, cpan_id;
     BigVec<int32_t> LUi_orig;         // L entries: original row ids (U: step ids)
     // chain[j] = 1 iff L(:,j) = {j+1} followed by the rows of L(:,j+1), i.e.
     // j and j+1 are consecutive columns of one supernode of L

@@ -1138,6 +1138,18 @@ void build_schedule(const Pattern &P, const Structure &S, double alpha,
     W.thr = thr;
     bool all_short = !W.pan.empty() && W.dense_m == 0 && W.pull_cols == 0;
     for (int32_t k = 0; k < n && all_short; k++) all_short = S.LUp[k + 1] - S.LUp[k] <= cap_short;
+    // panels of wide columns that the second list takes alone (a column of
+    // at most cap_short entries would go to one warp, which applies its
+    // dependencies by runs: other roundings)
+    W.cpan_id.clear();
+    for (const PanelDesc &d : W.pan) {
+        bool alone = d.pull > 0;
+        for (int32_t k = d.k0; k < d.k0 + d.nc && alone; k++) alone = S.LUp[k + 1] - S.LUp[k] > cap_short;
+        if (!alone) continue;
+        if (W.cpan_id.empty()) W.cpan_id = W.pan_id;
+        W.cpan_id[d.k0] = -1;
+    }
+    const bool second = all_short || !W.cpan_id.empty();   // a second task list
     // ---- EGraph levels, the dividing level (Section IV-B) and the tasks:
     // on a thread of their own, beside the slot maps and row-wise copies
     // below (they write disjoint members of W) ----
@@ -1167,8 +1179,8 @@ void build_schedule(const Pattern &P, const Structure &S, double alpha,
         // before the dividing level.  A panel is a task of its own at the place
         // of its last column: its columns' levels ascend, and a column that
         // depends on any of them depends on the last.
-        auto tasks = [&](bool panels, std::vector<int32_t> &task_ptr, std::vector<int32_t> &task_cols,
-                         std::vector<int32_t> &level_task_ptr) {
+        auto tasks = [&](const std::vector<int32_t> *pan_id, std::vector<int32_t> &task_ptr,
+                         std::vector<int32_t> &task_cols, std::vector<int32_t> &level_task_ptr) {
             task_ptr.assign(1, 0);
             task_cols.clear();
             task_cols.reserve(n);
@@ -1185,7 +1197,7 @@ void build_schedule(const Pattern &P, const Structure &S, double alpha,
                 for (int32_t p = W.level_ptr[l]; p < W.level_ptr[l + 1]; p++) {
                     const int32_t k = W.level_cols[p];
                     const int64_t len = S.LUp[k + 1] - S.LUp[k];
-                    if (panels && in_pan[k] >= 0) {
+                    if (pan_id && in_pan[k] >= 0 && (*pan_id)[W.pan[in_pan[k]].k0] >= 0) {
                         if (pan_end[k] < 0) continue;
                         close();
                         task_cols.push_back(W.pan[pan_end[k]].k0);
@@ -1217,35 +1229,38 @@ void build_schedule(const Pattern &P, const Structure &S, double alpha,
             }
             close();
         };
-        tasks(true, W.task_ptr, W.task_cols, W.level_task_ptr);
+        tasks(&W.pan_id, W.task_ptr, W.task_cols, W.level_task_ptr);
         W.ctask_ptr.clear();
         W.ctask_cols.clear();
         W.clevel_task_ptr.clear();
-        if (all_short) tasks(false, W.ctask_ptr, W.ctask_cols, W.clevel_task_ptr);
+        if (second) tasks(all_short ? nullptr : &W.cpan_id, W.ctask_ptr, W.ctask_cols, W.clevel_task_ptr);
     });
     // ---- A slot -> position in its column (columns are sorted) ----
     const int64_t nnzA = (int64_t)P.Ai.size();
     W.amap.assign(nnzA, -1);
-    W.camap.assign(all_short ? nnzA : 0, -1);
+    W.camap.assign(second ? nnzA : 0, -1);
     parallel_chunks(n, 2048, [&](int32_t c0, int32_t c1, int) {
         for (int32_t c = c0; c < c1; c++) {
             const int32_t k = P.qinv[c];
             const int32_t *col = S.LUi.data() + S.LUp[k];
             const int32_t len = (int32_t)(S.LUp[k + 1] - S.LUp[k]);
             const PanelDesc *d = in_pan[k] >= 0 ? &W.pan[in_pan[k]] : nullptr;
+            // the second list takes the column alone
+            const bool alone = all_short || (d && second && W.cpan_id[d->k0] < 0);
             for (int32_t p = P.Ap[c]; p < P.Ap[c + 1]; p++) {
                 const int32_t s = S.pinv[P.Ai[p]];
                 int32_t at = -1;
-                if (d && !all_short && s < d->k0 + d->nc) {   // the slot in the panel, if the column has the row
+                if (d && !alone && s < d->k0 + d->nc) {   // the slot in the panel, if the column has the row
                     const int32_t *u = W.prow.data() + d->uoff;
                     const int64_t q = s < d->k0 ? std::lower_bound(u, u + d->nu, s) - u : d->nu + (s - d->k0);
                     if (u[q] == s && ((W.pmask[d->uoff + q] >> (k - d->k0)) & 1)) at = (int32_t)q;
                     W.amap[p] = at;
+                    if (second) W.camap[p] = at;
                     continue;
                 }
                 const int32_t *it = std::lower_bound(col, col + len, s);
                 at = (it != col + len && *it == s) ? (int32_t)(it - col) : -1;
-                if (all_short) W.camap[p] = at;
+                if (alone) W.camap[p] = at;
                 if (d && at >= 0) {
                     const int32_t *u = W.prow.data() + d->uoff;
                     if (s < d->k0) at = (int32_t)(std::lower_bound(u, u + d->nu, s) - u);
@@ -1254,6 +1269,7 @@ void build_schedule(const Pattern &P, const Structure &S, double alpha,
                     else at = d->nu + d->nc + (at - S.nU[k] - (d->k0 + d->nc - 1 - k));
                 }
                 W.amap[p] = at;
+                if (second && !alone) W.camap[p] = at;
             }
         }
     });
